@@ -41,125 +41,224 @@ __device__ __forceinline__ double std_normal(uint32_t s, uint32_t index, uint32_
     return __dmul_rn(r, cos(__dmul_rn(two_pi, u2)));
 }
 
+// The recipe's last step in float64: half away from zero, clamped at 0 and at
+// the type's maximum.
+template <typename DT>
+__device__ __forceinline__ DT round_demand(double x)
+{
+    const double dmax = sizeof(DT) == 2 ? 32767.0 : 2147483647.0;
+    double rnd = floor(x);
+    if (__dsub_rn(x, rnd) >= 0.5) rnd = __dadd_rn(rnd, 1.0);
+    rnd = fmin(fmax(rnd, 0.0), dmax);
+    return (DT)(long long)rnd;
+}
+
+__device__ __forceinline__ double correlated_f64(double mu, double f, double e)
+{
+    const double y = __dadd_rn(__dmul_rn(0.6, f), __dmul_rn(0.8, e));
+    return __dmul_rn(mu, exp(__dsub_rn(__dmul_rn(0.3, y), 0.045)));
+}
+
 // One demand by the recipe in float64: what every entry is defined by.
 template <typename DT>
 __device__ __noinline__ DT demand_f64(const GenParams &g, uint32_t s, int row)
 {
     const uint32_t k0 = (uint32_t)g.seed, k1 = (uint32_t)(g.seed >> 32);
-    const double dmax = sizeof(DT) == 2 ? 32767.0 : 2147483647.0;
     const double mu = (double)g.mu[row];
-    double x;
-    if (g.kind == 1) {
-        const double f = std_normal(s, (uint32_t)(g.region[row] & 3), 1u, k0, k1);
-        const double e = std_normal(s, (uint32_t)row, 0u, k0, k1);
-        const double y = __dadd_rn(__dmul_rn(0.6, f), __dmul_rn(0.8, e));
-        x = __dmul_rn(mu, exp(__dsub_rn(__dmul_rn(0.3, y), 0.045)));
-    } else {
-        const double z = std_normal(s, (uint32_t)row, 2u, k0, k1);
-        x = __dadd_rn(mu, __dmul_rn(__dmul_rn(0.3, mu), z));
-    }
-    double rnd = floor(x);
-    if (__dsub_rn(x, rnd) >= 0.5) rnd = __dadd_rn(rnd, 1.0);   // half away from zero
-    rnd = fmin(fmax(rnd, 0.0), dmax);
-    return (DT)(long long)rnd;
+    if (g.kind == 1)
+        return round_demand<DT>(correlated_f64(mu, std_normal(s, (uint32_t)(g.region[row] & 3), 1u, k0, k1),
+                                               std_normal(s, (uint32_t)row, 0u, k0, k1)));
+    return round_demand<DT>(__dadd_rn(mu, __dmul_rn(__dmul_rn(0.3, mu), std_normal(s, (uint32_t)row, 2u, k0, k1))));
+}
+
+__device__ __forceinline__ float lg2_ftz(float x)
+{
+    float r;
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ float ex2_ftz(float x)
+{
+    float r;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ float rsqrt_ftz(float x)
+{
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ float cos_ftz(float x)
+{
+    float r;
+    asm("cos.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
 }
 
 // The same standard normal in float32, with a bound `err` on its distance
-// from the float64 value. From the documented errors of the intrinsics
-// (__logf 2^-21.41 absolute on [0.5, 2] and 3 ulp elsewhere, rsqrtf 2 ulp,
-// __cosf 2^-21.19 absolute on [-pi, pi]) and the roundings of u1 (2^-23) and
-// of the angle (3 * 2^-24 * pi):
+// from the float64 value. From the documented errors of the PTX instructions
+// (lg2 2^-22 absolute on (0.5, 2) and relative elsewhere, rsqrt 2^-22.9
+// relative, cos 2^-20.5 absolute on [-pi, pi]) and the roundings of u1
+// (2^-23 relative, 2 * 2^-23 of t), of the products (2^-24 each) and of the
+// angle (3 * 2^-24 * pi):
 //   t = -2 ln u1:  |dt| <= 1.0e-6 + 4.0e-7 t
 //   r = sqrt(t):   |dr| <= |dt| / r + 3.1e-7 r
-//   z = r cos:     |dz| <= |dr| + 1.05e-6 r  <=  1.0e-6 / r + 1.8e-6 r
-// A t below 1e-4 (5e-5 of all draws: u1 near 1, where the square root
-// amplifies dt) reports an infinite bound and z = 0.
-__device__ __forceinline__ float std_normal_f32(uint32_t wx, uint32_t wy, float &err)
+//   z = r cos:     |dz| <= |dr| + 1.3e-6 r  <=  1.0e-6 / r + 2.1e-6 r
+// below t = 1e-4 (5e-5 of all draws: u1 near 1, where the square root
+// amplifies dt) the bound does not hold and `ok` says so (NaN included).
+__device__ __forceinline__ float std_normal_f32(uint32_t wx, uint32_t wy, float &err, bool &ok)
 {
     const float u1 = ((float)wx + 0.5f) * 2.3283064365386963e-10f;
-    const float t = -2.0f * __logf(u1);
-    const float ri = rsqrtf(t), r = t * ri;
-    const float z = r * __cosf((float)(int32_t)wy * 1.4629180792671596e-9f);   // pi 2^-31
-    const bool ok = t > 1e-4f;
-    err = ok ? fmaf(1.0e-6f, ri, 1.8e-6f * r) : __int_as_float(0x7f800000);
-    return ok ? z : 0.0f;
+    const float t = -1.3862943611198906f * lg2_ftz(u1);                        // -2 ln 2
+    const float ri = rsqrt_ftz(t), r = t * ri;
+    ok = t > 1e-4f;
+    err = fmaf(1.0e-6f, ri, 2.1e-6f * r);
+    return r * cos_ftz((float)(int32_t)wy * 1.4629180792671596e-9f);           // pi 2^-31
 }
+
+// The parts of Philox4x32-10 at counter (s, row, domain, 0) that depend on
+// (s, domain) alone: the first two rounds and half of the third. A thread
+// walks the rows of one scenario, so they are formed once.
+struct PhiloxColumn {
+    uint32_t k0, k1, a, b, c, d, hi, lo;
+    __device__ __forceinline__ PhiloxColumn(uint32_t s, uint32_t domain, uint32_t key0, uint32_t key1)
+        : k0(key0), k1(key1)
+    {
+        a = __umulhi(kPhiloxM1, domain) ^ k0;                                  // ^ row: round 0's x
+        const uint32_t z0 = __umulhi(kPhiloxM0, s) ^ k1;
+        c = kPhiloxM0 * s ^ (k1 + kPhiloxW1);                                  // ^ hi(M0 x): round 1's z
+        b = kPhiloxM1 * z0;                                                    // round 1's y
+        const uint32_t x1 = __umulhi(kPhiloxM1, z0) ^ (kPhiloxM1 * domain) ^ (k0 + kPhiloxW0);
+        hi = __umulhi(kPhiloxM0, x1) ^ (k1 + 2u * kPhiloxW1);                  // ^ w: round 2's z
+        lo = kPhiloxM0 * x1;                                                   // round 2's w
+        d = b ^ (k0 + 2u * kPhiloxW0);                                         // ^ hi(M1 z): round 2's x
+    }
+    __device__ __forceinline__ uint2 at(uint32_t row) const
+    {
+        const uint32_t x0 = a ^ row;                                           // the same for all threads
+        const uint32_t z1 = __umulhi(kPhiloxM0, x0) ^ c;
+        uint32_t x = __umulhi(kPhiloxM1, z1) ^ d, y = kPhiloxM1 * z1, z = (kPhiloxM0 * x0) ^ hi, w = lo;
+#pragma unroll
+        for (int r = 3; r < 10; ++r) {
+            const uint32_t lo0 = kPhiloxM0 * x, hi0 = __umulhi(kPhiloxM0, x);
+            const uint32_t lo1 = kPhiloxM1 * z, hi1 = __umulhi(kPhiloxM1, z);
+            x = hi1 ^ y ^ (k0 + (uint32_t)r * kPhiloxW0);
+            y = lo1;
+            z = hi0 ^ w ^ (k1 + (uint32_t)r * kPhiloxW1);
+            w = lo0;
+        }
+        return make_uint2(x, y);
+    }
+};
 
 // What bounds it: the float64 pipe when every entry goes through it (GB300
 // issues one float64 warp instruction every 16 clocks per SM: 3784 us for
 // n = 200, S = 100,000, 10.6 GB/s of output). So each entry is evaluated in
-// float32 with a rigorous error bound first; when every value inside the
-// bound rounds to the same integer that integer is the float64 result. The
-// others (about 1e-4 of the entries at means of 5 to 30; all of them above
-// about 1e5, where float32 cannot decide) go through the float64 recipe:
-// collected in shared memory and evaluated densely after the block's rows, or
-// on the spot when the list is full. What bounds it now: the ten Philox
-// rounds and four special-function operations per entry.
+// float32 with a rigorous error bound first; when both ends of the bound
+// round to the same integer that integer is the float64 result. The others
+// (about 2e-4 of the entries at means of 5 to 30; all of them above about
+// 1e5, where float32 cannot decide) go through the float64 recipe: collected
+// in shared memory and evaluated densely after the block's rows, or on the
+// spot when the list is full. What bounds it now: issue of the Philox rounds
+// (14 wide multiplies) and the four special functions of an entry, 153 clocks
+// of a scheduler per 32 entries. 110 us at n = 200, S = 100,000 (1.01 ms at
+// n = 1000, S = 2^18); 132 us before the draws' common Philox rounds, the
+// bare special-function instructions and the paired float64 tail. Four blocks
+// a SM (64 registers): 123 us at one block, 119 us at six.
 constexpr int kGenThreads = 256;
 constexpr int kGenList = 512;
+constexpr int kGenRows = 64;                     // most rows of a block
 constexpr float kGenMax = 1.0e6f;                // float32 decides nothing above
 constexpr float kGenMagic = 12582912.0f;         // 1.5 * 2^23: adding it rounds to an integer
 
 template <typename DT, int KIND>
-__global__ void __launch_bounds__(kGenThreads) gen_demand_kernel(GenParams g, int rows_per_block)
+__global__ void __launch_bounds__(kGenThreads, 4) gen_demand_kernel(GenParams g, int rows_per_block)
 {
     __shared__ uint32_t s_list[kGenList];
     __shared__ int s_count;
+    __shared__ float s_f[4][kGenThreads];        // 0.6 F of the block's columns
+    __shared__ float2 s_row[kGenRows];           // mean, and the region's offset in s_f
     const long long s_block = (long long)blockIdx.x * kGenThreads;
-    const long long s = s_block + threadIdx.x;
+    const int tid = threadIdx.x;
+    const long long s = s_block + tid;
     const uint32_t k0 = (uint32_t)g.seed, k1 = (uint32_t)(g.seed >> 32);
     const int r0 = blockIdx.y * rows_per_block;
-    const int r1 = min(g.n, r0 + rows_per_block);
-    const float dmax = sizeof(DT) == 2 ? 32767.0f : 2147483648.0f;
-    if (threadIdx.x == 0) s_count = 0;
+    const int rows = min(g.n - r0, rows_per_block);
+    if (tid == 0) s_count = 0;
+    for (int k = tid; k < rows; k += kGenThreads)
+        s_row[k] = make_float2((float)g.mu[r0 + k], __int_as_float(KIND == 1 ? (g.region[r0 + k] & 3) * kGenThreads : 0));
     __syncthreads();
-    DT *out = reinterpret_cast<DT *>(g.out);
+    DT *out = reinterpret_cast<DT *>(g.out) + (long long)r0 * g.ld + s;
     if (s < g.S) {
-        float f[4] = {0.0f, 0.0f, 0.0f, 0.0f}, ef = 0.0f;
+        float ef = 0.0f;
         if (KIND == 1) {
+            bool fine = true;
 #pragma unroll
             for (int r = 0; r < 4; ++r) {
                 const uint4 w = philox4x32_10(make_uint4((uint32_t)s, (uint32_t)r, 1u, 0u), k0, k1);
                 float e;
-                f[r] = 0.6f * std_normal_f32(w.x, w.y, e);
+                bool ok;
+                const float f = std_normal_f32(w.x, w.y, e, ok);
+                s_f[r][tid] = ok ? 0.6f * f : 0.0f;
+                fine &= ok;
                 ef = fmaxf(ef, 0.18f * e);
             }
-            ef += 2.0e-6f;   // roundings of the exponent (|0.3 y| <= 2.9) and the products, __expf (5 ulp)
+            // + roundings of the exponent (|0.3 y| <= 2.9) and of the products, ex2 (2^-22)
+            ef = fine ? ef + 2.0e-6f : __int_as_float(0x7f800000);
         }
+        const PhiloxColumn px((uint32_t)s, KIND == 1 ? 0u : 2u, k0, k1);
 #pragma unroll 2
-        for (int row = r0; row < r1; ++row) {
-            const float mu = (float)g.mu[row];
-            const uint4 w = philox4x32_10(make_uint4((uint32_t)s, (uint32_t)row, KIND == 1 ? 0u : 2u, 0u), k0, k1);
+        for (int k = 0; k < rows; ++k, out += g.ld) {
+            const float2 rw = s_row[k];
+            const float mu = rw.x;
+            const uint2 w = px.at((uint32_t)(r0 + k));
             float e, x, err;
-            const float z = std_normal_f32(w.x, w.y, e);
+            bool ok;
+            const float z = std_normal_f32(w.x, w.y, e, ok);
+            float lo, hi;
             if (KIND == 1) {
-                const int reg = g.region[row] & 3;
-                const float fr = reg == 0 ? f[0] : reg == 1 ? f[1] : reg == 2 ? f[2] : f[3];
-                x = mu * __expf(fmaf(0.3f, fmaf(0.8f, z, fr), -0.045f));
+                const float y = fmaf(0.8f, z, (&s_f[0][0])[__float_as_int(rw.y) + tid]);
+                x = mu * ex2_ftz(fmaf(0.3f * 1.4426950408889634f, y, -0.045f * 1.4426950408889634f));
                 err = x * fmaf(0.24f, e, ef);
+                lo = x - err;
+                hi = x + err;
             } else {
                 x = fmaf(0.3f * mu, z, mu);
                 err = mu * fmaf(0.3f, e, 1.0e-6f + 3.0e-7f * fabsf(z));
+                lo = fmaxf(x - err, 0.0f);
+                hi = fmaxf(x + err, 0.0f);
             }
-            // nearest integers of both ends (an end on a tie is within the
-            // bound of it, so the other end rounds elsewhere or the list is
-            // only entered needlessly), clamped as the result is
-            const float lo = (fmaxf(x - err, 0.0f) + kGenMagic), hi = (fmaxf(x + err, 0.0f) + kGenMagic);
-            if (x < kGenMax && err < 1.0f && lo == hi) {
-                out[(long long)row * g.ld + s] = (DT)(int)fminf(lo - kGenMagic, dmax);
+            // nearest integers of both ends (an infinite or NaN bound makes them differ)
+            lo += kGenMagic;
+            hi += kGenMagic;
+            if (ok && x < kGenMax && lo == hi) {
+                const int v = __float_as_int(lo) - __float_as_int(kGenMagic);
+                *out = (DT)(sizeof(DT) == 2 ? min(v, 32767) : v);
             } else {
                 const int at = atomicAdd(&s_count, 1);
-                if (at < kGenList) s_list[at] = ((uint32_t)(row - r0) << 8) | threadIdx.x;
-                else out[(long long)row * g.ld + s] = demand_f64<DT>(g, (uint32_t)s, row);
+                if (at < kGenList) s_list[at] = ((uint32_t)k << 8) | (uint32_t)tid;
+                else *out = demand_f64<DT>(g, (uint32_t)s, r0 + k);
             }
         }
     }
     __syncthreads();
-    const int count = min(s_count, kGenList);
-    for (int k = threadIdx.x; k < count; k += kGenThreads) {
-        const int row = r0 + (int)(s_list[k] >> 8);
-        const long long c = s_block + (s_list[k] & 255u);
-        out[(long long)row * g.ld + c] = demand_f64<DT>(g, (uint32_t)c, row);
+    // Two neighbouring lanes share an entry of a correlated matrix: one draws
+    // the customer's normal, the other the region's, which halves the serial
+    // float64 chain that a block ends with.
+    const int count = min(s_count, kGenList), half = tid & 1;
+    for (int k0_ = 0; k0_ < count; k0_ += kGenThreads / 2) {
+        const int k = k0_ + (tid >> 1);
+        const uint32_t item = s_list[min(k, count - 1)];
+        const int row = r0 + (int)(item >> 8);
+        const long long c = s_block + (item & 255u);
+        const uint32_t index = KIND == 1 && half ? (uint32_t)(g.region[row] & 3) : (uint32_t)row;
+        const double z = std_normal((uint32_t)c, index, KIND == 1 ? (half ? 1u : 0u) : 2u, k0, k1);
+        const double mu = (double)g.mu[row];
+        double x;
+        if (KIND == 1) x = correlated_f64(mu, __shfl_xor_sync(0xffffffffu, z, 1), z);
+        else x = __dadd_rn(mu, __dmul_rn(__dmul_rn(0.3, mu), z));
+        if (!half && k < count) reinterpret_cast<DT *>(g.out)[(long long)row * g.ld + c] = round_demand<DT>(x);
     }
 }
 
@@ -203,7 +302,7 @@ cudaError_t launch_gen_demand(const GenParams &g, int esize, cudaStream_t stream
     const long long bx = (g.S + kGenThreads - 1) / kGenThreads;
     // 64 rows a block spread the four factor draws of a column thin; fewer
     // where that leaves less than four blocks of 256 for each of 152 SMs.
-    int rows = 64;
+    int rows = kGenRows;
     while (rows > 8 && bx * ((g.n + rows - 1) / rows) < 4 * 152) rows >>= 1;
     const dim3 grid((unsigned)bx, (unsigned)((g.n + rows - 1) / rows));
     if (esize == 2) {
