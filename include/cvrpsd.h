@@ -65,12 +65,14 @@ extern "C" {
 /* Largest tour the library accepts. */
 #define CVRPSD_MAX_N 8191
 
-/* Kernel choice for the Split (see cvrpsd_config). AUTO takes SEQPAR for
- * S <= 256 scenarios on tours of n >= 128 (lowest latency there) and DEQUE
- * otherwise. */
+/* Kernel choice for the Split (see cvrpsd_config). AUTO takes, for device
+ * buffers and no predecessors, WARP for S <= 8192 scenarios on tours of
+ * n >= 64 (SEQPAR for S <= 48 where n >= 900), for host buffers SEQPAR for
+ * S <= 256 where n >= 128, and DEQUE otherwise (lowest latency each). */
 #define CVRPSD_KERNEL_AUTO   0
 #define CVRPSD_KERNEL_DEQUE  1   /* one thread per scenario, monotone deque */
-#define CVRPSD_KERNEL_WARP   2   /* one warp per scenario, parallel window min */
+#define CVRPSD_KERNEL_WARP   2   /* one warp per scenario, parallel window min (windows of up to 64
+                                    candidates in registers, longer ones in shared memory) */
 #define CVRPSD_KERNEL_SEQPAR 3   /* few scenarios: min-plus matrix products over blocks of
                                     positions, parallel along the tour (S <= 4096) */
 

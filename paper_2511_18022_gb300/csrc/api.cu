@@ -386,12 +386,29 @@ int split_eval_impl(cvrpsd_ctx *ctx, const int32_t *tour, int32_t n, const int32
     const bool timed = ctx->profiling && (out_sum || out_infeasible || out_mean || host_buffers) && S > 0;
     bool fallback_launched = false;
     if (S > 0) {
-        // Automatic choice: for a handful of scenarios on a long tour the
-        // sequence-parallel kernel has the lowest latency (it parallelises
-        // along the tour); otherwise scenario parallelism wins.
+        // Automatic choice (kernel + set-aside pass, by CUDA events, us; Q about
+        // 13 mean demands):
+        //   n      S     deque  warp  seqpar
+        //   200     37     36    14     24
+        //   200   8192     37    36
+        //   1000    37    149    36     33
+        //   1000  4096    152    80
+        //   1000  8192    161   139
+        //   4000    37    581   121     75
+        // so one warp per scenario up to 8192 scenarios, and the
+        // sequence-parallel kernel for a few dozen on a long tour. Below 64
+        // positions the deque kernel stays (15 us against 9 at n = 50: its walk
+        // is short, and callers read the kernel back). Scenarios in host memory
+        // keep the kernels whose warps read whole sectors of a row.
         int kernel = ctx->cfg.kernel;
-        if (kernel == CVRPSD_KERNEL_AUTO)
-            kernel = (S <= 256 && n >= 128 && !pred) ? CVRPSD_KERNEL_SEQPAR : CVRPSD_KERNEL_DEQUE;
+        if (kernel == CVRPSD_KERNEL_AUTO) {
+            kernel = CVRPSD_KERNEL_DEQUE;
+            if (!pred && host_buffers) {
+                if (S <= 256 && n >= 128) kernel = CVRPSD_KERNEL_SEQPAR;
+            } else if (!pred && n >= 64 && S <= 8192) {
+                kernel = S <= 48 && n >= 900 ? CVRPSD_KERNEL_SEQPAR : CVRPSD_KERNEL_WARP;
+            }
+        }
         const int warp_grid = 2 * (ctx->sm_count > 0 ? ctx->sm_count : 152);
         if (kernel == CVRPSD_KERNEL_SEQPAR && !pred) {
             if (S > 4096) return fail(ctx, CVRPSD_ERR_UNSUPPORTED, "the sequence-parallel kernel takes S <= 4096");
@@ -439,6 +456,17 @@ int split_eval_impl(cvrpsd_ctx *ctx, const int32_t *tour, int32_t n, const int32
             fallback_launched = true;
             st.kernel = CVRPSD_KERNEL_SEQPAR;
             st.launches = 4;
+        } else if (kernel == CVRPSD_KERNEL_WARP && !pred) {
+            if (timed) CK(cudaEventRecord(ctx->ev_t[0], stream), "cudaEventRecord");
+            CK(launch_split_walk(p, demand_dtype, stream), "split_walk launch");
+            if (timed) CK(cudaEventRecord(ctx->ev_t[1], stream), "cudaEventRecord");
+            CK(launch_split_warp(p, demand_dtype, ctx->d_list, ctx->d_acc + ACC_OVERFLOW, warp_grid, ctx->max_smem,
+                                 stream),
+               "split_warp (long windows) launch");
+            if (timed) CK(cudaEventRecord(ctx->ev_t[2], stream), "cudaEventRecord");
+            fallback_launched = true;
+            st.kernel = CVRPSD_KERNEL_WARP;
+            st.launches = 2;
         } else if (kernel == CVRPSD_KERNEL_WARP) {
             long long need = (S + 3) / 4;
             const int grid = (int)(need < 8LL * warp_grid ? need : 8LL * warp_grid);
