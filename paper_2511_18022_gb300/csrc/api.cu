@@ -110,11 +110,11 @@ int ensure_scratch(cvrpsd_ctx *ctx, long long S)
     // Each resource on its own: after a failed allocation the next call
     // retries only what is still missing.
     if (!ctx->d_acc) {
-        CK(dev_alloc(ctx, &ctx->d_acc, ACC_ALLOC_WORDS * sizeof(unsigned long long)), "cudaMalloc(acc)");
+        CK(dev_alloc(ctx, &ctx->d_acc, 2 * ACC_ALLOC_WORDS * sizeof(unsigned long long)), "cudaMalloc(acc)");
         // the sticky status word starts clear and is never zeroed per call
-        CK(cudaMemset(ctx->d_acc, 0, ACC_ALLOC_WORDS * sizeof(unsigned long long)), "clear accumulators");
+        CK(cudaMemset(ctx->d_acc, 0, 2 * ACC_ALLOC_WORDS * sizeof(unsigned long long)), "clear accumulators");
     }
-    if (!ctx->h_acc) CK(host_alloc(ctx, &ctx->h_acc, ACC_ALLOC_WORDS * sizeof(unsigned long long)), "cudaMallocHost(acc)");
+    if (!ctx->h_acc) CK(host_alloc(ctx, &ctx->h_acc, 2 * ACC_ALLOC_WORDS * sizeof(unsigned long long)), "cudaMallocHost(acc)");
     if (!ctx->d_tab) CK(dev_alloc(ctx, &ctx->d_tab, (CVRPSD_MAX_N + 1) * sizeof(TourStep)), "cudaMalloc(tab)");
     if (!ctx->h_tab) CK(host_alloc(ctx, &ctx->h_tab, (CVRPSD_MAX_N + 1) * sizeof(TourStep)), "cudaMallocHost(tab)");
     if (!ctx->ev_tab) CK(cudaEventCreateWithFlags(&ctx->ev_tab, cudaEventDisableTiming), "cudaEventCreate");
@@ -354,15 +354,13 @@ int split_eval_impl(cvrpsd_ctx *ctx, const int32_t *tour, int32_t n, const int32
     int rc = ensure_scratch(ctx, S);
     if (rc) return rc;
 
-    // The pinned table may still be feeding the previous call's copy.
-    CK(cudaEventSynchronize(ctx->ev_tab), "cudaEventSynchronize");
+    // The pinned table may still be feeding an earlier call's copy.
+    if (ctx->tab_use == cvrpsd_ctx::TAB_EVENT) CK(cudaEventSynchronize(ctx->ev_tab), "cudaEventSynchronize");
+    if (ctx->tab_use == cvrpsd_ctx::TAB_UNKNOWN) CK(cudaDeviceSynchronize(), "cudaDeviceSynchronize");
+    ctx->tab_use = cvrpsd_ctx::TAB_FREE;
     int32_t g0 = 0;
     rc = build_tour_table(ctx, tour, n, dist, Q, ctx->h_tab, &g0);
     if (rc) return rc;
-    CK(cudaMemcpyAsync(ctx->d_tab, ctx->h_tab, (size_t)n * sizeof(TourStep), cudaMemcpyHostToDevice, stream),
-       "upload tour table");
-    CK(cudaEventRecord(ctx->ev_tab, stream), "cudaEventRecord");
-    CK(cudaMemsetAsync(ctx->d_acc, 0, ACC_WORDS * sizeof(unsigned long long), stream), "clear accumulators");
 
     SplitParams p{};
     p.tab = ctx->d_tab;
@@ -376,40 +374,82 @@ int split_eval_impl(cvrpsd_ctx *ctx, const int32_t *tour, int32_t n, const int32
     p.K = key_scale(n);
     p.out_cost = out_cost;
     p.acc = ctx->d_acc;
+    p.sticky = ctx->d_acc + ACC_STICKY;
     p.ovf_list = ctx->d_list;
     p.pred = pred;
     p.ldp = ldp;
+
+    const bool want_host = out_sum || out_infeasible || out_mean || host_buffers;
+    // Automatic choice (kernel + set-aside pass, by CUDA events, us; Q about
+    // 13 mean demands):
+    //   n      S     deque  warp  seqpar
+    //   200     37     36    14     24
+    //   200   8192     37    36
+    //   1000    37    149    36     33
+    //   1000  4096    152    80
+    //   1000  8192    161   139
+    //   4000    37    581   121     75
+    // so one warp per scenario up to 8192 scenarios, and the
+    // sequence-parallel kernel for a few dozen on a long tour. Below 64
+    // positions the deque kernel stays (15 us against 9 at n = 50: its walk
+    // is short, and callers read the kernel back). Scenarios in host memory
+    // keep the kernels whose warps read whole sectors of a row.
+    int kernel = ctx->cfg.kernel;
+    if (kernel == CVRPSD_KERNEL_AUTO) {
+        kernel = CVRPSD_KERNEL_DEQUE;
+        if (!pred && host_buffers) {
+            if (S <= 256 && n >= 128) kernel = CVRPSD_KERNEL_SEQPAR;
+        } else if (!pred && n >= 64 && S <= 8192) {
+            kernel = S <= 48 && n >= 900 ? CVRPSD_KERNEL_SEQPAR : CVRPSD_KERNEL_WARP;
+        }
+    }
+    DequeShape shape{128, 1, 16};
+    if (ctx->cfg.threads) shape = DequeShape{ctx->cfg.threads, ctx->cfg.spt, ctx->cfg.ring};
+    if (shape.threads > 256) shape.threads = 256;   // 512 threads: batched path only
+    // The parameter-table walk wherever it applies (one scenario per
+    // thread, no predecessor output, n <= 4032, ...).
+    // Host buffers keep the global-table walk: its prefetch runs twice
+    // as far ahead, which the host link's latency wants.
+    const bool v2_ok = deque2_supported(p, demand_dtype) && !host_buffers;
+    const bool param_walk = kernel == CVRPSD_KERNEL_DEQUE && v2_ok && ctx->cfg.variant != CVRPSD_WALK_GLOBAL_TABLE &&
+                            (ctx->cfg.variant == CVRPSD_WALK_PARAM_TABLE || !ctx->cfg.threads || shape.spt == 1);
+
+    // Host outputs of one kernel: the launch itself hands them over (the
+    // totals of the second accumulator set, see block_finish), and the pass
+    // over set-aside scenarios follows only if there are any. n = 50, S =
+    // 1000 took a table upload, a memset, two kernels and a copy back.
+    const bool one_launch = want_host && S > 0 && kernel != CVRPSD_KERNEL_SEQPAR && !(kernel == CVRPSD_KERNEL_WARP && pred);
+    if (one_launch) {
+        p.acc = ctx->d_acc + ACC_ALLOC_WORDS;
+        p.done = ctx->h_acc + ACC_ALLOC_WORDS;
+        if (ctx->acc_dirty)
+            CK(cudaMemsetAsync(p.acc, 0, ACC_ALLOC_WORDS * sizeof(unsigned long long), stream), "clear accumulators");
+        ctx->acc_dirty = true;   // until this call has read its totals
+    } else {
+        CK(cudaMemsetAsync(ctx->d_acc, 0, ACC_WORDS * sizeof(unsigned long long), stream), "clear accumulators");
+    }
+    const auto upload_table = [&]() {
+        ctx->tab_use = cvrpsd_ctx::TAB_UNKNOWN;
+        cudaError_t e = cudaMemcpyAsync(ctx->d_tab, ctx->h_tab, (size_t)n * sizeof(TourStep), cudaMemcpyHostToDevice,
+                                        stream);
+        if (e == cudaSuccess && !want_host) {   // a call that waits needs no event
+            e = cudaEventRecord(ctx->ev_tab, stream);
+            if (e == cudaSuccess) ctx->tab_use = cvrpsd_ctx::TAB_EVENT;
+        }
+        return e;
+    };
+    if (!(one_launch && param_walk)) CK(upload_table(), "upload tour table");
 
     cvrpsd_stats st{};
     st.overflow = -1;
     st.kernel_ms = st.fallback_ms = -1.0f;
     const bool timed = ctx->profiling && (out_sum || out_infeasible || out_mean || host_buffers) && S > 0;
     bool fallback_launched = false;
+    const int warp_grid = 2 * (ctx->sm_count > 0 ? ctx->sm_count : 152);
+    const auto aside_pass = [&]() {
+        return launch_split_warp(p, demand_dtype, p.ovf_list, p.acc + ACC_OVERFLOW, warp_grid, ctx->max_smem, stream);
+    };
     if (S > 0) {
-        // Automatic choice (kernel + set-aside pass, by CUDA events, us; Q about
-        // 13 mean demands):
-        //   n      S     deque  warp  seqpar
-        //   200     37     36    14     24
-        //   200   8192     37    36
-        //   1000    37    149    36     33
-        //   1000  4096    152    80
-        //   1000  8192    161   139
-        //   4000    37    581   121     75
-        // so one warp per scenario up to 8192 scenarios, and the
-        // sequence-parallel kernel for a few dozen on a long tour. Below 64
-        // positions the deque kernel stays (15 us against 9 at n = 50: its walk
-        // is short, and callers read the kernel back). Scenarios in host memory
-        // keep the kernels whose warps read whole sectors of a row.
-        int kernel = ctx->cfg.kernel;
-        if (kernel == CVRPSD_KERNEL_AUTO) {
-            kernel = CVRPSD_KERNEL_DEQUE;
-            if (!pred && host_buffers) {
-                if (S <= 256 && n >= 128) kernel = CVRPSD_KERNEL_SEQPAR;
-            } else if (!pred && n >= 64 && S <= 8192) {
-                kernel = S <= 48 && n >= 900 ? CVRPSD_KERNEL_SEQPAR : CVRPSD_KERNEL_WARP;
-            }
-        }
-        const int warp_grid = 2 * (ctx->sm_count > 0 ? ctx->sm_count : 152);
         if (kernel == CVRPSD_KERNEL_SEQPAR && !pred) {
             if (S > 4096) return fail(ctx, CVRPSD_ERR_UNSUPPORTED, "the sequence-parallel kernel takes S <= 4096");
             const int blocks = seqpar_blocks(n), W = seqpar_width();
@@ -449,9 +489,7 @@ int split_eval_impl(cvrpsd_ctx *ctx, const int32_t *tour, int32_t n, const int32
             if (timed) CK(cudaEventRecord(ctx->ev_t[0], stream), "cudaEventRecord");
             CK(launch_seqpar(a, demand_dtype, stream), "seqpar launch");
             if (timed) CK(cudaEventRecord(ctx->ev_t[1], stream), "cudaEventRecord");
-            CK(launch_split_warp(p, demand_dtype, ctx->d_list, ctx->d_acc + ACC_OVERFLOW, warp_grid, ctx->max_smem,
-                                 stream),
-               "split_warp (set-aside scenarios) launch");
+            CK(aside_pass(), "split_warp (set-aside scenarios) launch");
             if (timed) CK(cudaEventRecord(ctx->ev_t[2], stream), "cudaEventRecord");
             fallback_launched = true;
             st.kernel = CVRPSD_KERNEL_SEQPAR;
@@ -460,13 +498,8 @@ int split_eval_impl(cvrpsd_ctx *ctx, const int32_t *tour, int32_t n, const int32
             if (timed) CK(cudaEventRecord(ctx->ev_t[0], stream), "cudaEventRecord");
             CK(launch_split_walk(p, demand_dtype, stream), "split_walk launch");
             if (timed) CK(cudaEventRecord(ctx->ev_t[1], stream), "cudaEventRecord");
-            CK(launch_split_warp(p, demand_dtype, ctx->d_list, ctx->d_acc + ACC_OVERFLOW, warp_grid, ctx->max_smem,
-                                 stream),
-               "split_warp (long windows) launch");
-            if (timed) CK(cudaEventRecord(ctx->ev_t[2], stream), "cudaEventRecord");
-            fallback_launched = true;
             st.kernel = CVRPSD_KERNEL_WARP;
-            st.launches = 2;
+            st.launches = 1;
         } else if (kernel == CVRPSD_KERNEL_WARP) {
             long long need = (S + 3) / 4;
             const int grid = (int)(need < 8LL * warp_grid ? need : 8LL * warp_grid);
@@ -477,19 +510,7 @@ int split_eval_impl(cvrpsd_ctx *ctx, const int32_t *tour, int32_t n, const int32
             st.kernel = CVRPSD_KERNEL_WARP;
             st.launches = 1;
         } else {
-            DequeShape shape{128, 1, 16};
-            if (ctx->cfg.threads) shape = DequeShape{ctx->cfg.threads, ctx->cfg.spt, ctx->cfg.ring};
-            if (shape.threads > 256) shape.threads = 256;   // 512 threads: batched path only
-            // The parameter-table walk wherever it applies (one scenario per
-            // thread, no predecessor output, n <= 4032, ...).
-            // Host buffers keep the global-table walk: its prefetch runs twice
-            // as far ahead, which the host link's latency wants.
-            const bool v2_ok = deque2_supported(p, demand_dtype) && !host_buffers;
-            const int variant = ctx->cfg.variant == CVRPSD_WALK_GLOBAL_TABLE || !v2_ok ? CVRPSD_WALK_GLOBAL_TABLE
-                              : (ctx->cfg.variant == CVRPSD_WALK_PARAM_TABLE || !ctx->cfg.threads || shape.spt == 1)
-                                  ? CVRPSD_WALK_PARAM_TABLE
-                                  : CVRPSD_WALK_GLOBAL_TABLE;
-            if (variant == CVRPSD_WALK_PARAM_TABLE) {
+            if (param_walk) {
                 if (timed) CK(cudaEventRecord(ctx->ev_t[0], stream), "cudaEventRecord");
                 DequeShape ran{};
                 const int rounds = ctx->cfg.rounds;
@@ -507,12 +528,7 @@ int split_eval_impl(cvrpsd_ctx *ctx, const int32_t *tour, int32_t n, const int32
                 st.ring = ran.ring;
                 st.variant = CVRPSD_WALK_PARAM_TABLE;
                 st.rounds = rounds;
-                CK(launch_split_warp(p, demand_dtype, ctx->d_list, ctx->d_acc + ACC_OVERFLOW, warp_grid,
-                                     ctx->max_smem, stream),
-                   "split_warp (set-aside scenarios) launch");
-                st.launches = 2;
-                fallback_launched = true;
-                if (timed) CK(cudaEventRecord(ctx->ev_t[2], stream), "cudaEventRecord");
+                st.launches = 1;
                 goto launched;
             }
             if (host_buffers && !ctx->cfg.threads) shape = DequeShape{128, 1, 16};
@@ -541,37 +557,54 @@ int split_eval_impl(cvrpsd_ctx *ctx, const int32_t *tour, int32_t n, const int32
             st.ring = shape.ring;
             st.variant = CVRPSD_WALK_GLOBAL_TABLE;
             st.launches = 1;
-            // Scenarios the deque kernel set aside (ring too small, a demand above
-            // Q, a negative demand) are evaluated by the warp kernel; with none
-            // set aside its blocks exit at once.
-            CK(launch_split_warp(p, demand_dtype, ctx->d_list, ctx->d_acc + ACC_OVERFLOW, warp_grid,
-                                 ctx->max_smem, stream),
-               "split_warp (set-aside scenarios) launch");
-            st.launches = 2;
-            fallback_launched = true;
-            if (timed) CK(cudaEventRecord(ctx->ev_t[2], stream), "cudaEventRecord");
         }
     }
 launched:
+    // Scenarios the main kernel set aside (ring or window too long, a demand
+    // above Q, a negative demand) are evaluated by the warp kernel: at once
+    // where the call doesn't look at the totals before it returns (with none
+    // set aside its blocks exit), or once the host has read that there are some.
+    if (S > 0 && !one_launch && st.launches == 1 && !(kernel == CVRPSD_KERNEL_WARP && pred)) {
+        CK(aside_pass(), "split_warp (set-aside scenarios) launch");
+        st.launches = 2;
+        fallback_launched = true;
+        if (timed) CK(cudaEventRecord(ctx->ev_t[2], stream), "cudaEventRecord");
+    }
     ctx->stats = st;
     log_msg(ctx, CVRPSD_LOG_DEBUG, "split n=%d S=%lld: kernel %d walk %d threads %d spt %d ring %d rounds %d", n,
             (long long)S, st.kernel, st.variant, st.threads, st.spt, st.ring, st.rounds);
-    if (!out_sum && !out_infeasible && !out_mean && !host_buffers) return CVRPSD_OK;
+    if (!want_host) return CVRPSD_OK;
 
-    CK(cudaMemcpyAsync(ctx->h_acc, ctx->d_acc, ACC_WORDS * sizeof(unsigned long long), cudaMemcpyDeviceToHost,
-                       stream),
-       "read accumulators");
+    unsigned long long *a = ctx->h_acc + (one_launch ? ACC_ALLOC_WORDS : 0);
+    if (!one_launch)
+        CK(cudaMemcpyAsync(a, p.acc, ACC_WORDS * sizeof(unsigned long long), cudaMemcpyDeviceToHost, stream),
+           "read accumulators");
     CK(cudaStreamSynchronize(stream), "cudaStreamSynchronize");
-    const unsigned long long *a = ctx->h_acc;
-    ctx->stats.overflow = (int64_t)a[ACC_OVERFLOW];
+    ctx->tab_use = cvrpsd_ctx::TAB_FREE;
     if (timed) {
         float ms = 0;
         CK(cudaEventElapsedTime(&ms, ctx->ev_t[0], ctx->ev_t[1]), "cudaEventElapsedTime");
         ctx->stats.kernel_ms = ms;
-        if (fallback_launched) {
-            CK(cudaEventElapsedTime(&ms, ctx->ev_t[1], ctx->ev_t[2]), "cudaEventElapsedTime");
-            ctx->stats.fallback_ms = ms;
-        }
+    }
+    if (one_launch && a[ACC_OVERFLOW]) {
+        if (param_walk) CK(upload_table(), "upload tour table");
+        if (timed) CK(cudaEventRecord(ctx->ev_t[1], stream), "cudaEventRecord");
+        CK(aside_pass(), "split_warp (set-aside scenarios) launch");
+        if (timed) CK(cudaEventRecord(ctx->ev_t[2], stream), "cudaEventRecord");
+        CK(cudaMemcpyAsync(a, p.acc, ACC_WORDS * sizeof(unsigned long long), cudaMemcpyDeviceToHost, stream),
+           "read accumulators");
+        CK(cudaMemsetAsync(p.acc, 0, ACC_ALLOC_WORDS * sizeof(unsigned long long), stream), "clear accumulators");
+        CK(cudaStreamSynchronize(stream), "cudaStreamSynchronize");
+        ctx->tab_use = cvrpsd_ctx::TAB_FREE;
+        ctx->stats.launches = 2;
+        fallback_launched = true;
+    }
+    if (one_launch) ctx->acc_dirty = false;
+    ctx->stats.overflow = (int64_t)a[ACC_OVERFLOW];
+    if (timed && fallback_launched) {
+        float ms = 0;
+        CK(cudaEventElapsedTime(&ms, ctx->ev_t[1], ctx->ev_t[2]), "cudaEventElapsedTime");
+        ctx->stats.fallback_ms = ms;
     }
     if (a[ACC_STATUS] & ST_INDEX)
         return fail(ctx, CVRPSD_ERR_DEVICE_STATUS, "a kernel index check failed (checked build)");

@@ -16,12 +16,15 @@ struct cvrpsd_ctx {
     int device = 0;
     int sm_count = 0;
     int max_smem = 48 * 1024;              // opt-in shared memory per block
-    unsigned long long *d_acc = nullptr;   // ACC_WORDS
+    unsigned long long *d_acc = nullptr;   // two sets of ACC_ALLOC_WORDS: cleared per call, zero between calls
     int32_t *d_list = nullptr;             // overflow list
     long long list_cap = 0;
     TourStep *d_tab = nullptr;
     TourStep *h_tab = nullptr;             // pinned
     unsigned long long *h_acc = nullptr;   // pinned
+    bool acc_dirty = false;                // the second set may not be zero (a call failed half-way)
+    enum { TAB_FREE, TAB_EVENT, TAB_UNKNOWN } tab_use = TAB_FREE;   // what may still read h_tab: ev_tab, or work of a
+                                                                    // call that failed half-way
     int32_t *d_gen = nullptr;              // mu[n], region[n]
     int32_t *h_gen = nullptr;              // pinned
     cudaEvent_t ev_tab = nullptr;          // tab upload done

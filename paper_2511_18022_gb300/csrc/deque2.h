@@ -56,6 +56,7 @@ struct Walk2Params {
     unsigned long long *acc;   // device [ACC_WORDS]
     int32_t *ovf_list;         // device [S]
     unsigned long long *status;   // device word for index-check status bits
+    unsigned long long *done;     // see SplitParams
 };
 
 // Whether the second walk can run this Split (otherwise the first walk runs):

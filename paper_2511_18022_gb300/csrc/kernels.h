@@ -10,8 +10,13 @@ namespace cvrpsd {
 // ACC_WORDS are zeroed per call; ACC_STICKY collects the status bits of every
 // call until the host reads and clears it (cvrpsd_check_inputs), so that a
 // call that returned without waiting still has its input errors reported.
+//
+// A call that returns host outputs and runs one kernel uses a second set of
+// these words that is zero between calls: the kernel's last block (by
+// ACC_TICKET) hands the totals to the host and clears them again, so the call
+// is that one launch (see block_finish).
 enum AccWord { ACC_SUM = 0, ACC_INFEASIBLE = 1, ACC_OVERFLOW = 2, ACC_STATUS = 3, ACC_WORDS = 4, ACC_STICKY = 4,
-               ACC_ALLOC_WORDS = 8 };
+               ACC_TICKET = 5, ACC_ALLOC_WORDS = 8 };
 
 // Device status bits (ACC_STATUS, and a batch's BACC_STATUS).
 enum StatusBits { ST_NEGATIVE_DEMAND = 1, ST_INDEX = 2 };
@@ -57,6 +62,8 @@ struct SplitParams {
     uint32_t K;                   // key scale: power of two > n
     int32_t *out_cost;            // device [S] or nullptr
     unsigned long long *acc;      // device [ACC_WORDS]
+    unsigned long long *sticky;   // device word that collects status bits over calls
+    unsigned long long *done;     // page-locked host [ACC_WORDS] for the totals, or nullptr (acc keeps them)
     int32_t *ovf_list;            // device [S]: scenarios the deque could not hold
     int16_t *pred;                // device [n][ldp] or nullptr: optimal predecessor of each position
     long long ldp;

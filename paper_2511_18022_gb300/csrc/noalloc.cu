@@ -182,6 +182,7 @@ extern "C" int cvrpsd_split_eval_noalloc(const int32_t *tour, int32_t n, const i
             p.K = key_scale(n);
             p.out_cost = out_cost;
             p.acc = acc;
+            p.sticky = acc + ACC_STICKY;
             p.ovf_list = list;
             // The parameter-table walk where it applies (no device memory beyond
             // the fixed scratch: its table travels in the launch parameters),

@@ -239,6 +239,27 @@ __device__ __forceinline__ void block_accumulate(long long sum, unsigned inf, un
     }
 }
 
+// After block_accumulate, with `done` set: the grid's last block writes the
+// totals to page-locked host memory and clears them for the next call, unless
+// scenarios were set aside (the host then launches the pass over them, which
+// adds to the totals left here). It takes the place of a clearing memset and
+// a copy back around the kernel.
+__device__ __forceinline__ void block_finish(unsigned long long *acc, unsigned long long *done)
+{
+    if (!done || threadIdx.x != 0) return;   // thread 0 did the block's atomics
+    __threadfence();
+    if (atomicAdd(acc + ACC_TICKET, 1ull) != (unsigned long long)gridDim.x - 1) return;
+    __threadfence();
+    volatile unsigned long long *a = acc, *d = done;
+    const bool aside = a[ACC_OVERFLOW] != 0;
+#pragma unroll
+    for (int k = 0; k < ACC_WORDS; ++k) {
+        d[k] = a[k];
+        if (!aside) a[k] = 0;
+    }
+    a[ACC_TICKET] = 0;
+}
+
 // Positions of one prefetch block. GUARD: the block may run past n; the last
 // position reads f(n) instead of pushing. `tab` reads the tour table; the
 // block's first row carries the host's flag for a C_i <= 0 inside the block.
@@ -407,6 +428,7 @@ __global__ void __launch_bounds__(T, d1_min_blocks<T>()) split_deque_kernel(Spli
         p.demand, p.ld, p.S, s_first, n, p.Q, p.L, p.K, p.g0, sbase, tab, tid, p.out_cost, set_aside,
         p.acc + ACC_STATUS, p.pred, p.ldp);
     block_accumulate(sum, 0u, 0u, p.acc);
+    block_finish(p.acc, p.done);
 }
 
 }  // namespace cvrpsd

@@ -362,6 +362,7 @@ __global__ void __launch_bounds__(T, d2_min_blocks<R, T>()) split_deque2_kernel(
         }
     }
     block_accumulate(sum, 0u, 0u, p.acc);
+    block_finish(p.acc, p.done);
 }
 
 }  // namespace cvrpsd

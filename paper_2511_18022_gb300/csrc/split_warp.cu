@@ -274,7 +274,7 @@ __global__ void __launch_bounds__(128) split_warp_kernel(SplitParams p, const in
         if (inf) atomicAdd(p.acc + ACC_INFEASIBLE, (unsigned long long)inf);
         if (status) {
             atomicOr(p.acc + ACC_STATUS, (unsigned long long)status);
-            atomicOr(p.acc + ACC_STICKY, (unsigned long long)status);
+            atomicOr(p.sticky, (unsigned long long)status);
         }
     }
 }
@@ -304,8 +304,9 @@ __global__ void __launch_bounds__(32 * kWalkWarps) split_walk_kernel(SplitParams
             }
         }
     }
-    if (status) atomicOr(p.acc + ACC_STICKY, (unsigned long long)status);
+    if (status) atomicOr(p.sticky, (unsigned long long)status);
     block_accumulate(sum, inf, status, p.acc);
+    block_finish(p.acc, p.done);
 }
 
 cudaError_t launch_split_walk(const SplitParams &p, int esize, cudaStream_t stream)
