@@ -514,12 +514,9 @@ int split_eval_impl(cvrpsd_ctx *ctx, const int32_t *tour, int32_t n, const int32
                 if (timed) CK(cudaEventRecord(ctx->ev_t[0], stream), "cudaEventRecord");
                 DequeShape ran{};
                 const int rounds = ctx->cfg.rounds;
-                // untuned default: 128 threads, rings of 16 (13 blocks fill an SM's
-                // shared memory; rings of 8 need a ring-overflow test on every push
-                // and set aside more scenarios, and measured 20 % slower at n = 1000)
                 const DequeShape want = ctx->cfg.threads ? DequeShape{shape.threads, 1, shape.ring}
-                                                         : DequeShape{128, 1, 16};
-                CK(launch_split_deque2(p, ctx->h_tab, demand_dtype, want, rounds, &ran, stream),
+                                                         : DequeShape{0, 1, 0};
+                CK(launch_split_deque2(p, ctx->h_tab, demand_dtype, want, rounds, ctx->sm_count, &ran, stream),
                    "split_deque2 launch");
                 if (timed) CK(cudaEventRecord(ctx->ev_t[1], stream), "cudaEventRecord");
                 st.kernel = CVRPSD_KERNEL_DEQUE;
@@ -1005,6 +1002,15 @@ int cvrpsd_batch_create(cvrpsd_ctx *ctx, int32_t T, const cvrpsd_tour_desc *tour
     bp.list = b->d_list;
     bp.list_cap = list_cap;
     bp.max_n = max_n;
+    bp.T = T;
+    int smooth = 0;
+    for (int t = 0; t < T; ++t) {
+        const TourStep *c = htab.data() + tab_off[t];
+        int rises = 0;
+        for (int k = 3; k < hd[t].n; ++k) rises += rising(c[k - 3].c, c[k - 2].c, c[k - 1].c, c[k].c);
+        smooth += smooth_table(rises, hd[t].n);
+    }
+    bp.smooth = 2 * smooth > T;
     bp.walk2 = demand_dtype == CVRPSD_I16;
     for (int t = 0; t < T; ++t) bp.walk2 &= batch2_keys_fit(hd[t].n, hd[t].Q, hd[t].K);
     int per_sm = 0;

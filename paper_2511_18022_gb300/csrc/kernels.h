@@ -116,7 +116,7 @@ struct TourDev {
 
 // Batch accumulator header; per tour three words follow: sum, infeasible
 // count, status bits.
-enum BatchAccWord { BACC_COUNTER = 0, BACC_LIST = 1, BACC_STATUS = 2, BACC_WORDS = 4 };
+enum BatchAccWord { BACC_COUNTER = 0, BACC_LIST = 1, BACC_STATUS = 2, BACC_SMOOTH = 3, BACC_WORDS = 4 };
 enum BatchStatusBits { BST_LIST_FULL = 1 };   // shares its word with ST_INDEX (2)
 
 struct BatchParams {
@@ -132,6 +132,9 @@ struct BatchParams {
     int max_n;                    // largest tour
     int walk2;                    // int16 demands and keys that cannot wrap in every tour: the
                                   // second walk runs the one-scenario-per-thread shapes
+    int T;                        // tours
+    int smooth;                   // second walk: 1 if most tours are smooth (smooth_table), 0 if not, -1 if only
+                                  // the device knows (their number in BACC_SMOOTH)
 };
 
 // Dynamic shared memory of the batch kernel: rings, then the current tour's table.
@@ -193,7 +196,7 @@ int seqpar_width();
 cudaError_t launch_neighbors(const int32_t *base, int n, const int32_t *moves, int M, int32_t *out, cudaStream_t st);
 cudaError_t launch_tour_tables(const int32_t *tours, int T, int n, const int32_t *dist, int32_t *D_out,
                                TourStep *tabs, TourDev *descs, const void *demand, long long ld, int Q, int L,
-                               uint32_t K, cudaStream_t st);
+                               uint32_t K, unsigned long long *smooth, cudaStream_t st);
 cudaError_t launch_tour_means(const unsigned long long *acc, int T, long long S, double *mean, long long *sum,
                               long long *inf, cudaStream_t st);
 cudaError_t launch_topk(const float *scores, int M, int k, int32_t *idx_out, cudaStream_t st);

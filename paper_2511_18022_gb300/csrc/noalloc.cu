@@ -190,7 +190,7 @@ extern "C" int cvrpsd_split_eval_noalloc(const int32_t *tour, int32_t n, const i
             DequeShape shape{128, 1, 16};
             cudaError_t e = cudaSuccess;
             if (deque2_supported(p, demand_dtype)) {
-                e = launch_split_deque2(p, g_host_tab, demand_dtype, shape, 0, nullptr, stream);
+                e = launch_split_deque2(p, g_host_tab, demand_dtype, DequeShape{0, 1, 0}, 0, ds.sm_count, nullptr, stream);
             } else {
                 while (split_deque_smem(p, shape) > (size_t)ds.max_smem) {
                     if (shape.threads > 64) shape.threads >>= 1;

@@ -5,6 +5,7 @@
 // needs no host round trip.
 #include <stdint.h>
 
+#include "deque2.h"
 #include "kernels.h"
 #include "tour_table.h"
 
@@ -47,14 +48,16 @@ cudaError_t launch_neighbors(const int32_t *base, int n, const int32_t *moves, i
 // per-block flag for C_i <= 0 is an OR over kPrefetch consecutive positions.
 __global__ void tour_tables_kernel(const int32_t *tours, int T, int n, const int32_t *dist, int32_t *D_out,
                                    TourStep *tabs, TourDev *descs, const void *demand, long long ld, int Q, int L,
-                                   uint32_t K)
+                                   uint32_t K, unsigned long long *smooth)
 {
     __shared__ long long s_len[32];
+    __shared__ int s_rises[32];
     const long long N1 = (long long)n + 1;
     for (int t = blockIdx.x; t < T; t += gridDim.x) {
         const int32_t *tour = tours + (long long)t * n;
         TourStep *tab = tabs + (long long)t * n;
         long long len = 0;
+        int rises = 0;
         const int rounds = (n + blockDim.x - 1) / blockDim.x;
         for (int r = 0; r < rounds; ++r) {
             const int k = r * blockDim.x + threadIdx.x;
@@ -73,6 +76,10 @@ __global__ void tour_tables_kernel(const int32_t *tours, int T, int n, const int
             const unsigned nonpos = __ballot_sync(0xffffffffu, k < n - 1 && c <= 0);
             const int lane = threadIdx.x & 31;
             const unsigned group = (nonpos >> (lane & ~(kPrefetch - 1))) & ((1u << kPrefetch) - 1);
+            // positions whose last three C_i rose (see rising), counted from the fourth of a warp's 32
+            const int c1 = __shfl_up_sync(0xffffffffu, c, 1), c2 = __shfl_up_sync(0xffffffffu, c, 2);
+            const int c3 = __shfl_up_sync(0xffffffffu, c, 3);
+            rises += lane >= 3 && k < n - 1 && rising(c3, c2, c1, c);
             if (k < n) {
                 if ((k % kPrefetch) == 0 && group) row |= kRowFlagNonPositive;
                 tab[k].row = row;
@@ -83,8 +90,13 @@ __global__ void tour_tables_kernel(const int32_t *tours, int T, int n, const int
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) len += __shfl_xor_sync(0xffffffffu, len, o);
         if ((threadIdx.x & 31) == 0) s_len[threadIdx.x >> 5] = len;
+        rises = __reduce_add_sync(0xffffffffu, rises);
+        if ((threadIdx.x & 31) == 0) s_rises[threadIdx.x >> 5] = rises;
         __syncthreads();
         if (threadIdx.x == 0) {
+            int all = 0;
+            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) all += s_rises[w];
+            if (smooth_table(all, n)) atomicAdd(smooth, 1ull);
             long long Dn = 0;
             for (int w = 0; w < (int)(blockDim.x >> 5); ++w) Dn += s_len[w];
             const int last = min(max(tour[n - 1], 1), n);
@@ -109,10 +121,10 @@ __global__ void tour_tables_kernel(const int32_t *tours, int T, int n, const int
 
 cudaError_t launch_tour_tables(const int32_t *tours, int T, int n, const int32_t *dist, int32_t *D_out,
                                TourStep *tabs, TourDev *descs, const void *demand, long long ld, int Q, int L,
-                               uint32_t K, cudaStream_t st)
+                               uint32_t K, unsigned long long *smooth, cudaStream_t st)
 {
     if (T == 0) return cudaSuccess;
-    tour_tables_kernel<<<T < 8192 ? T : 8192, 256, 0, st>>>(tours, T, n, dist, D_out, tabs, descs, demand, ld, Q, L, K);
+    tour_tables_kernel<<<T < 8192 ? T : 8192, 256, 0, st>>>(tours, T, n, dist, D_out, tabs, descs, demand, ld, Q, L, K, smooth);
     return cudaGetLastError();
 }
 

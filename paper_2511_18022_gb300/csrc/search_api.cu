@@ -144,7 +144,7 @@ int cvrpsd_split_eval_tours(cvrpsd_ctx *ctx, const int32_t *d_tours, int32_t T, 
     CK(cudaMemsetAsync(ctx->mt_acc, 0, sizeof(unsigned long long) * (BACC_WORDS + 3LL * T), stream),
        "clear accumulators");
     CK(launch_tour_tables(d_tours, T, n, ctx->mt_dist, nullptr, ctx->mt_tabs, ctx->mt_descs, demand, ld, Q,
-                          L < n ? L : n + 1, K, stream),
+                          L < n ? L : n + 1, K, ctx->mt_acc + BACC_SMOOTH, stream),
        "tour tables");
     BatchParams bp{};
     bp.tours = ctx->mt_descs;
@@ -156,6 +156,8 @@ int cvrpsd_split_eval_tours(cvrpsd_ctx *ctx, const int32_t *d_tours, int32_t T, 
     bp.list = ctx->mt_list;
     bp.list_cap = ctx->mt_list_cap;
     bp.max_n = n;
+    bp.T = T;
+    bp.smooth = -1;
     bp.walk2 = demand_dtype == CVRPSD_I16 && batch2_keys_fit(n, Q, K);
     int per_sm = 0;
     CK(launch_split_batch(bp, demand_dtype, L < n, shape, 0, true, &per_sm, stream), "configure batch kernel");

@@ -51,9 +51,15 @@ constexpr int b2_min_blocks()
     return m < 1 ? 1 : (m > 32 ? 32 : m);
 }
 
-template <int R, int T, bool LCAP>
+// SMOOTH: the walk of smooth tours (see smooth_table), a kernel of its own: both
+// walks in one kernel cost the other one registers (64 tours of n = 100..1000
+// under 8192 scenarios 434 -> 443 us; out of line worse). Where the host has
+// the tables it launches one of the two; where they were built on the device
+// both are launched and the blocks of the one that does not apply exit.
+template <int R, int T, bool LCAP, bool SMOOTH>
 __global__ void __launch_bounds__(T, b2_min_blocks<R, T>()) split_batch2_kernel(BatchParams b)
 {
+    if (b.smooth < 0 && (2 * b.acc[BACC_SMOOTH] > (unsigned long long)b.T) != SMOOTH) return;
     extern __shared__ __align__(16) unsigned char smem[];   // rings [R][T], then the table
     __shared__ int s_item;
     __shared__ long long s_sum[T / 32];
@@ -105,7 +111,7 @@ __global__ void __launch_bounds__(T, b2_min_blocks<R, T>()) split_batch2_kernel(
         p.status = status;
         const long long s = (long long)it.y * T + tid;
         bool aside = false;
-        const int c = walk2_scenario<int16_t, R, T, LCAP, true>(p, tab, s, rs, (uint32_t)tid * 8u, aside);
+        const int c = walk2_scenario<int16_t, R, T, LCAP, true, SMOOTH>(p, tab, s, rs, (uint32_t)tid * 8u, aside);
         long long sum = 0;
         if (s < b.S) {
             if (aside) {
@@ -130,11 +136,11 @@ __global__ void __launch_bounds__(T, b2_min_blocks<R, T>()) split_batch2_kernel(
     }
 }
 
-template <int R, int T, bool LCAP>
+template <int R, int T, bool LCAP, bool SMOOTH>
 static cudaError_t launch2_one(const BatchParams &b, const DequeShape &shape, int grid, bool configure_only,
                                int *blocks_per_sm, cudaStream_t stream)
 {
-    auto kern = split_batch2_kernel<R, T, LCAP>;
+    auto kern = split_batch2_kernel<R, T, LCAP, SMOOTH>;
     const size_t smem = split_batch_smem(b.max_n, shape);
     if (configure_only) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -152,12 +158,22 @@ static cudaError_t launch2_one(const BatchParams &b, const DequeShape &shape, in
     X(128, 64) X(256, 16) X(256, 32) X(512, 16)
 
 template <bool LCAP>
-static cudaError_t dispatch2(const BatchParams &b, const DequeShape &s, int grid, bool configure_only,
+static cudaError_t dispatch2(BatchParams b, const DequeShape &s, int grid, bool configure_only,
                              int *blocks_per_sm, cudaStream_t st)
 {
+    // The walk of smooth tours is compiled for the library's own shape and the
+    // one a tuner picks.
+    if (b.smooth != 0 && s.spt == 1 && s.ring == 16 && (s.threads == 256 || s.threads == 512)) {
+        const cudaError_t e = s.threads == 256
+            ? launch2_one<16, 256, LCAP, true>(b, s, grid, configure_only, blocks_per_sm, st)
+            : launch2_one<16, 512, LCAP, true>(b, s, grid, configure_only, blocks_per_sm, st);
+        if (e != cudaSuccess || b.smooth > 0) return e;
+    } else {
+        b.smooth = 0;
+    }
 #define CVRPSD_CASE(T_, R_)                                                            \
     if (s.threads == T_ && s.spt == 1 && s.ring == R_)                                \
-        return launch2_one<R_, T_, LCAP>(b, s, grid, configure_only, blocks_per_sm, st);
+        return launch2_one<R_, T_, LCAP, false>(b, s, grid, configure_only, blocks_per_sm, st);
     CVRPSD_BATCH2_SHAPES(CVRPSD_CASE)
 #undef CVRPSD_CASE
     return cudaErrorInvalidValue;

@@ -5,9 +5,9 @@
 
 namespace cvrpsd {
 
-cudaError_t dispatch_deque2_i16_cap_fast(const Walk2Params &p, const void *tab, const DequeShape &s, long long grid,
-                                         cudaStream_t st);
-cudaError_t dispatch_deque2_i16_nocap_fast(const Walk2Params &p, const void *tab, const DequeShape &s,
+cudaError_t dispatch_deque2_i16_cap_fast(const Walk2Params &p, const void *tab, const DequeShape &s, bool smooth,
+                                         long long grid, cudaStream_t st);
+cudaError_t dispatch_deque2_i16_nocap_fast(const Walk2Params &p, const void *tab, const DequeShape &s, bool smooth,
                                            long long grid, cudaStream_t st);
 cudaError_t dispatch_deque2_general(const Walk2Params &p, const void *tab, int esize, bool lcap, bool nowrap,
                                     bool large, const DequeShape &s, long long grid, cudaStream_t st);
@@ -17,10 +17,10 @@ cudaError_t dispatch_deque2_i32(const Walk2Params &p, const void *tab, bool lcap
 // A launch's parameters may take at most 32764 bytes.
 static_assert(sizeof(TabParam<kTab2Large>) + sizeof(Walk2Params) <= 32764, "tour table too large for the parameters");
 
-template <typename DT, int R, int T, bool LCAP, bool NOWRAP, int CAP>
+template <typename DT, int R, int T, bool LCAP, bool NOWRAP, int CAP, bool SMOOTH = false>
 static cudaError_t launch2(const Walk2Params &p, const void *tab, long long grid, cudaStream_t st)
 {
-    split_deque2_kernel<DT, R, T, LCAP, NOWRAP, CAP>
+    split_deque2_kernel<DT, R, T, LCAP, NOWRAP, CAP, SMOOTH>
         <<<(unsigned)grid, T, 0, st>>>(p, *static_cast<const TabParam<CAP> *>(tab));
     return cudaGetLastError();
 }
@@ -32,11 +32,13 @@ static cudaError_t launch2(const Walk2Params &p, const void *tab, long long grid
     if (s.threads == T_ && s.ring == R_) return launch2<DT, R_, T_, LCAP, NOWRAP, CAP>(p, tab, grid, st);
 
 template <typename DT, bool LCAP, bool NOWRAP, int CAP>
-static cudaError_t dispatch_wide(const Walk2Params &p, const void *tab, const DequeShape &s, long long grid,
-                                 cudaStream_t st)
+static cudaError_t dispatch_wide(const Walk2Params &p, const void *tab, const DequeShape &s, bool smooth,
+                                 long long grid, cudaStream_t st)
 {
+    if (smooth && s.threads == 128 && s.ring == 16)
+        return launch2<DT, 16, 128, LCAP, NOWRAP, CAP, true>(p, tab, grid, st);
     CVRPSD_D2_SHAPE(64, 8) CVRPSD_D2_SHAPE(64, 16) CVRPSD_D2_SHAPE(128, 8) CVRPSD_D2_SHAPE(128, 16)
-    CVRPSD_D2_SHAPE(256, 8) CVRPSD_D2_SHAPE(256, 16)
+    CVRPSD_D2_SHAPE(256, 8) CVRPSD_D2_SHAPE(256, 16) CVRPSD_D2_SHAPE(64, 32)
     return cudaErrorInvalidValue;
 }
 
@@ -50,9 +52,9 @@ static cudaError_t dispatch_narrow(const Walk2Params &p, const void *tab, const 
 #undef CVRPSD_D2_SHAPE
 
 #if CVRPSD_DEQUE2_PART == 0
-cudaError_t dispatch_deque2_i16_cap_fast(const Walk2Params &p, const void *tab, const DequeShape &s, long long grid,
-                                         cudaStream_t st)
-{ return dispatch_wide<int16_t, true, true, kTab2Small>(p, tab, s, grid, st); }
+cudaError_t dispatch_deque2_i16_cap_fast(const Walk2Params &p, const void *tab, const DequeShape &s, bool smooth,
+                                         long long grid, cudaStream_t st)
+{ return dispatch_wide<int16_t, true, true, kTab2Small>(p, tab, s, smooth, grid, st); }
 
 namespace {
 
@@ -68,22 +70,35 @@ bool keys_fit(const SplitParams &p, int esize)
 
 // Picks the compiled kernel class of this Split and launches it.
 cudaError_t route(const Walk2Params &w, const void *tab, const SplitParams &p, int esize, const DequeShape &s,
-                  long long grid, cudaStream_t st)
+                  bool smooth, long long grid, cudaStream_t st)
 {
     const bool lcap = p.L < p.n, nowrap = keys_fit(p, esize), large = p.n > kTab2Small;
     if (esize == 4) return dispatch_deque2_i32(w, tab, lcap, nowrap, large, s, grid, st);
     if (nowrap && !large) {
-        cudaError_t e = lcap ? dispatch_deque2_i16_cap_fast(w, tab, s, grid, st)
-                             : dispatch_deque2_i16_nocap_fast(w, tab, s, grid, st);
+        cudaError_t e = lcap ? dispatch_deque2_i16_cap_fast(w, tab, s, smooth, grid, st)
+                             : dispatch_deque2_i16_nocap_fast(w, tab, s, smooth, grid, st);
         if (e != cudaErrorInvalidValue) return e;
     }
     return dispatch_deque2_general(w, tab, esize, lcap, nowrap, large, s, grid, st);
 }
 
-// The shape that runs: the requested one if its class compiles it, else (128, 16).
-DequeShape compiled_shape(const SplitParams &p, int esize, const DequeShape &s)
+// The shape that runs: the requested one if its class compiles it, else
+// (128, 16): 13 blocks fill an SM's shared memory; rings of 8 need a
+// ring-overflow test on every push and set aside more scenarios, and measured
+// 20 % slower at n = 1000. Without a request, rings of 32 where all scenarios
+// are resident with them too (14 blocks of 64 on an SM): they cost nothing
+// there (n = 200, S = 100,000 in random order 50.6 against 51.5 us) and hold
+// the long deques of smooth tours (in strips 60.8 against 70.7 us; n = 1000
+// without a route-length cap 271 us against 286 and 2026 more for the 76 % of
+// scenarios that outgrow rings of 16).
+constexpr int kRing32Blocks = 14;
+DequeShape compiled_shape(const SplitParams &p, int esize, const DequeShape &s, int sm_count)
 {
     const bool wide = esize == 2 && keys_fit(p, esize) && p.n <= kTab2Small;
+    if (!s.threads) {
+        const bool fits = p.S <= 64LL * kRing32Blocks * sm_count;
+        return wide && fits ? DequeShape{64, 1, 32} : DequeShape{128, 1, 16};
+    }
     const bool listed = (s.threads == 64 || s.threads == 128 || s.threads == 256) && (s.ring == 8 || s.ring == 16);
     if (wide && listed) return DequeShape{s.threads, 1, s.ring};
     return DequeShape{128, 1, 16};
@@ -102,9 +117,9 @@ bool deque2_supported(const SplitParams &p, int esize)
 }
 
 cudaError_t launch_split_deque2(const SplitParams &p, const TourStep *tab, int esize, const DequeShape &shape,
-                                int rounds, DequeShape *shape_ran, cudaStream_t stream)
+                                int rounds, int sm_count, DequeShape *shape_ran, cudaStream_t stream)
 {
-    const DequeShape s = compiled_shape(p, esize, shape);
+    const DequeShape s = compiled_shape(p, esize, shape, sm_count);
     if (shape_ran) *shape_ran = s;
     // The table as the kernel reads it, built in a host buffer large enough
     // for either capacity (passed by value as the launch's parameters).
@@ -116,7 +131,9 @@ cudaError_t launch_split_deque2(const SplitParams &p, const TourStep *tab, int e
     const size_t words = large ? sizeof(big.nonpos) / 4 : sizeof(small.nonpos) / 4;
     for (size_t k = 0; k < words; ++k) nonpos[k] = 0;
     const unsigned long long pitch = (unsigned long long)p.ld * esize;
+    int rises = 0;
     for (int k = 0; k < p.n; ++k) {
+        rises += k >= 3 && rising(tab[k - 3].c, tab[k - 2].c, tab[k - 1].c, tab[k].c);
         e[k].x = (uint32_t)(tab[k].row & kRowMask);
         e[k].y = (uint32_t)tab[k].c;
         // Position k + 1 >= 2 with C_k > 0 and C_{k+1} > C_k: no back pops.
@@ -144,12 +161,13 @@ cudaError_t launch_split_deque2(const SplitParams &p, const TourStep *tab, int e
     const long long tiles = (p.S + s.threads - 1) / s.threads;
     const long long grid = rounds > 0 ? (tiles + rounds - 1) / rounds : tiles;
     w.stride = grid * s.threads;
-    return route(w, large ? (const void *)&big : (const void *)&small, p, esize, s, grid, stream);
+    return route(w, large ? (const void *)&big : (const void *)&small, p, esize, s,
+                 smooth_table(rises, p.n), grid, stream);
 }
 #elif CVRPSD_DEQUE2_PART == 1
-cudaError_t dispatch_deque2_i16_nocap_fast(const Walk2Params &p, const void *tab, const DequeShape &s,
+cudaError_t dispatch_deque2_i16_nocap_fast(const Walk2Params &p, const void *tab, const DequeShape &s, bool smooth,
                                            long long grid, cudaStream_t st)
-{ return dispatch_wide<int16_t, false, true, kTab2Small>(p, tab, s, grid, st); }
+{ return dispatch_wide<int16_t, false, true, kTab2Small>(p, tab, s, smooth, grid, st); }
 #elif CVRPSD_DEQUE2_PART == 2
 // Every other combination, with the (128, 16) shape only.
 cudaError_t dispatch_deque2_general(const Walk2Params &p, const void *tab, int esize, bool lcap, bool nowrap,

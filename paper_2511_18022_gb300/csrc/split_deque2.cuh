@@ -248,14 +248,21 @@ __device__ __forceinline__ bool walk2_exact(const Deque2 &d, int i0, uint32_t K,
     return __any_sync(0xffffffffu, risk);
 }
 
-template <typename DT, int R, int T, bool LCAP, bool NOWRAP, bool GUARD, typename TB>
+// SMOOTH (see smooth_table): the tests of a block that needs the exact
+// positions and those of one holding some C_i <= 0 share one copy of the code.
+template <typename DT, int R, int T, bool LCAP, bool NOWRAP, bool GUARD, bool SMOOTH, typename TB>
 __device__ __forceinline__ void walk2_block(Deque2 &d, const uint32_t (&q)[kPrefetch2], const TB &tab,
                                             int i0, int n, uint32_t K, uint32_t QK, int L, int Q, uint32_t rs,
                                             bool exact, int &out)
 {
     constexpr bool kBlockOvf = block_ovf<R>();
     const bool general = tab.general(i0);
-    if (exact) {
+    if (SMOOTH) {
+        if (exact || general)
+            walk2_steps<DT, R, T, LCAP, true, NOWRAP, GUARD, true>(d, q, tab, i0, n, K, QK, L, Q, rs, out);
+        else
+            walk2_steps<DT, R, T, false, !kBlockOvf, NOWRAP, GUARD, false>(d, q, tab, i0, n, K, QK, L, Q, rs, out);
+    } else if (exact) {
         if (general)
             walk2_steps<DT, R, T, LCAP, true, NOWRAP, GUARD, true>(d, q, tab, i0, n, K, QK, L, Q, rs, out);
         else
@@ -280,7 +287,7 @@ __device__ __forceinline__ void prefetch2(const char *base, const TB &tab, int i
 // The walk of one scenario (column s; a thread past S walks column 0 and
 // reports nothing: every lane takes part in the votes). Returns f(n) or
 // sets *aside.
-template <typename DT, int R, int T, bool LCAP, bool NOWRAP, typename TB>
+template <typename DT, int R, int T, bool LCAP, bool NOWRAP, bool SMOOTH, typename TB>
 __device__ __forceinline__ int walk2_scenario(const Walk2Params &p, const TB &tab, long long s,
                                               uint32_t rs, uint32_t slot0, bool &aside)
 {
@@ -302,22 +309,25 @@ __device__ __forceinline__ int walk2_scenario(const Walk2Params &p, const TB &ta
     unsigned long long *status = p.status;
     prefetch2<DT, true>(base, tab, 1, n, pitch, status, qa);
     int i0 = 1;
-    // One exactness vote covers both prefetch blocks of an iteration.
+    // One exactness vote covers both prefetch blocks of an iteration; on a
+    // smooth tour a span that fails it asks again for each block.
     constexpr int kSpan = 2 * kPrefetch2;
     for (; i0 + 3 * kPrefetch2 - 1 < n; i0 += 2 * kPrefetch2) {
         prefetch2<DT, false>(base, tab, i0 + kPrefetch2, n, pitch, status, qb);
         const bool ex = walk2_exact<R, T, LCAP, NOWRAP, kSpan>(d, i0, K, L);
-        walk2_block<DT, R, T, LCAP, NOWRAP, false>(d, qa, tab, i0, n, K, QK, L, Q, rs, ex, out);
+        const bool ea = SMOOTH ? ex && walk2_exact<R, T, LCAP, NOWRAP, kPrefetch2>(d, i0, K, L) : ex;
+        walk2_block<DT, R, T, LCAP, NOWRAP, false, SMOOTH>(d, qa, tab, i0, n, K, QK, L, Q, rs, ea, out);
         prefetch2<DT, false>(base, tab, i0 + 2 * kPrefetch2, n, pitch, status, qa);
-        walk2_block<DT, R, T, LCAP, NOWRAP, false>(d, qb, tab, i0 + kPrefetch2, n, K, QK, L, Q, rs, ex, out);
+        const bool eb = SMOOTH ? ex && walk2_exact<R, T, LCAP, NOWRAP, kPrefetch2>(d, i0 + kPrefetch2, K, L) : ex;
+        walk2_block<DT, R, T, LCAP, NOWRAP, false, SMOOTH>(d, qb, tab, i0 + kPrefetch2, n, K, QK, L, Q, rs, eb, out);
     }
     for (; i0 <= n; i0 += 2 * kPrefetch2) {
         prefetch2<DT, true>(base, tab, i0 + kPrefetch2, n, pitch, status, qb);
         const bool ex = walk2_exact<R, T, LCAP, NOWRAP, kSpan>(d, i0, K, L);
-        walk2_block<DT, R, T, LCAP, NOWRAP, true>(d, qa, tab, i0, n, K, QK, L, Q, rs, ex, out);
+        walk2_block<DT, R, T, LCAP, NOWRAP, true, SMOOTH>(d, qa, tab, i0, n, K, QK, L, Q, rs, ex, out);
         if (i0 + kPrefetch2 > n) break;
         prefetch2<DT, true>(base, tab, i0 + 2 * kPrefetch2, n, pitch, status, qa);
-        walk2_block<DT, R, T, LCAP, NOWRAP, true>(d, qb, tab, i0 + kPrefetch2, n, K, QK, L, Q, rs, ex, out);
+        walk2_block<DT, R, T, LCAP, NOWRAP, true, SMOOTH>(d, qb, tab, i0 + kPrefetch2, n, K, QK, L, Q, rs, ex, out);
     }
     aside = d.frozen || d.qmax > (uint32_t)Q;
     return out;
@@ -334,7 +344,7 @@ constexpr int kD2ThreadsPerSM = 2048;
 template <int R, int T>
 constexpr int d2_min_blocks() { return kD2ThreadsPerSM / T; }
 
-template <typename DT, int R, int T, bool LCAP, bool NOWRAP, int CAP>
+template <typename DT, int R, int T, bool LCAP, bool NOWRAP, int CAP, bool SMOOTH>
 __global__ void __launch_bounds__(T, d2_min_blocks<R, T>()) split_deque2_kernel(const Walk2Params p, const __grid_constant__ TabParam<CAP> tab)
 {
     // Rings [R][T] of (g, key) slots: thread t's slot k is at byte
@@ -350,7 +360,7 @@ __global__ void __launch_bounds__(T, d2_min_blocks<R, T>()) split_deque2_kernel(
     for (long long sb = (long long)blockIdx.x * T; sb < p.S; sb += p.stride) {
         const long long s = sb + tid;
         bool aside = false;
-        const int c = walk2_scenario<DT, R, T, LCAP, NOWRAP>(p, tab, s, rs, slot0, aside);
+        const int c = walk2_scenario<DT, R, T, LCAP, NOWRAP, SMOOTH>(p, tab, s, rs, slot0, aside);
         if (s < p.S) {
             if (aside) {
                 const unsigned long long idx = atomicAdd(p.acc + ACC_OVERFLOW, 1ull);
