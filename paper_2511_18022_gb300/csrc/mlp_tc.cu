@@ -1,5 +1,5 @@
-// Layers 1 and 2 of the surrogate network's forward pass on the tensor cores
-// (tcgen05, TMEM). Layer 1:
+// The surrogate network's matrix products on the tensor cores (tcgen05,
+// TMEM). Layer 1, forward:
 //
 // Per tour the layer is a small matrix product: the pre-activations of the
 // H = 256 hidden units at the n positions are W1' (H x 16) times F' (16 x n),
@@ -13,19 +13,31 @@
 // columns, so the mean-pooling over positions is a sum along each thread's
 // own row: ReLU and sum in registers, no cross-thread reduction.
 //
-// One persistent CTA per SM (eight warps), looping over tours:
-//   - W1' is staged in shared memory once, in the canonical K-major layout
-//     without swizzle (8-row x 16-byte core matrices; 128 bytes between the
-//     two core matrices along K, 256 bytes between 8-row groups);
-//   - per chunk of up to 256 positions the threads compute the features
-//     (the cumulative expected load is a block scan) and write F' in the same
-//     layout; one thread issues two MMAs (hidden units 0-127 and 128-255 into
-//     TMEM columns [0, 256) and [256, 512)) and commits them to an mbarrier;
-//   - every warp waits on the mbarrier (bounded: after a fixed number of
-//     polls it records an error and stops), loads its 32 lanes x 32 columns
-//     at a time (tcgen05.ld 32x32b) and accumulates ReLU over the positions.
-// The CTA allocates all 512 TMEM columns once and releases them at exit; its
-// shared-memory request keeps one CTA per SM, so allocations never contend.
+// One persistent CTA per SM holds two lines that take its tours in turn. A
+// line's warps have roles, so that the features of later chunks, the MMAs of
+// the next piece and the pooling of this one overlap:
+//   - four producer warps, each a tour of its own at a time: per 32 positions
+//     (one per lane) a warp gathers the features (a step ahead), forms the
+//     cumulative expected load by a scan and writes F' into one of its four
+//     stages of shared memory, 128 positions each;
+//   - one thread issues the MMAs of a stage (hidden units 0-127 and 128-255)
+//     into the line's half of tensor memory;
+//   - eight pooling warps read it (tcgen05.ld 32x32b) and accumulate, position
+//     after position.
+// The stages are handed on by mbarriers, with waits that give up after a fixed
+// number of polls (all roles then stop and an error is recorded). Operands lie in the canonical K-major layout without swizzle
+// (8-row x 16-byte core matrices; 128 bytes between the two core matrices
+// along K, 256 bytes between 8-row groups).
+//
+// What bounds it: the pooling's two operations per (unit, position), 210 M
+// pairs for 4096 tours of n = 200 (10.8 us at one ALU-pipe maximum per two
+// clocks; a tcgen05.ld takes about 175 clocks and an addition waits 4 for the
+// one before, which four pooling warps on a scheduler hide). 81 us with one
+// chunk at a time per CTA, each step behind the one before it. The producers'
+// 1000 clocks a step are latency, so a producer's stages hold a tour or more;
+// a stage's way through the waits of the three roles takes about 1250 clocks
+// beside its pooling, so one stage of 128 positions per line (34 us) beats two
+// of 64 (40 us).
 #include <cuda_bf16.h>
 #include <stdint.h>
 
@@ -37,35 +49,31 @@ namespace cvrpsd {
 namespace {
 
 constexpr int kTcThreads = 256;          // eight warps
-constexpr int kTcChunk = 256;            // positions per MMA (N <= 256)
 constexpr int kTcK = 16;                 // one kind::f16 MMA step
 constexpr uint32_t kTmemCols = 512;      // two 128 x 256 FP32 accumulators
-// Shared memory the kernel asks for beyond its static arrays: enough that a
-// second CTA cannot share the SM (and its tensor memory).
-constexpr size_t kTcSmemPad = 120 * 1024;
 
-__global__ void __launch_bounds__(kTcThreads, 1) mlp_layer1_tc_kernel(MlpLayer1Args a)
+constexpr int kF1Piece = 128;            // positions per stage
+constexpr int kF1Lines = 2;
+constexpr int kF1Pool = 8;               // pooling warps of a line: 0-7 and 8-15
+constexpr int kF1Prod = 4;               // producer warps of a line: 16-19 and 20-23
+// F' stages of a producer, and their size (backward: with FP32 features after
+// the operand). 128 KB either way: one CTA per SM.
+template <bool BWD> constexpr int f1_depth = BWD ? 2 : 4;
+template <bool BWD> constexpr size_t f1_stage = kF1Piece * kTcK * 2 + (BWD ? kF1Piece * 32 : 0);
+constexpr size_t kF1Smem = kF1Lines * kF1Prod * f1_depth<false> * f1_stage<false>;
+static_assert(kF1Smem == kF1Lines * kF1Prod * f1_depth<true> * f1_stage<true>, "same stages' total");
+constexpr int kF1Threads = 32 * kF1Lines * (kF1Pool + kF1Prod + 1);   // MMA warps 24 and 25
+
+__device__ __forceinline__ uint32_t pack_bf16x2(__nv_bfloat16 a, __nv_bfloat16 b)
 {
-    __shared__ __align__(128) unsigned char s_w1[kMlpH * kTcK * 2];      // W1' (H x 16), 8 KB
-    __shared__ __align__(128) unsigned char s_f[kTcChunk * kTcK * 2];    // F' (256 x 16), 8 KB
-    __shared__ __align__(8) unsigned long long s_mbar;
-    __shared__ uint32_t s_tmem;
-    __shared__ float s_part[kTcThreads / 32];
-    __shared__ float s_carry;
-    __shared__ int s_abort;
-    extern __shared__ unsigned char s_pad[];   // occupancy guard only (kTcSmemPad bytes)
-    (void)s_pad;
+    return (uint32_t)__bfloat16_as_ushort(a) | ((uint32_t)__bfloat16_as_ushort(b) << 16);
+}
 
-    const int j = threadIdx.x, lane = j & 31, w = j >> 5;
-    const int n = a.n;
-    const long long N1 = (long long)n + 1;
-    const uint32_t w1_s = (uint32_t)__cvta_generic_to_shared(s_w1);
-    const uint32_t f_s = (uint32_t)__cvta_generic_to_shared(s_f);
-    const uint32_t mbar = (uint32_t)__cvta_generic_to_shared(&s_mbar);
-
-    // W1' = [W1 | b1 | W1 | 0]: row h, columns 0..4 and 6..10 weights, 5 bias,
-    // 11..15 zero.
-    for (int e = j; e < kMlpH * kTcK; e += kTcThreads) {
+// W1' = [W1 | b1 | W1 | 0] in shared memory: row h, columns 0..4 and 6..10
+// weights, 5 bias, 11..15 zero.
+__device__ __forceinline__ void stage_w1(const MlpLayer1Args &a, unsigned char *s_w1, int tid, int threads)
+{
+    for (int e = tid; e < kMlpH * kTcK; e += threads) {
         const int h = e / kTcK, k = e % kTcK;
         __nv_bfloat16 v = __float2bfloat16_rn(0.0f);
         if (k < kMlpIn1) v = a.w1[h * kMlpIn1 + k];
@@ -73,258 +81,480 @@ __global__ void __launch_bounds__(kTcThreads, 1) mlp_layer1_tc_kernel(MlpLayer1A
         else if (k < 2 * kMlpIn1 + 1) v = a.w1[h * kMlpIn1 + k - kMlpIn1 - 1];
         *reinterpret_cast<__nv_bfloat16 *>(s_w1 + tc::kmajor_offset(h, k, 2)) = v;
     }
-    if (j == 0) {
-        tc::mbar_init(mbar);
+}
+
+// The 16 columns of F' for one position: feature pairs and the bias's 1.
+__device__ __forceinline__ void feature_row(bool valid, const float4 &cu, float cum, __nv_bfloat16 (&f)[kTcK])
+{
+#pragma unroll
+    for (int q = 0; q < kTcK; ++q) f[q] = __float2bfloat16_rn(0.0f);
+    if (valid) {
+        const float v[kMlpIn1] = {cu.x, cu.y, cu.z, cu.w, cum - floorf(cum)};
+#pragma unroll
+        for (int q = 0; q < kMlpIn1; ++q) {
+            f[q] = __float2bfloat16_rn(v[q]);
+            f[q + kMlpIn1 + 1] = __float2bfloat16_rn(v[q] - __bfloat162float(f[q]));
+        }
+        f[kMlpIn1] = __float2bfloat16_rn(1.0f);
+    }
+}
+
+// Row j of F': two 16-byte halves (k 0..7 and 8..15).
+__device__ __forceinline__ void store_feature_row(unsigned char *s_f, int j, const __nv_bfloat16 (&f)[kTcK])
+{
+#pragma unroll
+    for (int half_k = 0; half_k < 2; ++half_k) {
+        const __nv_bfloat16 *p = f + half_k * 8;
+        *reinterpret_cast<uint4 *>(s_f + tc::kmajor_offset(j, half_k * 8, 2)) =
+            make_uint4(pack_bf16x2(p[0], p[1]), pack_bf16x2(p[2], p[3]), pack_bf16x2(p[4], p[5]), pack_bf16x2(p[6], p[7]));
+    }
+}
+
+// What a producer lane gathers for its position: loads a step ahead of the
+// ids' use, two ahead of the values'.
+struct FeatureItem {
+    int c, nx;         // customer there and the next one, as the tour has them
+    float4 cu;         // its features
+    int edge, first;   // length of the edge to the next one (the depot after the last), from the depot
+};
+
+__device__ __forceinline__ void item_ids(const MlpLayer1Args &a, long long t, int k, FeatureItem &x)
+{
+    const int32_t *tour = a.tours + (t < a.T ? t : 0) * a.n;
+    x.c = __ldg(tour + min(k, a.n - 1));
+    x.nx = __ldg(tour + min(k + 1, a.n - 1));
+}
+__device__ __forceinline__ void item_gather(const MlpLayer1Args &a, int k, FeatureItem &x)
+{
+    const int c = min(max(x.c, 1), a.n), nx = k + 1 < a.n ? min(max(x.nx, 1), a.n) : 0;
+    x.cu = __ldg(reinterpret_cast<const float4 *>(a.cust) + c - 1);
+    x.edge = __ldg(a.dist + (long long)c * (a.n + 1) + nx);
+    x.first = __ldg(a.dist + c);
+}
+
+// (a, b) += m * (x, y) as one packed operation.
+__device__ __forceinline__ void fma2(unsigned long long &ab, unsigned long long m2, unsigned long long xy)
+{
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(ab) : "l"(m2), "l"(xy));
+}
+__device__ __forceinline__ float2 unpack2(unsigned long long v)
+{
+    return make_float2(__uint_as_float((uint32_t)v), __uint_as_float((uint32_t)(v >> 32)));
+}
+
+// BWD: layer 1's backward pass in the same roles. With m_hk = [pre_hk > 0] the
+// ReLU mask of hidden unit h at position k, the gradient of tour t is
+//     dW1[h][:] += (dz_th / n) * sum_k m_hk F[k][:]    (F with the bias's 1)
+// so the pooling warps recompute the pre-activations as the forward pass does
+// (no per-position activations are stored) and add the feature rows where the
+// mask is set: a broadcast of the row from shared memory and three packed FP32
+// multiply-adds per (unit, position). Each thread scales its unit's six sums by
+// dz_th / n after a tour; the sums reach the gradient once per CTA.
+template <bool BWD>
+__global__ void __launch_bounds__(kF1Threads, 1) mlp_layer1_tc_kernel(MlpLayer1Args a)
+{
+    constexpr int kF1Depth = f1_depth<BWD>;
+    constexpr size_t kF1StageBytes = f1_stage<BWD>, kF1Rows = kF1Piece * kTcK * 2;   // FP32 rows' offset in a stage
+    __shared__ __align__(128) unsigned char s_w1[kMlpH * kTcK * 2];                    // W1' (H x 16), 8 KB
+    __shared__ __align__(8) unsigned long long s_full[kF1Lines][kF1Prod][kF1Depth], s_empty[kF1Lines][kF1Prod][kF1Depth];
+    __shared__ __align__(8) unsigned long long s_tfull[kF1Lines], s_tempty[kF1Lines];        // TMEM halves
+    __shared__ uint32_t s_tmem;
+    __shared__ int s_abort;
+    __shared__ float s_gw[BWD ? kMlpIn1 + 1 : 1][kMlpH];
+    extern __shared__ __align__(128) unsigned char s_f[];   // F' (128 x 16), 4 KB each: [line][producer][stage]
+
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const int n = a.n;
+    auto bar = [](unsigned long long &b) { return (uint32_t)__cvta_generic_to_shared(&b); };
+
+    stage_w1(a, s_w1, tid, kF1Threads);
+    if (tid == 0) {
+        for (int l = 0; l < kF1Lines; ++l) {
+            for (int p = 0; p < kF1Prod; ++p)
+                for (int k = 0; k < kF1Depth; ++k) {
+                    tc::mbar_init_count(bar(s_full[l][p][k]), 1);
+                    tc::mbar_init_count(bar(s_empty[l][p][k]), BWD ? 1 + kF1Pool : 1);
+                }
+            tc::mbar_init_count(bar(s_tfull[l]), 1);
+            tc::mbar_init_count(bar(s_tempty[l]), kF1Pool);
+        }
+        tc::mbar_init_fence();
         s_abort = 0;
     }
     if (w == 0) tc::tmem_alloc((uint32_t)__cvta_generic_to_shared(&s_tmem), kTmemCols);
+    tc::fence_operands();
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
     const uint32_t tmem = s_tmem;
-    const uint64_t a_desc0 = tc::smem_desc(w1_s, 128, 256);
-    const uint64_t a_desc1 = tc::smem_desc(w1_s + 16 * 256, 128, 256);   // hidden units 128..255
-    const uint64_t b_desc = tc::smem_desc(f_s, 128, 256);
-    // This warp's TMEM rows: lanes 32 (w % 4) .. +31 of accumulator w / 4.
-    const int half = w >> 2;
-    const uint32_t t_row = tmem + ((uint32_t)(32 * (w & 3)) << 16) + (uint32_t)(half * kTcChunk);
-    const int h = half * 128 + 32 * (w & 3) + lane;
-    const __nv_bfloat16 one = __float2bfloat16_rn(1.0f), zero = __float2bfloat16_rn(0.0f);
-    uint32_t parity = 0;
 
-    for (int t = blockIdx.x; t < a.T; t += gridDim.x) {
-        const int32_t *tour = a.tours + (long long)t * n;
-        float len = 0.0f, acc = 0.0f;
-        if (j == 0) s_carry = 0.0f;
-        __syncthreads();
-        for (int k0 = 0; k0 < n; k0 += kTcChunk) {
-            // features of positions k0 .. k0 + 255 (thread j: position k0 + j)
-            const int k = k0 + j;
-            float m = 0.0f;
-            int c = 1;
-            if (k < n) {
-                c = min(max(tour[k], 1), n);
-                m = a.cust[(c - 1) * 4 + 2];
-                const int nx = k + 1 < n ? min(max(tour[k + 1], 1), n) : 0;
-                len += (float)a.dist[(long long)c * N1 + nx];
-                if (k == 0) len += (float)a.dist[c];
-            }
-            float v = m;
+    // A line's tours: blockIdx.x + line * gridDim.x, and on by twice the grid.
+    const long long step = (long long)kF1Lines * gridDim.x;
+    if (w < kF1Lines * kF1Pool) {
+        // pooling: this warp's TMEM rows are lanes 32 (w % 4) .. +31 of one of the line's two accumulators
+        const int line = w >> 3, half = (w >> 2) & 1, h = half * 128 + 32 * (w & 3) + lane;
+        const uint32_t row = tmem + ((uint32_t)(32 * (w & 3)) << 16) + (uint32_t)(line * 256 + half * kF1Piece);
+        int q = 0;                                           // stage number within the line
+        int p = 0;                                           // producer of this tour, and its next stage in bits 4 p ..
+        uint32_t slot = 0;
+        float gw[kMlpIn1 + 1] = {0, 0, 0, 0, 0, 0};
+        for (long long t = blockIdx.x + (long long)line * gridDim.x; t < a.T; t += step, p = (p + 1) % kF1Prod) {
+            float acc = 0.0f;
+            unsigned long long s01 = 0, s23 = 0, s45 = 0;
+            bool ok = true;
+            for (int p0 = 0; p0 < n; p0 += kF1Piece, ++q) {
+                ok = __all_sync(0xffffffffu, tc::mbar_wait_role(bar(s_tfull[line]), (uint32_t)q & 1u, &s_abort, a.err));
+                if (!ok) break;
+                tc::fence_after_sync();
+                // columns past n hold 0 up to the next multiple of 32
+                const int cols = (min(kF1Piece, n - p0) + 31) / 32 * 32;
+                for (int col = 0; col < cols; col += 32) {
+                    uint32_t r[32];
+                    tc::tmem_ld32_issue(row + (uint32_t)col, r);
+                    tc::tmem_ld_wait(r);
+                    if (col + 32 >= cols) {                  // all of the stage is in registers
+                        tc::fence_before_sync();
+                        __syncwarp();
+                        if (lane == 0) tc::mbar_arrive(bar(s_tempty[line]));
+                    }
+                    if (BWD) {
+                        const uint32_t f_s = (uint32_t)((slot >> (4 * p)) & (kF1Depth - 1));
+                        const ulonglong2 *f = reinterpret_cast<const ulonglong2 *>(
+                            s_f + ((line * kF1Prod + p) * kF1Depth + f_s) * kF1StageBytes + kF1Rows) + 2 * col;
 #pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const float u = __shfl_up_sync(0xffffffffu, v, o);
-                if (lane >= o) v += u;
-            }
-            if (lane == 31) s_part[w] = v;
-            __syncthreads();
-            float off = s_carry;
-            for (int q = 0; q < w; ++q) off += s_part[q];
-            const float cum = off + v;
-            __nv_bfloat16 f[kTcK];
+                        for (int k = 0; k < 32; ++k) {
+                            const ulonglong2 f03 = f[2 * k];
+                            const unsigned long long f45 = f[2 * k + 1].x;
+                            const uint32_t m = __uint_as_float(r[k]) > 0.0f ? 0x3f800000u : 0u;
+                            const unsigned long long m2 = ((unsigned long long)m << 32) | m;
+                            fma2(s01, m2, f03.x);
+                            fma2(s23, m2, f03.y);
+                            fma2(s45, m2, f45);
+                        }
+                    } else {
 #pragma unroll
-            for (int q = 0; q < kTcK; ++q) f[q] = zero;
-            if (k < n) {
-                const float v[kMlpIn1] = {a.cust[(c - 1) * 4 + 0], a.cust[(c - 1) * 4 + 1], m,
-                                          a.cust[(c - 1) * 4 + 3], cum - floorf(cum)};
-#pragma unroll
-                for (int q = 0; q < kMlpIn1; ++q) {
-                    f[q] = __float2bfloat16_rn(v[q]);
-                    f[q + kMlpIn1 + 1] = __float2bfloat16_rn(v[q] - __bfloat162float(f[q]));
+                        for (int k = 0; k < 32; ++k) acc += fmaxf(__uint_as_float(r[k]), 0.0f);
+                    }
                 }
-                f[kMlpIn1] = one;
-            }
-            // row j of F': two 16-byte halves (k 0..7 and 8..15)
-#pragma unroll
-            for (int half_k = 0; half_k < 2; ++half_k) {
-                uint4 pack;
-                uint32_t *pw = reinterpret_cast<uint32_t *>(&pack);
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const uint32_t lo = __bfloat16_as_ushort(f[half_k * 8 + 2 * q]);
-                    const uint32_t hi = __bfloat16_as_ushort(f[half_k * 8 + 2 * q + 1]);
-                    pw[q] = lo | (hi << 16);
+                if (BWD) {                                   // the stage's feature rows are read
+                    __syncwarp();
+                    if (lane == 0) tc::mbar_arrive(bar(s_empty[line][p][(slot >> (4 * p)) & (kF1Depth - 1)]));
+                    slot = (slot + (1u << (4 * p))) & (0x1111u * (kF1Depth - 1));
                 }
-                *reinterpret_cast<uint4 *>(s_f + tc::kmajor_offset(j, half_k * 8, 2)) = pack;
             }
-            __syncthreads();
-            if (j == kTcThreads - 1) s_carry = cum;
-            // operands visible to the tensor cores, previous TMEM reads retired
-            tc::fence_operands();
-            tc::fence_before_sync();
-            __syncthreads();
-            tc::fence_after_sync();
-            const int cnt = min(kTcChunk, n - k0);
-            const uint32_t ncols = (uint32_t)((cnt + 31) / 32 * 32);
-            if (j == 0) {
-                const uint32_t idesc = tc::instr_desc(ncols);
-                tc::mma_bf16(tmem, a_desc0, b_desc, idesc, false);
-                tc::mma_bf16(tmem + kTcChunk, a_desc1, b_desc, idesc, false);
-                tc::mma_commit(mbar);
+            if (!ok) break;
+            if (BWD) {
+                const float g = a.dzt[t * kMlpH + h] / (float)n;
+                const float2 u01 = unpack2(s01), u23 = unpack2(s23), u45 = unpack2(s45);
+                gw[0] += g * u01.x;
+                gw[1] += g * u01.y;
+                gw[2] += g * u23.x;
+                gw[3] += g * u23.y;
+                gw[4] += g * u45.x;
+                gw[5] += g * u45.y;
+                continue;
             }
-            if (!tc::mbar_wait(mbar, parity)) {
-                atomicOr(a.err, 1u);
-                s_abort = 1;
-            }
-            parity ^= 1u;
-            tc::fence_after_sync();
-            __syncthreads();
-            if (s_abort) break;
-            // ReLU and sum along this thread's row (positions past n hold 0)
-            for (uint32_t col = 0; col < ncols; col += 32) {
-                float r[32];
-                tc::tmem_ld32(t_row + col, r);
+            const float z = acc / (float)n;
+            if (a.zt) a.zt[t * kMlpIn2 + h] = z;
+            const size_t off = (size_t)(t / kL2M) * kL2Tile + tc::kmajor_offset((int)(t % kL2M), h, kL2Kc);
+            const __nv_bfloat16 hi = __float2bfloat16_rn(z);
+            *reinterpret_cast<__nv_bfloat16 *>(a.z_hi + off) = hi;
+            *reinterpret_cast<__nv_bfloat16 *>(a.z_lo + off) = __float2bfloat16_rn(z - __bfloat162float(hi));
+        }
+        if (BWD) {
+            // the lines' sums together, once to the gradient
+            if (line == 1) {
 #pragma unroll
-                for (int q = 0; q < 32; ++q) acc += fmaxf(r[q], 0.0f);
+                for (int k = 0; k < kMlpIn1 + 1; ++k) s_gw[k][h] = gw[k];
+            }
+            asm volatile("barrier.cta.sync 1, %0;" ::"n"(32 * kF1Lines * kF1Pool) : "memory");
+            if (line == 0) {
+#pragma unroll
+                for (int k = 0; k < kMlpIn1; ++k) atomicAdd(a.gw1 + h * kMlpIn1 + k, gw[k] + s_gw[k][h]);
+                atomicAdd(a.gb1 + h, gw[kMlpIn1] + s_gw[kMlpIn1][h]);
             }
         }
-        if (s_abort) break;
-        // tour length: block sum of the per-thread partial lengths
+    } else if (w < kF1Lines * (kF1Pool + kF1Prod)) {
+        // producer p takes the line's tours p, p + 4, ...
+        const int pw = w - kF1Lines * kF1Pool, line = pw / kF1Prod, p = pw % kF1Prod;
+        const long long stride = step * kF1Prod;
+        unsigned char *stages = s_f + pw * kF1Depth * kF1StageBytes;
+        long long t = blockIdx.x + (long long)line * gridDim.x + p * step;
+        long long t1 = t;                                    // (t1, k1): the step after this one
+        int k1 = lane;
+        auto next = [&](long long &tt, int &kk) {
+            kk += 32;
+            if (kk - lane >= n) {
+                kk = lane;
+                tt += stride;
+            }
+        };
+        FeatureItem x, y;                                    // this step's, the next one's
+        item_ids(a, t, lane, x);
+        item_gather(a, lane, x);
+        next(t1, k1);
+        item_ids(a, t1, k1, y);
+        int q = 0;                                           // stage number of this warp
+        bool ok = true;
+        for (; t < a.T && ok; t += stride) {
+            float carry = 0.0f, len = 0.0f;
+            for (int k0 = 0; k0 < n; k0 += 32) {
+                const int k = k0 + lane;
+                FeatureItem z;
+                long long t2 = t1;
+                int k2 = k1;
+                next(t2, k2);
+                item_ids(a, t2, k2, z);
+                item_gather(a, k1, y);
+                const bool valid = k < n;
+                float v = valid ? x.cu.z : 0.0f;
+                if (valid) len += (float)x.edge;
+                if (k == 0) len += (float)x.first;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) len += __shfl_xor_sync(0xffffffffu, len, o);
-        __syncthreads();
-        if (lane == 0) s_part[w] = len;
-        __syncthreads();
-        if (j == 0) {
-            float tl = 0.0f;
-            for (int q = 0; q < kTcThreads / 32; ++q) tl += s_part[q];
-            a.zt[(long long)t * kMlpIn2 + kMlpH] = (tl - a.len_mean) * a.len_inv_sd;
+                for (int o = 1; o < 32; o <<= 1) {
+                    const float u = __shfl_up_sync(0xffffffffu, v, o);
+                    if (lane >= o) v += u;
+                }
+                const float cum = carry + v;
+                carry = __shfl_sync(0xffffffffu, cum, 31);
+                __nv_bfloat16 f[kTcK];
+                feature_row(valid, x.cu, cum, f);
+                const int s = q % kF1Depth, in = k0 % kF1Piece;
+                if (in == 0)
+                    ok = __all_sync(0xffffffffu, tc::mbar_wait_role(bar(s_empty[line][p][s]), ((uint32_t)(q / kF1Depth) & 1u) ^ 1u,
+                                                                    &s_abort, a.err));
+                if (!ok) break;
+                store_feature_row(stages + s * kF1StageBytes, in + lane, f);
+                if (BWD) {                                   // the pairs' values, as the forward operand has them
+                    float v6[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+#pragma unroll
+                    for (int o = 0; o < kMlpIn1; ++o) v6[o] = __bfloat162float(f[o]) + __bfloat162float(f[o + kMlpIn1 + 1]);
+                    v6[kMlpIn1] = __bfloat162float(f[kMlpIn1]);
+                    float4 *rows = reinterpret_cast<float4 *>(stages + s * kF1StageBytes + kF1Rows) + 2 * (in + lane);
+                    rows[0] = make_float4(v6[0], v6[1], v6[2], v6[3]);
+                    rows[1] = make_float4(v6[4], v6[5], 0.0f, 0.0f);
+                }
+                if (in + 32 == kF1Piece || k0 + 32 >= n) {
+                    tc::fence_operands();
+                    __syncwarp();
+                    if (lane == 0) tc::mbar_arrive(bar(s_full[line][p][s]));
+                    ++q;
+                }
+                x = y;
+                y = z;
+                t1 = t2;
+                k1 = k2;
+            }
+            if (!ok) break;
+            if constexpr (!BWD) {
+                // tour length: sum over the warp; the rest of row t of the head's operand
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) len += __shfl_xor_sync(0xffffffffu, len, o);
+                if (lane == 0) {
+                    const float u = (len - a.len_mean) * a.len_inv_sd;
+                    if (a.zt) a.zt[t * kMlpIn2 + kMlpH] = u;
+                    const size_t off = (size_t)(t / kL2M) * kL2Tile + tc::kmajor_offset((int)(t % kL2M), kMlpH, kL2Kc);
+                    const __nv_bfloat16 hi = __float2bfloat16_rn(u), one = __float2bfloat16_rn(1.0f);
+                    const __nv_bfloat16 lo = __float2bfloat16_rn(u - __bfloat162float(hi)), none = __float2bfloat16_rn(0.0f);
+                    *reinterpret_cast<uint4 *>(a.z_hi + off) = make_uint4(pack_bf16x2(hi, one), 0u, 0u, 0u);
+                    *reinterpret_cast<uint4 *>(a.z_hi + off + 128) = make_uint4(0u, 0u, 0u, 0u);
+                    *reinterpret_cast<uint4 *>(a.z_lo + off) = make_uint4(pack_bf16x2(lo, none), 0u, 0u, 0u);
+                    *reinterpret_cast<uint4 *>(a.z_lo + off + 128) = make_uint4(0u, 0u, 0u, 0u);
+                }
+            }
         }
-        a.zt[(long long)t * kMlpIn2 + h] = acc / (float)n;
+    } else {
+        if (lane == 0) {
+            // Everything that does not change with the piece is formed before the
+            // loop: this thread's chain of waits and issues is on every piece's way.
+            const int line = w - kF1Lines * (kF1Pool + kF1Prod);
+            const uint32_t w1_s = (uint32_t)__cvta_generic_to_shared(s_w1);
+            const uint64_t a_desc0 = tc::smem_desc(w1_s, 128, 256);
+            const uint64_t a_desc1 = tc::smem_desc(w1_s + 16 * 256, 128, 256);   // hidden units 128..255
+            const uint64_t b_desc0 = tc::smem_desc((uint32_t)__cvta_generic_to_shared(s_f + line * (kF1Smem / kF1Lines)), 128, 256);
+            constexpr uint64_t kStageDesc = kF1StageBytes >> 4;                   // between stages, in the descriptor
+            static_assert(kF1Prod * kF1Depth <= 32 && kF1Depth <= 8, "a phase bit per stage, four bits per producer's next stage");
+            const uint32_t full = bar(s_full[line][0][0]), empty = bar(s_empty[line][0][0]);
+            const uint32_t tfull = bar(s_tfull[line]), tempty = bar(s_tempty[line]);
+            const uint32_t acc = tmem + (uint32_t)(line * 256);
+            const uint32_t idesc = tc::instr_desc(kF1Piece), idesc_last = tc::instr_desc((uint32_t)(((n - 1) % kF1Piece) / 32 * 32 + 32));
+            uint32_t phase = 0, slot = 0;                    // full[p][s]'s parity in bit kF1Depth p + s; producer p's s in bits 4 p ..
+            uint32_t tphase = 1;
+            int p = 0;
+            bool ok = true;
+            for (long long t = blockIdx.x + (long long)line * gridDim.x; t < a.T && ok; t += step, p = (p + 1) % kF1Prod) {
+                for (int left = n; left > 0; left -= kF1Piece) {
+                    const uint32_t x = kF1Depth * p + ((slot >> (4 * p)) & (kF1Depth - 1));
+                    ok = tc::mbar_wait_role(full + 8u * x, (phase >> x) & 1u, &s_abort, a.err) &&
+                         tc::mbar_wait_role(tempty, tphase, &s_abort, a.err);
+                    if (!ok) break;
+                    tc::fence_after_sync();
+                    const uint64_t bd = b_desc0 + kStageDesc * x;
+                    const uint32_t id = left > kF1Piece ? idesc : idesc_last;
+                    tc::mma_bf16(acc, a_desc0, bd, id, false);
+                    tc::mma_bf16(acc + kF1Piece, a_desc1, bd, id, false);
+                    tc::mma_commit(tfull);
+                    tc::mma_commit(empty + 8u * x);
+                    phase ^= 1u << x;
+                    slot = (slot + (1u << (4 * p))) & (0x1111u * (kF1Depth - 1));
+                    tphase ^= 1u;
+                }
+            }
+        }
+        __syncwarp();
     }
     tc::fence_before_sync();
     __syncthreads();
     if (w == 0) tc::tmem_dealloc(tmem, kTmemCols);
 }
 
-// ---------------------------------------------------------------- layer 2
+// ---------------------------------------------------------------- the head
 //
-// U = relu([z; t] W2^T + b2) for a tile of 128 tours and 64 of the 256 hidden
-// units: M = 128 tours, N = 64, K = 257 inputs + 1 (the bias rides in W2' as
-// column 257 against a constant 1) padded to 272 = 17 MMA steps. The pooled
-// inputs are FP32; each is split into BF16 hi + lo parts (hi = bf16(v),
-// lo = bf16(v - hi)) and both products are accumulated, so the result keeps
-// about 16 significant bits of the inputs against the exact BF16 weights:
-// the FP32 layer's accuracy on the tensor cores. Operands are staged 16 bytes
-// (one core-matrix row) per store.
-constexpr int kL2K = 272;                 // padded K
-constexpr int kL2Kc = kL2K / 8;           // 16-byte core-matrix columns per row group
-constexpr int kL2M = 128;                 // tours per CTA
-constexpr int kL2N = 64;                  // hidden units per CTA
-constexpr size_t kL2A = (size_t)kL2M * kL2K * 2;   // one 128 x 272 BF16 operand
-constexpr size_t kL2B = (size_t)kL2N * kL2K * 2;
-constexpr size_t kL2Smem = 2 * kL2A + kL2B;        // A hi, A lo, B
-constexpr uint32_t kL2TmemCols = 64;
+// Layer 2, layer 3 and the loss for a tile of 128 tours:
+// U = relu([z; t] W2^T + b2), y = w3 . U + b3. M = 128 tours, N = 256 hidden
+// units in two halves, K = 257 inputs + 1 (the bias rides in W2' as column 257
+// against a constant 1) padded to 272 = 17 MMA steps. The pooled inputs are
+// FP32, split by layer 1 into BF16 hi + lo parts (hi = bf16(v), lo =
+// bf16(v - hi)); both products are accumulated, so the result keeps about 16
+// significant bits of the inputs against the exact BF16 weights: the FP32
+// layer's accuracy on the tensor cores. Layer 1 writes its parts, and the
+// weight update W2', in the operands' own layout, so a CTA fetches them with
+// three bulk copies (the second half of W2' with a fourth, once the first
+// half's MMAs have read its room); a thread owns a tour's row of the
+// accumulator, so the output is a sum in registers.
+//
+// What bounds it: copying 272 KB into a CTA, then latency (one CTA per 128
+// tours: 32 for 4096). Before, with FP32 inputs converted element by element
+// and the output layer apart: 20.6 + 7.1 us for 4096 tours.
+constexpr size_t kHeadSmem = 3 * kL2Tile;          // A hi, A lo, half of W2'
+constexpr uint32_t kHeadTmemCols = 256;
 
-__device__ __forceinline__ uint32_t pack_bf16x2(__nv_bfloat16 a, __nv_bfloat16 b)
-{
-    return (uint32_t)__bfloat16_as_ushort(a) | ((uint32_t)__bfloat16_as_ushort(b) << 16);
-}
-
-__global__ void __launch_bounds__(kTcThreads, 1) mlp_layer2_tc_kernel(const float *zt, int T,
-                                                                      const __nv_bfloat16 *w2,
-                                                                      const __nv_bfloat16 *b2, float *U,
-                                                                      unsigned int *err)
+__global__ void __launch_bounds__(kTcThreads, 1) mlp_head_kernel(MlpHeadArgs a)
 {
     extern __shared__ __align__(128) unsigned char smem[];   // A hi | A lo | B
-    __shared__ __align__(8) unsigned long long s_mbar;
+    __shared__ __align__(8) unsigned long long s_load[2], s_mma[2];
     __shared__ uint32_t s_tmem;
-    unsigned char *a_hi = smem, *a_lo = smem + kL2A, *bw = smem + 2 * kL2A;
+    __shared__ float s_w3[kMlpH];
     const int j = threadIdx.x, lane = j & 31, w = j >> 5;
-    const int t0 = blockIdx.x * kL2M, o0 = blockIdx.y * kL2N;
-    const uint32_t mbar = (uint32_t)__cvta_generic_to_shared(&s_mbar);
-    // B = W2' rows o0 .. o0 + 63: weights, bias at column 257, zeros after;
-    // item = (row, group of 8 columns)
-    for (int e = j; e < kL2N * kL2Kc; e += kTcThreads) {
-        const int r = e / kL2Kc, g = e % kL2Kc;
-        uint32_t pw[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            __nv_bfloat16 v[2];
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int k = 8 * g + 2 * q + h;
-                v[h] = k < kMlpIn2 ? w2[(long long)(o0 + r) * kMlpIn2 + k]
-                                   : (k == kMlpIn2 ? b2[o0 + r] : __float2bfloat16_rn(0.0f));
-            }
-            pw[q] = pack_bf16x2(v[0], v[1]);
+    const long long tile = blockIdx.x;
+    auto bar = [](unsigned long long &b) { return (uint32_t)__cvta_generic_to_shared(&b); };
+    const uint32_t sa = (uint32_t)__cvta_generic_to_shared(smem);
+    const uint32_t sb = sa + 2 * (uint32_t)kL2Tile;
+    if (j == 0) {
+        for (int k = 0; k < 2; ++k) {
+            tc::mbar_init_count(bar(s_load[k]), 1);
+            tc::mbar_init_count(bar(s_mma[k]), 1);
         }
-        *reinterpret_cast<uint4 *>(bw + tc::kmajor_offset(r, 8 * g, kL2Kc)) = make_uint4(pw[0], pw[1], pw[2], pw[3]);
+        tc::mbar_init_fence();
+        tc::mbar_expect(bar(s_load[0]), 3 * (uint32_t)kL2Tile);
+        tc::bulk_load(sa, a.z_hi + tile * kL2Tile, (uint32_t)kL2Tile, bar(s_load[0]));
+        tc::bulk_load(sa + (uint32_t)kL2Tile, a.z_lo + tile * kL2Tile, (uint32_t)kL2Tile, bar(s_load[0]));
+        tc::bulk_load(sb, a.w2b, (uint32_t)kL2Tile, bar(s_load[0]));
     }
-    // A = [z; t; 1] of tours t0 .. t0 + 127, split into BF16 hi and lo parts
-    for (int e = j; e < kL2M * kL2Kc; e += kTcThreads) {
-        const int r = e / kL2Kc, g = e % kL2Kc;
-        const int t = t0 + r;
-        uint32_t ph[4], pl[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            __nv_bfloat16 hi[2], lo[2];
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int k = 8 * g + 2 * q + h;
-                float v = 0.0f;
-                if (t < T) v = k < kMlpIn2 ? zt[(long long)t * kMlpIn2 + k] : (k == kMlpIn2 ? 1.0f : 0.0f);
-                hi[h] = __float2bfloat16_rn(v);
-                lo[h] = __float2bfloat16_rn(v - __bfloat162float(hi[h]));
-            }
-            ph[q] = pack_bf16x2(hi[0], hi[1]);
-            pl[q] = pack_bf16x2(lo[0], lo[1]);
-        }
-        const uint32_t off = tc::kmajor_offset(r, 8 * g, kL2Kc);
-        *reinterpret_cast<uint4 *>(a_hi + off) = make_uint4(ph[0], ph[1], ph[2], ph[3]);
-        *reinterpret_cast<uint4 *>(a_lo + off) = make_uint4(pl[0], pl[1], pl[2], pl[3]);
-    }
-    if (j == 0) tc::mbar_init(mbar);
-    if (w == 0) tc::tmem_alloc((uint32_t)__cvta_generic_to_shared(&s_tmem), kL2TmemCols);
-    tc::fence_operands();
+    s_w3[j] = __bfloat162float(a.w3[j]);
+    if (w == 0) tc::tmem_alloc((uint32_t)__cvta_generic_to_shared(&s_tmem), kHeadTmemCols);
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
     const uint32_t tmem = s_tmem;
     if (j == 0) {
-        const uint32_t idesc = tc::instr_desc(kL2N);
-        const uint32_t sa_hi = (uint32_t)__cvta_generic_to_shared(a_hi);
-        const uint32_t sa_lo = (uint32_t)__cvta_generic_to_shared(a_lo);
-        const uint32_t sb = (uint32_t)__cvta_generic_to_shared(bw);
-        const uint32_t sbo = kL2Kc * 128;
-        for (int step = 0; step < kL2K / 16; ++step) {
-            const uint32_t koff = (uint32_t)step * 256;     // two 16-byte core-matrix columns per step
-            const uint64_t bd = tc::smem_desc(sb + koff, 128, sbo);
-            tc::mma_bf16(tmem, tc::smem_desc(sa_hi + koff, 128, sbo), bd, idesc, step > 0);
-            tc::mma_bf16(tmem, tc::smem_desc(sa_lo + koff, 128, sbo), bd, idesc, true);
-        }
-        tc::mma_commit(mbar);
-    }
-    const bool ok = tc::mbar_wait(mbar, 0);
-    if (!ok && lane == 0) atomicOr(err, 1u);
-    tc::fence_after_sync();
-    __syncthreads();
-    if (ok && w < 4) {
-        // warp w: tours (lanes) 32 w .. 32 w + 31, all 64 hidden columns
-        const int t = t0 + 32 * w + lane;
-        const uint32_t row = tmem + ((uint32_t)(32 * w) << 16);
-#pragma unroll
-        for (int c = 0; c < kL2N; c += 32) {
-            float r[32];
-            tc::tmem_ld32(row + c, r);
-            if (t < T) {
-                float *out = U + (long long)t * kMlpH + o0 + c;
-#pragma unroll
-                for (int q = 0; q < 32; q += 4)
-                    *reinterpret_cast<float4 *>(out + q) = make_float4(fmaxf(r[q], 0.0f), fmaxf(r[q + 1], 0.0f),
-                                                                       fmaxf(r[q + 2], 0.0f), fmaxf(r[q + 3], 0.0f));
+        bool ok = true;
+        for (int half = 0; half < 2 && ok; ++half) {
+            if (half == 1) {
+                // the first half's MMAs have read its weights
+                ok = tc::mbar_wait(bar(s_mma[0]), 0);
+                if (!ok) break;
+                tc::mbar_expect(bar(s_load[1]), (uint32_t)kL2Tile);
+                tc::bulk_load(sb, a.w2b + kL2Tile, (uint32_t)kL2Tile, bar(s_load[1]));
             }
+            // (a copy under way is waited for in any case)
+            ok = tc::mbar_wait(bar(s_load[half]), 0);
+            if (!ok) break;
+            tc::fence_after_sync();
+            const uint32_t idesc = tc::instr_desc(128), sbo = kL2Kc * 128;
+            for (int step = 0; step < kL2K / 16; ++step) {
+                const uint32_t koff = (uint32_t)step * 256;     // two 16-byte core-matrix columns per step
+                const uint64_t bd = tc::smem_desc(sb + koff, 128, sbo);
+                tc::mma_bf16(tmem + half * 128, tc::smem_desc(sa + koff, 128, sbo), bd, idesc, step > 0);
+                tc::mma_bf16(tmem + half * 128, tc::smem_desc(sa + (uint32_t)kL2Tile + koff, 128, sbo), bd, idesc, true);
+            }
+            tc::mma_commit(bar(s_mma[half]));
+        }
+        if (!ok) atomicOr(a.err, 1u);
+    }
+    __syncwarp();
+    // warps 0-3 take the first half's units, 4-7 the second's; lane = tour
+    const int half = w >> 2, row = 32 * (w & 3) + lane;
+    const long long t = tile * kL2M + row;
+    const bool ok = __all_sync(0xffffffffu, tc::mbar_wait(bar(s_mma[half]), 0));
+    tc::fence_after_sync();
+    // w3 . u as 32 sums of every 32nd product, then their sum by halves: the
+    // second half's threads go on from the first half's sums (through shared
+    // memory, over the operands that both halves' MMAs have read).
+    float *s_sum = reinterpret_cast<float *>(smem);          // [32][128]
+    float d[32];
+    auto products = [&]() {
+        const uint32_t at = tmem + ((uint32_t)(32 * (w & 3)) << 16) + (uint32_t)(half * 128);
+#pragma unroll 1
+        for (int c = 0; c < 128; c += 32) {
+            float r[32];
+            tc::tmem_ld32(at + c, r);
+#pragma unroll
+            for (int k = 0; k < 32; ++k) r[k] = fmaxf(r[k], 0.0f);
+            const float *w3 = s_w3 + half * 128 + c;
+#pragma unroll
+            for (int k = 0; k < 32; ++k) d[k] = fmaf(r[k], w3[k], d[k]);
+            if (a.U && t < a.T) {
+                float *out = a.U + t * kMlpH + half * 128 + c;
+#pragma unroll
+                for (int k = 0; k < 32; k += 4)
+                    *reinterpret_cast<float4 *>(out + k) = make_float4(r[k], r[k + 1], r[k + 2], r[k + 3]);
+            }
+        }
+    };
+#pragma unroll
+    for (int k = 0; k < 32; ++k) d[k] = 0.0f;
+    if (ok && half == 0) products();
+    const bool all_ok = __syncthreads_and(ok);               // both halves' MMAs are done
+    if (all_ok && half == 0) {
+#pragma unroll
+        for (int k = 0; k < 32; ++k) s_sum[k * kL2M + row] = d[k];
+    }
+    __syncthreads();
+    if (all_ok && half == 1) {
+#pragma unroll
+        for (int k = 0; k < 32; ++k) d[k] = s_sum[k * kL2M + row];
+        products();
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+            for (int k = 0; k < o; ++k) d[k] += d[k + o];
+        float loss = 0.0f;
+        if (t < a.T) {
+            const float y = d[0] + __bfloat162float(a.b3[0]);
+            a.y[t] = y;
+            if (a.target) {
+                const float e = y - a.target[t];
+                a.dy[t] = 2.0f * e / (float)a.T;
+                loss = e * e / (float)a.T;
+            }
+        }
+        if (a.target) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, o);
+            if (lane == 0) atomicAdd(a.loss, loss);
         }
     }
     tc::fence_before_sync();
     __syncthreads();
-    if (w == 0) tc::tmem_dealloc(tmem, kL2TmemCols);
+    if (w == 0) tc::tmem_dealloc(tmem, kHeadTmemCols);
 }
 
 // ---------------------------------------------------------------- backward GEMMs
 //
 // C (M x N) = A (M x K) B (N x K)^T on the tensor cores, stored or added
-// atomically (split-K over blockIdx.z). One CTA computes a 128 x 160 tile of C
-// in tensor memory, K in chunks of 64 staged in shared memory in the K-major
+// atomically (split-K over blockIdx.z). One CTA computes a 128 x 96 tile of C
+// in tensor memory, K in chunks of 128 staged in shared memory in the K-major
 // layout of the forward kernels. FP32 operands are split into BF16 hi and
 // lo parts (hi = bf16(v), lo = bf16(v - hi)); a product of two split
 // operands takes hi*hi + hi*lo + lo*hi (the lo*lo term, at most 2^-18 of
@@ -333,17 +563,17 @@ __global__ void __launch_bounds__(kTcThreads, 1) mlp_layer2_tc_kernel(const floa
 // are read through an element rule: A(m, k) at a[m * lda + k], or at
 // a[k * lda + m] when transposed (AT); B likewise (BT), FP32 or BF16.
 constexpr int kGM = 128;                       // rows of C per CTA
-constexpr int kGN = 160;                       // columns of C per CTA (5 x 32)
-constexpr int kGK = 64;                        // K per staged chunk
+constexpr int kGN = 96;                        // columns of C per CTA (3 x 32)
+constexpr int kGK = 128;                       // K per staged chunk
 constexpr int kGKc = kGK / 8;                  // 16-byte core-matrix columns per row group
 constexpr size_t kGA = (size_t)kGM * kGK * 2;  // one BF16 A part
 constexpr size_t kGB = (size_t)kGN * kGK * 2;  // one BF16 B part
 constexpr size_t kGSmem = 2 * kGA + 2 * kGB;   // A hi, A lo, B hi, B lo
-// Requested dynamic shared memory: the operands plus padding so that at
-// most two CTAs share an SM (each holds 256 TMEM columns).
-constexpr size_t kGSmemReq = 100 * 1024;
+// Requested dynamic shared memory: the operands plus padding so that one CTA
+// of this kernel runs on an SM.
+constexpr size_t kGSmemReq = 120 * 1024;
 static_assert(kGSmem <= kGSmemReq, "GEMM operands exceed the requested shared memory");
-constexpr uint32_t kGTmemCols = 256;
+constexpr uint32_t kGTmemCols = 128;
 
 struct TcGemm {
     const float *a;          // FP32 A
@@ -380,6 +610,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_gemm_kernel(TcGemm g)
     for (int kc0 = k_begin; kc0 < k_end; kc0 += kGK) {
         // A: item = (row, group of 8 K columns); transposed operands read the
         // row index fastest, so neighbouring threads read neighbouring words
+#pragma unroll 4
         for (int e = j; e < kGM * kGKc; e += kTcThreads) {
             const int r = AT ? e % kGM : e / kGKc, gk = AT ? e / kGM : e % kGKc;
             const int m = m0 + r;
@@ -402,6 +633,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_gemm_kernel(TcGemm g)
             *reinterpret_cast<uint4 *>(a_hi + off) = make_uint4(ph[0], ph[1], ph[2], ph[3]);
             *reinterpret_cast<uint4 *>(a_lo + off) = make_uint4(pl[0], pl[1], pl[2], pl[3]);
         }
+#pragma unroll 3
         for (int e = j; e < kGN * kGKc; e += kTcThreads) {
             const int r = BT ? e % kGN : e / kGKc, gk = BT ? e / kGN : e % kGKc;
             const int nn = n0 + r;
@@ -495,245 +727,32 @@ cudaError_t tc_gemm(const TcGemm &g, cudaStream_t st)
     return cudaGetLastError();
 }
 
-// ---------------------------------------------------------------- layer 1 backward
-//
-// dW1 and db1 on the tensor cores. With m_hk = [pre_hk > 0] the ReLU mask of
-// hidden unit h at position k, the gradient of tour t is
-//     dW1'[h][:] += (dz_th / n) * sum_k m_hk F'[k][:]
-// (F' the 16-column feature rows of the forward pass: hi parts, the 1 of
-// the bias, lo parts), so per tour the contraction is Mask (H x n) times F'
-// (n x 16): the mask is exact in BF16 and F' is the forward operand, and
-// the per-unit factor is applied to the FP32 result. Per chunk of 224
-// positions one CTA recomputes the pre-activations as the forward pass does
-// (two 128 x 224 MMAs into TMEM columns [0, 224) and [256, 480)), turns them
-// into the mask in shared memory (K-major, row h, K = positions), and adds
-// Mask x F'^T into two 128 x 16 accumulators at columns 224 and 480
-// (14 MMA steps each) against F' stored transposed (row = feature, K =
-// position). After the tour's last chunk each thread scales its unit's row
-// by dz_th / n and keeps the sums; they reach the gradient once per CTA.
-constexpr int kBwChunk = 224;                  // positions per chunk (7 x 32)
-constexpr int kBwKc = kBwChunk / 8;            // 28 core-matrix columns along positions
-constexpr size_t kBwMaskHalf = (size_t)128 * kBwChunk * 2;   // one half's mask, BF16
-constexpr size_t kBwF2 = (size_t)16 * kBwChunk * 2;          // F' transposed
-constexpr size_t kBwSmem = 2 * kBwMaskHalf + kBwF2;          // dynamic part
-constexpr uint32_t kBwAcc0 = kBwChunk, kBwAcc1 = 256 + kBwChunk;   // TMEM columns of the two sums
-
-__global__ void __launch_bounds__(kTcThreads, 1) mlp_layer1_bwd_tc_kernel(MlpLayer1Args a)
-{
-    __shared__ __align__(128) unsigned char s_w1[kMlpH * kTcK * 2];      // W1' (H x 16), as forward
-    __shared__ __align__(128) unsigned char s_f[kBwChunk * kTcK * 2];    // F' (224 x 16), as forward
-    __shared__ __align__(8) unsigned long long s_mbar;
-    __shared__ uint32_t s_tmem;
-    __shared__ float s_part[kTcThreads / 32];
-    __shared__ float s_carry;
-    __shared__ int s_abort;
-    extern __shared__ __align__(128) unsigned char s_dyn[];   // mask half 0 | mask half 1 | F' transposed
-    unsigned char *s_mask = s_dyn, *s_f2 = s_dyn + 2 * kBwMaskHalf;
-
-    const int j = threadIdx.x, lane = j & 31, w = j >> 5;
-    const int n = a.n;
-    const uint32_t w1_s = (uint32_t)__cvta_generic_to_shared(s_w1);
-    const uint32_t f_s = (uint32_t)__cvta_generic_to_shared(s_f);
-    const uint32_t m_s = (uint32_t)__cvta_generic_to_shared(s_mask);
-    const uint32_t f2_s = (uint32_t)__cvta_generic_to_shared(s_f2);
-    const uint32_t mbar = (uint32_t)__cvta_generic_to_shared(&s_mbar);
-
-    for (int e = j; e < kMlpH * kTcK; e += kTcThreads) {
-        const int h = e / kTcK, k = e % kTcK;
-        __nv_bfloat16 v = __float2bfloat16_rn(0.0f);
-        if (k < kMlpIn1) v = a.w1[h * kMlpIn1 + k];
-        else if (k == kMlpIn1) v = a.b1[h];
-        else if (k < 2 * kMlpIn1 + 1) v = a.w1[h * kMlpIn1 + k - kMlpIn1 - 1];
-        *reinterpret_cast<__nv_bfloat16 *>(s_w1 + tc::kmajor_offset(h, k, 2)) = v;
-    }
-    if (j == 0) {
-        tc::mbar_init(mbar);
-        s_abort = 0;
-    }
-    if (w == 0) tc::tmem_alloc((uint32_t)__cvta_generic_to_shared(&s_tmem), kTmemCols);
-    tc::fence_before_sync();
-    __syncthreads();
-    tc::fence_after_sync();
-    const uint32_t tmem = s_tmem;
-    const uint64_t a_desc0 = tc::smem_desc(w1_s, 128, 256);
-    const uint64_t a_desc1 = tc::smem_desc(w1_s + 16 * 256, 128, 256);
-    const uint64_t b_desc = tc::smem_desc(f_s, 128, 256);
-    const int half = w >> 2;
-    const int hl = 32 * (w & 3) + lane;                  // row within the half
-    const int h = half * 128 + hl;
-    const uint32_t t_row = tmem + ((uint32_t)(32 * (w & 3)) << 16);
-    const uint32_t pre_col = (uint32_t)(half * 256), acc_col = half ? kBwAcc1 : kBwAcc0;
-    unsigned char *my_mask = s_mask + (size_t)half * kBwMaskHalf;
-    const __nv_bfloat16 one = __float2bfloat16_rn(1.0f), zero = __float2bfloat16_rn(0.0f);
-    const uint32_t one2 = (uint32_t)__bfloat16_as_ushort(one);
-    uint32_t parity = 0;
-    float gw[kMlpIn1 + 1] = {0, 0, 0, 0, 0, 0};
-
-    for (int t = blockIdx.x; t < a.T; t += gridDim.x) {
-        const int32_t *tour = a.tours + (long long)t * n;
-        if (j == 0) s_carry = 0.0f;
-        __syncthreads();
-        int chunk = 0;
-        for (int k0 = 0; k0 < n; k0 += kBwChunk, ++chunk) {
-            // features of positions k0 .. k0 + 223 (thread j < 224: position k0 + j)
-            const int k = k0 + j;
-            const bool valid = j < kBwChunk && k < n;
-            float m = 0.0f;
-            int c = 1;
-            if (valid) {
-                c = min(max(tour[k], 1), n);
-                m = a.cust[(c - 1) * 4 + 2];
-            }
-            float v = m;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const float u = __shfl_up_sync(0xffffffffu, v, o);
-                if (lane >= o) v += u;
-            }
-            if (lane == 31) s_part[w] = v;
-            __syncthreads();
-            float off = s_carry;
-            for (int q = 0; q < w; ++q) off += s_part[q];
-            const float cum = off + v;
-            __nv_bfloat16 f[kTcK];
-#pragma unroll
-            for (int q = 0; q < kTcK; ++q) f[q] = zero;
-            if (valid) {
-                const float v5[kMlpIn1] = {a.cust[(c - 1) * 4 + 0], a.cust[(c - 1) * 4 + 1], m,
-                                           a.cust[(c - 1) * 4 + 3], cum - floorf(cum)};
-#pragma unroll
-                for (int q = 0; q < kMlpIn1; ++q) {
-                    f[q] = __float2bfloat16_rn(v5[q]);
-                    f[q + kMlpIn1 + 1] = __float2bfloat16_rn(v5[q] - __bfloat162float(f[q]));
-                }
-                f[kMlpIn1] = one;
-            }
-            if (j < kBwChunk) {
-#pragma unroll
-                for (int half_k = 0; half_k < 2; ++half_k) {
-                    uint32_t pw[4];
-#pragma unroll
-                    for (int q = 0; q < 4; ++q)
-                        pw[q] = (uint32_t)__bfloat16_as_ushort(f[half_k * 8 + 2 * q]) |
-                                ((uint32_t)__bfloat16_as_ushort(f[half_k * 8 + 2 * q + 1]) << 16);
-                    *reinterpret_cast<uint4 *>(s_f + tc::kmajor_offset(j, half_k * 8, 2)) =
-                        make_uint4(pw[0], pw[1], pw[2], pw[3]);
-                }
-                // the same values transposed: row = feature, K = position
-#pragma unroll
-                for (int q = 0; q < kTcK; ++q)
-                    *reinterpret_cast<__nv_bfloat16 *>(s_f2 + tc::kmajor_offset(q, j, kBwKc)) = f[q];
-            }
-            // the scan carry: the last position of this chunk (thread 223)
-            __syncthreads();
-            if (j == kBwChunk - 1) s_carry = cum;
-            tc::fence_operands();
-            tc::fence_before_sync();
-            __syncthreads();
-            tc::fence_after_sync();
-            const int cnt = min(kBwChunk, n - k0);
-            const uint32_t ncols = (uint32_t)((cnt + 31) / 32 * 32);
-            if (j == 0) {
-                const uint32_t idesc = tc::instr_desc(ncols);
-                tc::mma_bf16(tmem, a_desc0, b_desc, idesc, false);
-                tc::mma_bf16(tmem + 256, a_desc1, b_desc, idesc, false);
-                tc::mma_commit(mbar);
-            }
-            if (!tc::mbar_wait(mbar, parity)) {
-                atomicOr(a.err, 1u);
-                s_abort = 1;
-            }
-            parity ^= 1u;
-            tc::fence_after_sync();
-            __syncthreads();
-            if (s_abort) break;
-            // the mask of this thread's unit: 8 positions per 16-byte store
-            for (uint32_t col = 0; col < (uint32_t)kBwChunk; col += 32) {
-                float r[32];
-                if (col < ncols) tc::tmem_ld32(t_row + pre_col + col, r);
-#pragma unroll
-                for (int g8 = 0; g8 < 4; ++g8) {
-                    uint32_t pw[4];
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const bool m0 = col < ncols && r[g8 * 8 + 2 * q] > 0.0f;
-                        const bool m1 = col < ncols && r[g8 * 8 + 2 * q + 1] > 0.0f;
-                        pw[q] = (m0 ? one2 : 0u) | ((m1 ? one2 : 0u) << 16);
-                    }
-                    *reinterpret_cast<uint4 *>(my_mask + tc::kmajor_offset(hl, (int)col + 8 * g8, kBwKc)) =
-                        make_uint4(pw[0], pw[1], pw[2], pw[3]);
-                }
-            }
-            tc::fence_operands();
-            tc::fence_before_sync();
-            __syncthreads();
-            tc::fence_after_sync();
-            if (j == 0) {
-                const uint32_t idesc = tc::instr_desc(16);
-                const uint32_t sbo = kBwKc * 128;
-                for (int step = 0; step < kBwChunk / 16; ++step) {
-                    const uint32_t koff = (uint32_t)step * 256;
-                    const uint64_t bd = tc::smem_desc(f2_s + koff, 128, sbo);
-                    tc::mma_bf16(tmem + kBwAcc0, tc::smem_desc(m_s + koff, 128, sbo), bd, idesc,
-                                 chunk > 0 || step > 0);
-                    tc::mma_bf16(tmem + kBwAcc1, tc::smem_desc(m_s + (uint32_t)kBwMaskHalf + koff, 128, sbo), bd,
-                                 idesc, chunk > 0 || step > 0);
-                }
-                tc::mma_commit(mbar);
-            }
-            if (!tc::mbar_wait(mbar, parity)) {
-                atomicOr(a.err, 1u);
-                s_abort = 1;
-            }
-            parity ^= 1u;
-            tc::fence_after_sync();
-            __syncthreads();
-            if (s_abort) break;
-        }
-        if (s_abort) break;
-        // this unit's row of Mask x F'^T: hi columns 0-4, bias 5, lo columns 6-10
-        float r[32];
-        tc::tmem_ld32(t_row + acc_col, r);
-        const float g = a.dzt[(long long)t * kMlpIn2 + h] / (float)n;
-#pragma unroll
-        for (int q = 0; q < kMlpIn1; ++q) gw[q] += g * (r[q] + r[q + kMlpIn1 + 1]);
-        gw[kMlpIn1] += g * r[kMlpIn1];
-        tc::fence_before_sync();
-        __syncthreads();                          // TMEM and shared operands are reused by the next tour
-        tc::fence_after_sync();
-    }
-#pragma unroll
-    for (int q = 0; q < kMlpIn1; ++q) atomicAdd(a.gw1 + h * kMlpIn1 + q, gw[q]);
-    atomicAdd(a.gb1 + h, gw[kMlpIn1]);
-    tc::fence_before_sync();
-    __syncthreads();
-    if (w == 0) tc::tmem_dealloc(tmem, kTmemCols);
-}
-
 }  // namespace
 
-cudaError_t mlp_layer2_tc(const float *zt, int T, const __nv_bfloat16 *w2, const __nv_bfloat16 *b2, float *U,
-                          unsigned int *err, cudaStream_t st)
+cudaError_t mlp_head(const MlpHeadArgs &a, cudaStream_t st)
 {
-    cudaError_t e = cudaFuncSetAttribute(mlp_layer2_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)kL2Smem);
+    cudaError_t e = cudaFuncSetAttribute(mlp_head_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kHeadSmem);
     if (e != cudaSuccess) return e;
-    const dim3 grid((unsigned)((T + kL2M - 1) / kL2M), kMlpH / kL2N);
-    mlp_layer2_tc_kernel<<<grid, kTcThreads, kL2Smem, st>>>(zt, T, w2, b2, U, err);
+    mlp_head_kernel<<<(unsigned)((a.T + kL2M - 1) / kL2M), kTcThreads, kHeadSmem, st>>>(a);
     return cudaGetLastError();
 }
 
-cudaError_t mlp_layer1_tc(const MlpLayer1Args &l1, int sm_count, cudaStream_t st)
+template <bool BWD>
+static cudaError_t layer1(const MlpLayer1Args &l1, int sm_count, cudaStream_t st)
 {
-    cudaError_t e = cudaFuncSetAttribute(mlp_layer1_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)kTcSmemPad);
+    cudaError_t e = cudaFuncSetAttribute(mlp_layer1_tc_kernel<BWD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)kF1Smem);
     if (e != cudaSuccess) return e;
     const int grid = l1.T < sm_count ? l1.T : sm_count;
-    mlp_layer1_tc_kernel<<<grid, kTcThreads, kTcSmemPad, st>>>(l1);
+    mlp_layer1_tc_kernel<BWD><<<grid, kF1Threads, kF1Smem, st>>>(l1);
     return cudaGetLastError();
 }
 
-// dZT (T x 257) = dU (T x 256) W2 (256 x 257): A = dU, B(n, k) = W2[k][n].
+cudaError_t mlp_layer1_tc(const MlpLayer1Args &l1, int sm_count, cudaStream_t st) { return layer1<false>(l1, sm_count, st); }
+cudaError_t mlp_layer1_bwd_tc(const MlpLayer1Args &l1, int sm_count, cudaStream_t st) { return layer1<true>(l1, sm_count, st); }
+
+// dZ (T x 256) = dU (T x 256) W2[:, 0..255]: A = dU, B(n, k) = W2[k][n] (the
+// tour length has no gradient to pass on).
 cudaError_t mlp_grad_zt_tc(const float *dU, int T, const __nv_bfloat16 *w2, float *dzt, unsigned int *err,
                            cudaStream_t st)
 {
@@ -743,11 +762,11 @@ cudaError_t mlp_grad_zt_tc(const float *dU, int T, const __nv_bfloat16 *w2, floa
     g.bh = w2;
     g.ldb = kMlpIn2;
     g.M = T;
-    g.N = kMlpIn2;
+    g.N = kMlpH;
     g.K = kMlpH;
     g.k_slab = kMlpH;
     g.out = dzt;
-    g.ldo = kMlpIn2;
+    g.ldo = kMlpH;
     g.err = err;
     return tc_gemm<false, true, true, false>(g, st);
 }
@@ -770,16 +789,6 @@ cudaError_t mlp_grad_w2_tc(const float *dU, const float *zt, int T, float *gw2, 
     g.ldo = kMlpIn2;
     g.err = err;
     return tc_gemm<true, true, false, true>(g, st);
-}
-
-cudaError_t mlp_layer1_bwd_tc(const MlpLayer1Args &l1, int sm_count, cudaStream_t st)
-{
-    cudaError_t e = cudaFuncSetAttribute(mlp_layer1_bwd_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)kBwSmem);
-    if (e != cudaSuccess) return e;
-    const int grid = l1.T < sm_count ? l1.T : sm_count;
-    mlp_layer1_bwd_tc_kernel<<<grid, kTcThreads, kBwSmem, st>>>(l1);
-    return cudaGetLastError();
 }
 
 }  // namespace cvrpsd

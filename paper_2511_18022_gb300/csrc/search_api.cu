@@ -252,7 +252,13 @@ struct cvrpsd_surrogate {
     int32_t *d_dist = nullptr;     // (n+1)^2
     float *d_p = nullptr, *d_g = nullptr, *d_m = nullptr, *d_v = nullptr;
     __nv_bfloat16 *d_pb = nullptr;
-    long long cap = 0;             // workspace rows
+    unsigned char *d_w2b = nullptr;   // W2 and b2 as the head's operand
+    unsigned char *d_zhi = nullptr, *d_zlo = nullptr;   // pooled inputs as the head's operand
+    // Workspaces, one allocation each: the pooled inputs as the head's operand
+    // (every call), and what a training step keeps.
+    unsigned char *ws_infer = nullptr;
+    float *ws_train = nullptr;
+    long long cap_infer = 0, cap_train = 0;   // rows
     float *d_zt = nullptr, *d_U = nullptr, *d_y = nullptr, *d_dy = nullptr, *d_dU = nullptr, *d_dzt = nullptr;
     float *d_loss = nullptr;
     unsigned int *d_err = nullptr;  // set by a tensor-core kernel whose wait gave up
@@ -266,30 +272,40 @@ void sur_free(cvrpsd_surrogate *s)
 {
     if (!s) return;
     for (void *p : {(void *)s->d_cust, (void *)s->d_dist, (void *)s->d_p, (void *)s->d_g, (void *)s->d_m,
-                    (void *)s->d_v, (void *)s->d_pb, (void *)s->d_zt, (void *)s->d_U, (void *)s->d_y,
-                    (void *)s->d_dy, (void *)s->d_dU, (void *)s->d_dzt, (void *)s->d_loss, (void *)s->d_err})
+                    (void *)s->d_v, (void *)s->d_pb, (void *)s->ws_infer, (void *)s->ws_train, (void *)s->d_loss,
+                    (void *)s->d_err, (void *)s->d_w2b})
         if (p) cudaFree(p);
     delete s;
 }
 
-int sur_workspace(cvrpsd_surrogate *s, long long T)
+int sur_workspace(cvrpsd_surrogate *s, long long T, bool train)
 {
     cvrpsd_ctx *ctx = s->ctx;
-    if (T <= s->cap) return CVRPSD_OK;
-    // The old buffers go first; until all new ones exist the capacity is 0,
+    // The old buffer goes first; until the new one exists the capacity is 0,
     // so a failed call leaves nothing that a later call could mistake for room.
-    s->cap = 0;
-    for (float **p : {&s->d_zt, &s->d_U, &s->d_y, &s->d_dy, &s->d_dU, &s->d_dzt}) {
-        if (*p) cudaFree(*p);
-        *p = nullptr;
+    if (T > s->cap_infer) {
+        s->cap_infer = 0;
+        if (s->ws_infer) cudaFree(s->ws_infer);
+        s->ws_infer = nullptr;
+        CK(dev_alloc(ctx, &s->ws_infer, 2 * mlp_tile_bytes(T)), "surrogate workspace");
+        s->cap_infer = T;
+        s->d_zhi = s->ws_infer;
+        s->d_zlo = s->ws_infer + mlp_tile_bytes(T);
     }
-    CK(dev_alloc(ctx, &s->d_zt, sizeof(float) * T * kMlpIn2), "surrogate workspace");
-    CK(dev_alloc(ctx, &s->d_U, sizeof(float) * T * kMlpH), "surrogate workspace");
-    CK(dev_alloc(ctx, &s->d_y, sizeof(float) * T), "surrogate workspace");
-    CK(dev_alloc(ctx, &s->d_dy, sizeof(float) * T), "surrogate workspace");
-    CK(dev_alloc(ctx, &s->d_dU, sizeof(float) * T * kMlpH), "surrogate workspace");
-    CK(dev_alloc(ctx, &s->d_dzt, sizeof(float) * T * kMlpIn2), "surrogate workspace");
-    s->cap = T;
+    if (train && T > s->cap_train) {
+        s->cap_train = 0;
+        if (s->ws_train) cudaFree(s->ws_train);
+        s->ws_train = nullptr;
+        // the rows that are written four floats at a time come first
+        CK(dev_alloc(ctx, &s->ws_train, sizeof(float) * T * (3 * kMlpH + kMlpIn2 + 2)), "surrogate workspace");
+        s->cap_train = T;
+        s->d_U = s->ws_train;
+        s->d_dU = s->d_U + T * kMlpH;
+        s->d_dzt = s->d_dU + T * kMlpH;
+        s->d_zt = s->d_dzt + T * kMlpH;
+        s->d_y = s->d_zt + T * kMlpIn2;
+        s->d_dy = s->d_y + T;
+    }
     return CVRPSD_OK;
 }
 
@@ -302,6 +318,7 @@ MlpWeights weights_of(const cvrpsd_surrogate *s)
     w.b2 = s->d_pb + kOffB2;
     w.w3 = s->d_pb + kOffW3;
     w.b3 = s->d_pb + kOffB3;
+    w.w2b = s->d_w2b;
     return w;
 }
 
@@ -318,6 +335,8 @@ MlpLayer1Args layer1_of(const cvrpsd_surrogate *s, const int32_t *tours, int T)
     a.len_mean = s->len_mean;
     a.len_inv_sd = s->len_inv_sd;
     a.zt = s->d_zt;
+    a.z_hi = s->d_zhi;
+    a.z_lo = s->d_zlo;
     a.err = s->d_err;
     a.sm_count = s->ctx->sm_count > 0 ? s->ctx->sm_count : 1;
     return a;
@@ -334,13 +353,13 @@ int sur_device_error(cvrpsd_surrogate *s)
     return CVRPSD_OK;
 }
 
-int sur_check(cvrpsd_surrogate *s, const int32_t *d_tours, int32_t T)
+int sur_check(cvrpsd_surrogate *s, const int32_t *d_tours, int32_t T, bool train)
 {
     cvrpsd_ctx *ctx = s->ctx;
     if (T < 1) return fail(ctx, CVRPSD_ERR_ARG, "T = %d", T);
     CK(cudaSetDevice(ctx->device), "cudaSetDevice");
     if (!is_device_ptr(d_tours, ctx->device)) return fail(ctx, CVRPSD_ERR_ARG, "tours must be device memory");
-    return sur_workspace(s, T);
+    return sur_workspace(s, T, train);
 }
 
 }  // namespace
@@ -407,6 +426,8 @@ int cvrpsd_surrogate_create(cvrpsd_ctx *ctx, int32_t n, const float *cust, const
     SK(dev_alloc(ctx, &s->d_m, sizeof(float) * kMlpParams), "cudaMalloc");
     SK(dev_alloc(ctx, &s->d_v, sizeof(float) * kMlpParams), "cudaMalloc");
     SK(dev_alloc(ctx, &s->d_pb, sizeof(__nv_bfloat16) * kMlpParams), "cudaMalloc");
+    SK(dev_alloc(ctx, &s->d_w2b, 2 * kL2Tile), "cudaMalloc");
+    SK(cudaMemset(s->d_w2b, 0, 2 * kL2Tile), "memset");
     SK(dev_alloc(ctx, &s->d_loss, sizeof(float)), "cudaMalloc");
     SK(dev_alloc(ctx, &s->d_err, sizeof(unsigned int)), "cudaMalloc");
     SK(cudaMemset(s->d_err, 0, sizeof(unsigned int)), "memset");
@@ -415,7 +436,7 @@ int cvrpsd_surrogate_create(cvrpsd_ctx *ctx, int32_t n, const float *cust, const
     SK(cudaMemcpy(s->d_p, p.data(), sizeof(float) * kMlpParams, cudaMemcpyHostToDevice), "upload");
     SK(cudaMemset(s->d_m, 0, sizeof(float) * kMlpParams), "memset");
     SK(cudaMemset(s->d_v, 0, sizeof(float) * kMlpParams), "memset");
-    SK(mlp_to_bf16(s->d_p, s->d_pb, nullptr), "bf16 copy");
+    SK(mlp_to_bf16(s->d_p, s->d_pb, s->d_w2b, nullptr), "bf16 copy");
     SK(cudaDeviceSynchronize(), "synchronize");
 #undef SK
     *out = s;
@@ -435,11 +456,13 @@ int cvrpsd_surrogate_predict(cvrpsd_surrogate *s, const int32_t *d_tours, int32_
     CVRPSD_TRACE("cvrpsd_surrogate_predict");
     if (!s) return CVRPSD_ERR_ARG;
     cvrpsd_ctx *ctx = s->ctx;
-    int rc = sur_check(s, d_tours, T);
+    int rc = sur_check(s, d_tours, T, false);
     if (rc) return rc;
     if (!is_device_ptr(d_pred, ctx->device)) return fail(ctx, CVRPSD_ERR_ARG, "pred must be device memory");
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream_ptr);
-    CK(mlp_forward(layer1_of(s, d_tours, T), weights_of(s), s->d_U, d_pred, nullptr, nullptr, nullptr, st),
+    MlpLayer1Args l1 = layer1_of(s, d_tours, T);
+    l1.zt = nullptr;   // read by the backward pass only, as U
+    CK(mlp_forward(l1, weights_of(s), nullptr, d_pred, nullptr, nullptr, nullptr, st),
        "surrogate forward");
     return CVRPSD_OK;
 }
@@ -462,14 +485,14 @@ int cvrpsd_surrogate_train_step(cvrpsd_surrogate *s, const int32_t *d_tours, int
     CVRPSD_TRACE("cvrpsd_surrogate_train_step");
     if (!s) return CVRPSD_ERR_ARG;
     cvrpsd_ctx *ctx = s->ctx;
-    int rc = sur_check(s, d_tours, T);
+    int rc = sur_check(s, d_tours, T, true);
     if (rc) return rc;
     if (!is_device_ptr(d_target, ctx->device)) return fail(ctx, CVRPSD_ERR_ARG, "targets must be device memory");
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream_ptr);
     rc = sur_grad(s, d_tours, T, d_target, st);
     if (rc) return rc;
     s->step += 1;
-    CK(mlp_adam(s->d_p, s->d_g, s->d_m, s->d_v, s->d_pb, lr, s->step, st), "adam");
+    CK(mlp_adam(s->d_p, s->d_g, s->d_m, s->d_v, s->d_pb, s->d_w2b, lr, s->step, st), "adam");
     if (d_loss) CK(cudaMemcpyAsync(d_loss, s->d_loss, sizeof(float), cudaMemcpyDeviceToDevice, st), "loss");
     return CVRPSD_OK;
 }
@@ -480,7 +503,7 @@ int cvrpsd_surrogate_gradients(cvrpsd_surrogate *s, const int32_t *d_tours, int3
     CVRPSD_TRACE("cvrpsd_surrogate_gradients");
     if (!s || !h_grad) return CVRPSD_ERR_ARG;
     cvrpsd_ctx *ctx = s->ctx;
-    int rc = sur_check(s, d_tours, T);
+    int rc = sur_check(s, d_tours, T, true);
     if (rc) return rc;
     if (!is_device_ptr(d_target, ctx->device)) return fail(ctx, CVRPSD_ERR_ARG, "targets must be device memory");
     rc = sur_grad(s, d_tours, T, d_target, nullptr);
@@ -507,7 +530,7 @@ int cvrpsd_surrogate_params(cvrpsd_surrogate *s, float *h_get, const float *h_se
     if (count) *count = kMlpParams;
     if (h_set) {
         CK(cudaMemcpy(s->d_p, h_set, sizeof(float) * kMlpParams, cudaMemcpyHostToDevice), "set parameters");
-        CK(mlp_to_bf16(s->d_p, s->d_pb, nullptr), "bf16 copy");
+        CK(mlp_to_bf16(s->d_p, s->d_pb, s->d_w2b, nullptr), "bf16 copy");
         CK(cudaDeviceSynchronize(), "synchronize");
     }
     if (h_get) CK(cudaMemcpy(h_get, s->d_p, sizeof(float) * kMlpParams, cudaMemcpyDeviceToHost), "get parameters");
@@ -550,7 +573,7 @@ int cvrpsd_surrogate_state(cvrpsd_surrogate *s, void *h_get, const void *h_set, 
         CK(cudaMemcpy(s->d_p, src, arr, cudaMemcpyHostToDevice), "restore parameters");
         CK(cudaMemcpy(s->d_m, src + arr, arr, cudaMemcpyHostToDevice), "restore first moments");
         CK(cudaMemcpy(s->d_v, src + 2 * arr, arr, cudaMemcpyHostToDevice), "restore second moments");
-        CK(mlp_to_bf16(s->d_p, s->d_pb, nullptr), "bf16 copy");
+        CK(mlp_to_bf16(s->d_p, s->d_pb, s->d_w2b, nullptr), "bf16 copy");
         CK(cudaDeviceSynchronize(), "synchronize");
         s->step = h.step;
         s->len_mean = h.len_mean;
