@@ -47,11 +47,21 @@ struct TabParam {
     // The walk's view of a table (see TabShared2 for the batch kernel's).
     __device__ __forceinline__ uint2 entry(int i) const { return e[i - 1]; }
     __device__ __forceinline__ uint32_t row(int i) const { return e[i - 1].x & kTab2RowMask; }
-    __device__ __forceinline__ bool general(int i0) const
+    // Flags of the span of two prefetch blocks from i0: read where they are used.
+    __device__ __forceinline__ uint32_t span(int i0) const { return 0; }
+    __device__ __forceinline__ bool general(uint32_t, int i0, int) const
     {
         const int m = (i0 - 1) / kPrefetch2;
         return (nonpos[m >> 5] >> (m & 31)) & 1u;
     }
+    __device__ __forceinline__ bool noback(uint32_t, int i, int) const { return (e[i - 1].x & kTab2NoBack) != 0; }
+    // C_i and demand rows of a prefetch block's positions.
+    struct Costs {};
+    __device__ __forceinline__ Costs costs(int) const { return {}; }
+    __device__ __forceinline__ int cost(const Costs &, int i, int) const { return (int)e[i - 1].y; }
+    struct Rows {};
+    __device__ __forceinline__ Rows rows(int) const { return {}; }
+    __device__ __forceinline__ uint32_t row_at(const Rows &, int i, int) const { return row(i); }
 #endif
 };
 

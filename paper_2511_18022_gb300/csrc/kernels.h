@@ -137,10 +137,12 @@ struct BatchParams {
                                   // the device knows (their number in BACC_SMOOTH)
 };
 
-// Dynamic shared memory of the batch kernel: rings, then the current tour's table.
+// Dynamic shared memory of the batch kernel: rings, then the current tour's
+// table and (second walk) a word of flags for every 8 positions.
 inline size_t split_batch_smem(int max_n, const DequeShape &shape)
 {
-    return (size_t)shape.spt * shape.ring * shape.threads * 8 + (size_t)max_n * sizeof(TourStep);
+    return (size_t)shape.spt * shape.ring * shape.threads * 8 + (size_t)((max_n + 3) / 4 * 4) * sizeof(TourStep) +
+           (size_t)((max_n + 7) / 8) * 4;
 }
 // Persistent deque kernel over all work items; with configure_only it only
 // sets the kernel's shared-memory limit (call before stream capture) and

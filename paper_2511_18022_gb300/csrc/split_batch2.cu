@@ -14,38 +14,60 @@
 
 namespace cvrpsd {
 
-// Shared-memory table entry of position i at byte (i - 1) * 8: x = demand
-// row | kTab2NoBack (no back pops at i) | kTab2SharedGeneral (on the first
-// entry of a prefetch block holding some C_i <= 0 with i < n), y = C_i.
-constexpr uint32_t kTab2SharedGeneral = 1u << 30;
-constexpr uint32_t kTab2SharedRowMask = kTab2SharedGeneral - 1u;
+// The tour's table in shared memory: the demand rows of its positions, their
+// C_i, both up to the next multiple of 4 (the last row and 0 again), so that a
+// prefetch block of 4 positions reads each in one load (1124 -> 1068 us for 64
+// tours of n = 200 under 65,536 scenarios against pairs read per position); and
+// a word of flags for every span of two prefetch blocks (8 positions): bit u
+// where no scenario can pop the back at the span's position u (kTab2NoBack of
+// the parameter table), bit 8 + m where its prefetch block m holds some C_i <= 0
+// with i < n.
+//
+// All threads of a block read the same entries, but a load from shared memory
+// gives the compiler no way to know that. The flags (and the tour's
+// parameters, below) therefore pass through a warp reduction of equal values,
+// whose result it keeps in uniform registers: branches on them are uniform,
+// and the walk takes 40 registers instead of 48, six blocks of 256 on an SM
+// instead of five.
+__device__ __forceinline__ int4 lds4(uint32_t a)
+{
+    int4 v;
+    asm volatile("ld.shared.v4.s32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a));
+    return v;
+}
+__device__ __forceinline__ int lane4(const int4 &v, int u) { return u == 0 ? v.x : u == 1 ? v.y : u == 2 ? v.z : v.w; }
 
 struct TabShared2 {
-    uint32_t a;   // shared-window address of entry 0
+    uint32_t a;       // shared-window address of the rows
+    uint32_t c;       // of the C_i
+    uint32_t f;       // of the flags
     static constexpr int kCap = 1 << 30;
-    __device__ __forceinline__ uint2 entry(int i) const
+    using Costs = int4;
+    using Rows = int4;
+    __device__ __forceinline__ int4 costs(int i0) const { return lds4(c + (uint32_t)(i0 - 1) * 4u); }
+    __device__ __forceinline__ int cost(const int4 &v, int, int u) const { return lane4(v, u); }
+    __device__ __forceinline__ int4 rows(int i0) const { return lds4(a + (uint32_t)(i0 - 1) * 4u); }
+    __device__ __forceinline__ uint32_t row_at(const int4 &v, int, int u) const { return (uint32_t)lane4(v, u); }
+    __device__ __forceinline__ uint32_t span(int i0) const
     {
-        const int2 v = lds2(a + (uint32_t)(i - 1) * 8u);
-        return make_uint2((uint32_t)v.x, (uint32_t)v.y);
+        return __reduce_or_sync(0xffffffffu, (uint32_t)lds1(f + (uint32_t)((i0 - 1) >> 3) * 4u));
     }
-    __device__ __forceinline__ uint32_t row(int i) const
-    {
-        return (uint32_t)lds1(a + (uint32_t)(i - 1) * 8u) & kTab2SharedRowMask;
-    }
-    __device__ __forceinline__ bool general(int i0) const
-    {
-        return ((uint32_t)lds1(a + (uint32_t)(i0 - 1) * 8u) & kTab2SharedGeneral) != 0;
-    }
+    __device__ __forceinline__ bool general(uint32_t fl, int, int at) const { return (fl >> (8 + at / kPrefetch2)) & 1u; }
+    __device__ __forceinline__ bool noback(uint32_t fl, int, int u) const { return (fl >> u) & 1u; }
 };
+static_assert(kPrefetch2 == 4, "a span's flags are for two blocks of four positions");
 
-// Blocks an SM holds: shared memory for the rings and a table of up to 1024
-// positions (1 KB reserved per block), at most 2048 threads and 32 blocks.
-// The registers this leaves (40 or more) keep the per-item tour parameters
-// out of local memory.
+__device__ __forceinline__ uint32_t uniform(uint32_t x) { return __reduce_or_sync(0xffffffffu, x); }
+
+// Blocks an SM holds (and the registers a thread may take): shared memory for
+// the rings and a table of a few hundred positions, or 2048 threads. 256
+// threads with rings of 16: six blocks of 40 registers (64 tours of n = 200
+// under 65,536 scenarios 1116 -> 1096 us, 64 tours of 100 to 1000 under 8192
+// 464 -> 453 us against five of 48; at n = 1000 the table leaves room for five).
 template <int R, int T>
 constexpr int b2_min_blocks()
 {
-    constexpr int by_smem = 233472 / (R * T * 8 + 8192 + 1024);
+    constexpr int by_smem = 233472 / (R * T * 8 + 4096 + 1024);
     constexpr int by_threads = 2048 / T;
     constexpr int m = by_smem < by_threads ? by_smem : by_threads;
     return m < 1 ? 1 : (m > 32 ? 32 : m);
@@ -65,8 +87,11 @@ __global__ void __launch_bounds__(T, b2_min_blocks<R, T>()) split_batch2_kernel(
     __shared__ long long s_sum[T / 32];
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const uint32_t rs = (uint32_t)__cvta_generic_to_shared(smem);
-    uint2 *tabp = reinterpret_cast<uint2 *>(smem + (size_t)R * T * 8);
-    const TabShared2 tab{rs + (uint32_t)R * T * 8};
+    const int cap = (b.max_n + 3) / 4 * 4;
+    int32_t *rowp = reinterpret_cast<int32_t *>(smem + (size_t)R * T * 8), *costp = rowp + cap;
+    uint32_t *flagp = reinterpret_cast<uint32_t *>(costp + cap);
+    const uint32_t row_s = rs + (uint32_t)R * T * 8;
+    const TabShared2 tab{row_s, row_s + 4u * cap, row_s + 8u * cap};
     unsigned long long *tacc = b.acc + BACC_WORDS;
     unsigned long long *status = b.acc + BACC_STATUS;
     int cur = -1;
@@ -81,20 +106,23 @@ __global__ void __launch_bounds__(T, b2_min_blocks<R, T>()) split_batch2_kernel(
         const TourDev td = b.tours[it.x];
         const int t = it.x;
         if (t != cur) {   // block-uniform; the loop-top barrier has retired the previous item
-            for (int k = tid; k < td.n; k += T) {
-                const int ck = td.tab[k].c;
-                uint32_t x = (uint32_t)(td.tab[k].row & kRowMask);
-                // position k + 1 >= 2 with C_k > 0 and C_{k+1} > C_k: no back pops
-                if (k >= 1) {
-                    const int cp = td.tab[k - 1].c;
-                    if (cp > 0 && ck > cp) x |= kTab2NoBack;
+            for (int k = tid; k < (td.n + 3) / 4 * 4; k += T) {
+                const TourStep e = td.tab[min(k, td.n - 1)];
+                rowp[k] = e.row & kRowMask;
+                costp[k] = k < td.n ? e.c : 0;
+            }
+            for (int m = tid; m < (td.n + 7) / 8; m += T) {
+                uint32_t fl = 0;
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    const int k = 8 * m + u;
+                    if (k >= td.n) break;
+                    const int ck = td.tab[k].c, cp = k ? td.tab[k - 1].c : 0;
+                    // position k + 1 >= 2 with C_k > 0 and C_{k+1} > C_k: no back pops
+                    if (cp > 0 && ck > cp) fl |= 1u << u;
+                    if (k < td.n - 1 && ck <= 0) fl |= 1u << (8 + u / kPrefetch2);
                 }
-                if (k % kPrefetch2 == 0) {
-                    bool np = false;
-                    for (int u = k; u < k + kPrefetch2 && u < td.n - 1; ++u) np |= td.tab[u].c <= 0;
-                    if (np) x |= kTab2SharedGeneral;
-                }
-                tabp[k] = make_uint2(x, (uint32_t)ck);
+                flagp[m] = fl;
             }
             __syncthreads();
             cur = t;
@@ -102,12 +130,12 @@ __global__ void __launch_bounds__(T, b2_min_blocks<R, T>()) split_batch2_kernel(
         Walk2Params p{};
         p.demand = td.demand;
         p.S = b.S;
-        p.n = td.n;
-        p.Q = td.Q;
-        p.L = td.L;
+        p.n = (int)uniform((uint32_t)td.n);
+        p.Q = (int)uniform((uint32_t)td.Q);
+        p.L = (int)uniform((uint32_t)td.L);
         p.g0 = td.g0;
-        p.K = td.K;
-        p.pitch = (uint32_t)(td.ld * 2);
+        p.K = uniform(td.K);
+        p.pitch = uniform((uint32_t)(td.ld * 2));
         p.status = status;
         const long long s = (long long)it.y * T + tid;
         bool aside = false;

@@ -202,28 +202,29 @@ template <> struct Dem2<int16_t> { using T = unsigned short; };
 template <> struct Dem2<int32_t> { using T = unsigned int; };
 
 template <typename DT, typename TB>
-__device__ __forceinline__ uint32_t load_dem2(const char *base, const TB &tab, int i, uint32_t pitch,
-                                              int n, unsigned long long *status)
+__device__ __forceinline__ uint32_t load_dem2(const char *base, const TB &tab, const typename TB::Rows &rows, int i, int u,
+                                              uint32_t pitch, int n, unsigned long long *status)
 {
     if (!index_ok(i >= 1 && i <= n && i <= TB::kCap, status)) return 0u;
-    const uint32_t row = tab.row(i);
+    const uint32_t row = tab.row_at(rows, i, u);
     if (!index_ok(row < (uint32_t)n, status)) return 0u;
     return (uint32_t)__ldcs(reinterpret_cast<const typename Dem2<DT>::T *>(base + (unsigned long long)row * pitch));
 }
 
-// Positions i0 .. i0 + kPrefetch2 - 1 (GUARD: the block may reach past n).
+// Positions i0 .. i0 + kPrefetch2 - 1 (GUARD: the block may reach past n), at
+// place `at` of the span whose flags are given.
 template <typename DT, int R, int T, bool LTEST, bool OVF, bool NOWRAP, bool GUARD, bool GENERAL, typename TB>
 __device__ __forceinline__ void walk2_steps(Deque2 &d, const uint32_t (&q)[kPrefetch2], const TB &tab,
-                                            int i0, int n, uint32_t K, uint32_t QK, int L, int Q, uint32_t rs, int &out)
+                                            uint32_t flags, int at, int i0, int n, uint32_t K, uint32_t QK, int L, int Q, uint32_t rs, int &out)
 {
     constexpr bool CLAMP = sizeof(DT) == 4;
+    const typename TB::Costs costs = tab.costs(i0);
 #pragma unroll
     for (int u = 0; u < kPrefetch2; ++u) {
         const int i = i0 + u;
         if (GUARD && i > n) break;
-        const uint2 e = tab.entry(i);
-        const int ci = (int)e.y;
-        const bool noback = (e.x & kTab2NoBack) != 0;
+        const int ci = tab.cost(costs, i, u);
+        const bool noback = tab.noback(flags, i, at + u);
         const uint32_t xi = QK + (uint32_t)i;
         if (!GUARD || i < n)
             dq2_step<R, T, LTEST, OVF, NOWRAP, CLAMP, true, GENERAL>(d, q[u], i, ci, K, xi, L, Q, rs, noback);
@@ -252,26 +253,26 @@ __device__ __forceinline__ bool walk2_exact(const Deque2 &d, int i0, uint32_t K,
 // positions and those of one holding some C_i <= 0 share one copy of the code.
 template <typename DT, int R, int T, bool LCAP, bool NOWRAP, bool GUARD, bool SMOOTH, typename TB>
 __device__ __forceinline__ void walk2_block(Deque2 &d, const uint32_t (&q)[kPrefetch2], const TB &tab,
-                                            int i0, int n, uint32_t K, uint32_t QK, int L, int Q, uint32_t rs,
+                                            uint32_t flags, int at, int i0, int n, uint32_t K, uint32_t QK, int L, int Q, uint32_t rs,
                                             bool exact, int &out)
 {
     constexpr bool kBlockOvf = block_ovf<R>();
-    const bool general = tab.general(i0);
+    const bool general = tab.general(flags, i0, at);
     if (SMOOTH) {
         if (exact || general)
-            walk2_steps<DT, R, T, LCAP, true, NOWRAP, GUARD, true>(d, q, tab, i0, n, K, QK, L, Q, rs, out);
+            walk2_steps<DT, R, T, LCAP, true, NOWRAP, GUARD, true>(d, q, tab, flags, at, i0, n, K, QK, L, Q, rs, out);
         else
-            walk2_steps<DT, R, T, false, !kBlockOvf, NOWRAP, GUARD, false>(d, q, tab, i0, n, K, QK, L, Q, rs, out);
+            walk2_steps<DT, R, T, false, !kBlockOvf, NOWRAP, GUARD, false>(d, q, tab, flags, at, i0, n, K, QK, L, Q, rs, out);
     } else if (exact) {
         if (general)
-            walk2_steps<DT, R, T, LCAP, true, NOWRAP, GUARD, true>(d, q, tab, i0, n, K, QK, L, Q, rs, out);
+            walk2_steps<DT, R, T, LCAP, true, NOWRAP, GUARD, true>(d, q, tab, flags, at, i0, n, K, QK, L, Q, rs, out);
         else
-            walk2_steps<DT, R, T, LCAP, true, NOWRAP, GUARD, false>(d, q, tab, i0, n, K, QK, L, Q, rs, out);
+            walk2_steps<DT, R, T, LCAP, true, NOWRAP, GUARD, false>(d, q, tab, flags, at, i0, n, K, QK, L, Q, rs, out);
     } else {
         if (general)
-            walk2_steps<DT, R, T, false, !kBlockOvf, NOWRAP, GUARD, true>(d, q, tab, i0, n, K, QK, L, Q, rs, out);
+            walk2_steps<DT, R, T, false, !kBlockOvf, NOWRAP, GUARD, true>(d, q, tab, flags, at, i0, n, K, QK, L, Q, rs, out);
         else
-            walk2_steps<DT, R, T, false, !kBlockOvf, NOWRAP, GUARD, false>(d, q, tab, i0, n, K, QK, L, Q, rs, out);
+            walk2_steps<DT, R, T, false, !kBlockOvf, NOWRAP, GUARD, false>(d, q, tab, flags, at, i0, n, K, QK, L, Q, rs, out);
     }
 }
 
@@ -279,9 +280,11 @@ template <typename DT, bool CLAMPI, typename TB>
 __device__ __forceinline__ void prefetch2(const char *base, const TB &tab, int i0, int n, uint32_t pitch,
                                           unsigned long long *status, uint32_t (&q)[kPrefetch2])
 {
+    // (a block past the last has no rows to look up: it reads row n)
+    const typename TB::Rows rows = tab.rows(CLAMPI && i0 > n ? (n - 1) / kPrefetch2 * kPrefetch2 + 1 : i0);
 #pragma unroll
     for (int u = 0; u < kPrefetch2; ++u)
-        q[u] = load_dem2<DT>(base, tab, CLAMPI ? min(i0 + u, n) : i0 + u, pitch, n, status);
+        q[u] = load_dem2<DT>(base, tab, rows, CLAMPI ? min(i0 + u, n) : i0 + u, u, pitch, n, status);
 }
 
 // The walk of one scenario (column s; a thread past S walks column 0 and
@@ -314,20 +317,22 @@ __device__ __forceinline__ int walk2_scenario(const Walk2Params &p, const TB &ta
     constexpr int kSpan = 2 * kPrefetch2;
     for (; i0 + 3 * kPrefetch2 - 1 < n; i0 += 2 * kPrefetch2) {
         prefetch2<DT, false>(base, tab, i0 + kPrefetch2, n, pitch, status, qb);
+        const uint32_t fl = tab.span(i0);
         const bool ex = walk2_exact<R, T, LCAP, NOWRAP, kSpan>(d, i0, K, L);
         const bool ea = SMOOTH ? ex && walk2_exact<R, T, LCAP, NOWRAP, kPrefetch2>(d, i0, K, L) : ex;
-        walk2_block<DT, R, T, LCAP, NOWRAP, false, SMOOTH>(d, qa, tab, i0, n, K, QK, L, Q, rs, ea, out);
+        walk2_block<DT, R, T, LCAP, NOWRAP, false, SMOOTH>(d, qa, tab, fl, 0, i0, n, K, QK, L, Q, rs, ea, out);
         prefetch2<DT, false>(base, tab, i0 + 2 * kPrefetch2, n, pitch, status, qa);
         const bool eb = SMOOTH ? ex && walk2_exact<R, T, LCAP, NOWRAP, kPrefetch2>(d, i0 + kPrefetch2, K, L) : ex;
-        walk2_block<DT, R, T, LCAP, NOWRAP, false, SMOOTH>(d, qb, tab, i0 + kPrefetch2, n, K, QK, L, Q, rs, eb, out);
+        walk2_block<DT, R, T, LCAP, NOWRAP, false, SMOOTH>(d, qb, tab, fl, kPrefetch2, i0 + kPrefetch2, n, K, QK, L, Q, rs, eb, out);
     }
     for (; i0 <= n; i0 += 2 * kPrefetch2) {
         prefetch2<DT, true>(base, tab, i0 + kPrefetch2, n, pitch, status, qb);
+        const uint32_t fl = tab.span(i0);
         const bool ex = walk2_exact<R, T, LCAP, NOWRAP, kSpan>(d, i0, K, L);
-        walk2_block<DT, R, T, LCAP, NOWRAP, true, SMOOTH>(d, qa, tab, i0, n, K, QK, L, Q, rs, ex, out);
+        walk2_block<DT, R, T, LCAP, NOWRAP, true, SMOOTH>(d, qa, tab, fl, 0, i0, n, K, QK, L, Q, rs, ex, out);
         if (i0 + kPrefetch2 > n) break;
         prefetch2<DT, true>(base, tab, i0 + 2 * kPrefetch2, n, pitch, status, qa);
-        walk2_block<DT, R, T, LCAP, NOWRAP, true, SMOOTH>(d, qb, tab, i0 + kPrefetch2, n, K, QK, L, Q, rs, ex, out);
+        walk2_block<DT, R, T, LCAP, NOWRAP, true, SMOOTH>(d, qb, tab, fl, kPrefetch2, i0 + kPrefetch2, n, K, QK, L, Q, rs, ex, out);
     }
     aside = d.frozen || d.qmax > (uint32_t)Q;
     return out;
