@@ -950,7 +950,7 @@ int cvrpsd_batch_create(cvrpsd_ctx *ctx, int32_t T, const cvrpsd_tour_desc *tour
         td.pad = 0;
     }
 
-    DequeShape shape{256, 1, 16};
+    DequeShape shape = batch_default_shape(max_n, (long long)T * S, ctx->sm_count);
     if (ctx->cfg.threads) {
         DequeShape want{ctx->cfg.threads, ctx->cfg.spt, ctx->cfg.ring};
         if (valid_batch_shape(want)) shape = want;

@@ -144,6 +144,28 @@ inline size_t split_batch_smem(int max_n, const DequeShape &shape)
     return (size_t)shape.spt * shape.ring * shape.threads * 8 + (size_t)((max_n + 3) / 4 * 4) * sizeof(TourStep) +
            (size_t)((max_n + 7) / 8) * 4;
 }
+// Launch shape without a request, rings of 16: the smallest blocks that hold all
+// scenarios at once (even shares for the SMs: 64 tours of 100 to 1000 customers
+// under 1000 scenarios 212 us with 64 threads, 250 with 256; 8 tours under 8192
+// 192 against 220), else the one with the most resident threads beside its
+// table (under 8192 scenarios 428 us with 512 threads, 452 with 256, whose
+// tables leave room for five blocks).
+inline DequeShape batch_default_shape(int max_n, long long scenarios, int sm_count)
+{
+    DequeShape best{256, 1, 16};
+    int most = 0;
+    for (int threads : {64, 128, 256, 512}) {
+        const DequeShape s{threads, 1, 16};
+        const int by_smem = (int)(233472 / (split_batch_smem(max_n, s) + 1024)), by_threads = 2048 / threads;
+        const int resident = (by_smem < by_threads ? by_smem : by_threads) * threads;
+        if (scenarios <= (long long)resident * sm_count) return s;
+        if (resident > most || (resident == most && threads <= 256)) {
+            most = resident;
+            best = s;
+        }
+    }
+    return best;
+}
 // Persistent deque kernel over all work items; with configure_only it only
 // sets the kernel's shared-memory limit (call before stream capture) and
 // reports blocks per SM in *blocks_per_sm.

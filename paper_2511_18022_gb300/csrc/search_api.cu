@@ -98,7 +98,7 @@ int cvrpsd_split_eval_tours(cvrpsd_ctx *ctx, const int32_t *d_tours, int32_t T, 
     const uint32_t K = key_scale(n);
     if ((long long)(Q + 1LL) * K + n >= (1LL << 31)) return fail(ctx, CVRPSD_ERR_UNSUPPORTED, "Q too large for n");
 
-    DequeShape shape{256, 1, 16};
+    DequeShape shape = batch_default_shape(n, (long long)T * S, ctx->sm_count);
     if (ctx->cfg.threads && (ctx->cfg.threads == 128 || ctx->cfg.threads == 256) && ctx->cfg.spt == 1 &&
         (ctx->cfg.ring == 16 || ctx->cfg.ring == 32))
         shape = DequeShape{ctx->cfg.threads, 1, ctx->cfg.ring};
