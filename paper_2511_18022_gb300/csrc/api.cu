@@ -410,7 +410,9 @@ int split_eval_impl(cvrpsd_ctx *ctx, const int32_t *tour, int32_t n, const int32
     // thread, no predecessor output, n <= 4032, ...).
     // Host buffers keep the global-table walk: its prefetch runs twice
     // as far ahead, which the host link's latency wants.
-    const bool v2_ok = deque2_supported(p, demand_dtype) && !host_buffers;
+    // Predecessors too, in the library's own shape (n = 200, S = 100,000: 103
+    // against 96 us per call; the other shapes are the first walk's).
+    const bool v2_ok = deque2_supported(p, demand_dtype) && !host_buffers && !(pred && ctx->cfg.threads);
     const bool param_walk = kernel == CVRPSD_KERNEL_DEQUE && v2_ok && ctx->cfg.variant != CVRPSD_WALK_GLOBAL_TABLE &&
                             (ctx->cfg.variant == CVRPSD_WALK_PARAM_TABLE || !ctx->cfg.threads || shape.spt == 1);
 

@@ -77,12 +77,15 @@ struct Walk2Params {
     int32_t *ovf_list;         // device [S]
     unsigned long long *status;   // device word for index-check status bits
     unsigned long long *done;     // see SplitParams
+    int16_t *pred;             // device [n][ldp] or nullptr
+    long long ldp;
 };
 
 // Whether the second walk can run this Split (otherwise the first walk runs):
-// no predecessor output, n <= kTab2Large, demand rows addressable with
+// n <= kTab2Large, demand rows addressable with
 // 32-bit byte offsets, and for int16 demands Q < 32768 (a negative demand
-// read as unsigned then exceeds Q).
+// read as unsigned then exceeds Q). Predecessors: int16 demands, keys that
+// cannot wrap, n <= kTab2Small, and the library's choice of shape.
 bool deque2_supported(const SplitParams &p, int esize);
 
 // Launch it. `tab` is the host copy of the tour table (TourStep rows with

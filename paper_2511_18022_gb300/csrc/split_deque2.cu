@@ -17,10 +17,10 @@ cudaError_t dispatch_deque2_i32(const Walk2Params &p, const void *tab, bool lcap
 // A launch's parameters may take at most 32764 bytes.
 static_assert(sizeof(TabParam<kTab2Large>) + sizeof(Walk2Params) <= 32764, "tour table too large for the parameters");
 
-template <typename DT, int R, int T, bool LCAP, bool NOWRAP, int CAP, bool SMOOTH = false>
+template <typename DT, int R, int T, bool LCAP, bool NOWRAP, int CAP, bool SMOOTH = false, bool PRED = false>
 static cudaError_t launch2(const Walk2Params &p, const void *tab, long long grid, cudaStream_t st)
 {
-    split_deque2_kernel<DT, R, T, LCAP, NOWRAP, CAP, SMOOTH>
+    split_deque2_kernel<DT, R, T, LCAP, NOWRAP, CAP, SMOOTH, PRED>
         <<<(unsigned)grid, T, 0, st>>>(p, *static_cast<const TabParam<CAP> *>(tab));
     return cudaGetLastError();
 }
@@ -35,6 +35,11 @@ template <typename DT, bool LCAP, bool NOWRAP, int CAP>
 static cudaError_t dispatch_wide(const Walk2Params &p, const void *tab, const DequeShape &s, bool smooth,
                                  long long grid, cudaStream_t st)
 {
+    if (p.pred && s.threads == 64 && s.ring == 32)
+        return launch2<DT, 32, 64, LCAP, NOWRAP, CAP, false, true>(p, tab, grid, st);
+    if (p.pred && s.threads == 128 && s.ring == 16)
+        return launch2<DT, 16, 128, LCAP, NOWRAP, CAP, false, true>(p, tab, grid, st);
+    if (p.pred) return cudaErrorInvalidValue;
     if (smooth && s.threads == 128 && s.ring == 16)
         return launch2<DT, 16, 128, LCAP, NOWRAP, CAP, true>(p, tab, grid, st);
     CVRPSD_D2_SHAPE(64, 8) CVRPSD_D2_SHAPE(64, 16) CVRPSD_D2_SHAPE(128, 8) CVRPSD_D2_SHAPE(128, 16)
@@ -108,7 +113,8 @@ DequeShape compiled_shape(const SplitParams &p, int esize, const DequeShape &s, 
 
 bool deque2_supported(const SplitParams &p, int esize)
 {
-    if (p.pred || p.n > kTab2Large || p.n < 1) return false;
+    if (p.n > kTab2Large || p.n < 1) return false;
+    if (p.pred && (esize != 2 || p.n > kTab2Small || !keys_fit(p, esize))) return false;
     if ((unsigned long long)p.ld * esize > 0xFFFFFFFFull) return false;   // 32-bit row pitch
     if ((unsigned long long)(p.n - 1) * (unsigned long long)p.ld * esize + (unsigned long long)p.S * esize >
         0xFFFFFFFFull)
@@ -157,6 +163,8 @@ cudaError_t launch_split_deque2(const SplitParams &p, const TourStep *tab, int e
     w.ovf_list = p.ovf_list;
     w.status = p.acc + ACC_STATUS;
     w.done = p.done;
+    w.pred = p.pred;
+    w.ldp = p.ldp;
     w.pitch = (uint32_t)pitch;
     const long long tiles = (p.S + s.threads - 1) / s.threads;
     const long long grid = rounds > 0 ? (tiles + rounds - 1) / rounds : tiles;

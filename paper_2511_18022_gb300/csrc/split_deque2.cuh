@@ -98,10 +98,13 @@ template <int R, bool NOWRAP> __host__ __device__ constexpr bool fold_frozen() {
 // One position. PUSH: candidate i enters (positions 1..n-1); the last
 // position only reads the window minimum. GENERAL: some C_i <= 0 in this
 // block, so back pops may empty the deque (see split_deque.cuh). LTEST: test
-// the front's route-length limit; OVF: test the push for ring overflow.
-template <int R, int T, bool LTEST, bool OVF, bool NOWRAP, bool CLAMP, bool PUSH, bool GENERAL>
+// the front's route-length limit; OVF: test the push for ring overflow. PRED:
+// *argmin gets the smallest optimal predecessor, the front's position: back
+// entries then go only when strictly larger, so among equal minima the oldest
+// stays in front (split_deque.cuh).
+template <int R, int T, bool LTEST, bool OVF, bool NOWRAP, bool CLAMP, bool PUSH, bool GENERAL, bool PRED>
 __device__ __forceinline__ int dq2_step(Deque2 &d, uint32_t q, int i, int ci, uint32_t K, uint32_t xi, int L, int Q,
-                                        uint32_t rs, bool noback)
+                                        uint32_t rs, bool noback, int *argmin)
 {
     constexpr uint32_t kStride = T * 8u;
     constexpr uint32_t kMask = R * T * 8u - 1u;
@@ -135,6 +138,7 @@ __device__ __forceinline__ int dq2_step(Deque2 &d, uint32_t q, int i, int ci, ui
         d.fx = e.y;
     }
     const int gi = d.fg + ci;
+    if (PRED) *argmin = (int)((uint32_t)d.fx & (K - 1u));
     if (!PUSH) return gi;
     const int x = (int)(d.pk + xi);       // K * (P(i) + Q) + i
     constexpr bool kFold = fold_frozen<R, NOWRAP>();
@@ -143,7 +147,7 @@ __device__ __forceinline__ int dq2_step(Deque2 &d, uint32_t q, int i, int ci, ui
     // front's, so the back walk stops there as in any other block.
     if (!GENERAL || ci > 0) {
         if (!noback) {
-            bool pb = (d.bg >= gi) & (kFold || !d.frozen);
+            bool pb = (PRED ? d.bg > gi : d.bg >= gi) & (kFold || !d.frozen);
             // Where the back can pop at all (C_i <= C_{i-1} or C_{i-1} <= 0),
             // nearly every warp pops at least once (lanes whose front did
             // not move pop the back whenever C_i <= C_{i-1}): the first step
@@ -153,14 +157,14 @@ __device__ __forceinline__ int dq2_step(Deque2 &d, uint32_t q, int i, int ci, ui
                 const int below = lds1(rs + bp);
                 d.b = pb ? bp : d.b;
                 d.bg = pb ? below : d.bg;
-                pb = pb & (below >= gi);
+                pb = pb & (PRED ? below > gi : below >= gi);
             }
             while (__any_sync(0xffffffffu, pb)) {
                 const uint32_t bp = (d.b - kStride) & kMask;
                 const int below = lds1(rs + bp);
                 d.b = pb ? bp : d.b;
                 d.bg = pb ? below : d.bg;
-                pb = pb & (below >= gi);
+                pb = pb & (PRED ? below > gi : below >= gi);
             }
         }
         d.b = (d.b + kStride) & kMask;
@@ -170,7 +174,7 @@ __device__ __forceinline__ int dq2_step(Deque2 &d, uint32_t q, int i, int ci, ui
             if (kFold && ovf) d.fg = gi, d.fx = x;
         }
     } else {
-        bool pb = (d.bg >= gi) & (kFold || !d.frozen);
+        bool pb = (PRED ? d.bg > gi : d.bg >= gi) & (kFold || !d.frozen);
         bool empty = false;
         while (__any_sync(0xffffffffu, pb)) {
             const bool emp = d.b == d.h;
@@ -179,7 +183,7 @@ __device__ __forceinline__ int dq2_step(Deque2 &d, uint32_t q, int i, int ci, ui
             empty |= pb & emp;
             d.b = pb ? bp : d.b;
             d.bg = pb ? below : d.bg;
-            pb = pb & !emp & (below >= gi);
+            pb = pb & !emp & (PRED ? below > gi : below >= gi);
         }
         d.b = (d.b + kStride) & kMask;
         if (empty) {
@@ -213,9 +217,10 @@ __device__ __forceinline__ uint32_t load_dem2(const char *base, const TB &tab, c
 
 // Positions i0 .. i0 + kPrefetch2 - 1 (GUARD: the block may reach past n), at
 // place `at` of the span whose flags are given.
-template <typename DT, int R, int T, bool LTEST, bool OVF, bool NOWRAP, bool GUARD, bool GENERAL, typename TB>
+template <typename DT, int R, int T, bool LTEST, bool OVF, bool NOWRAP, bool GUARD, bool GENERAL, bool PRED, typename TB>
 __device__ __forceinline__ void walk2_steps(Deque2 &d, const uint32_t (&q)[kPrefetch2], const TB &tab,
-                                            uint32_t flags, int at, int i0, int n, uint32_t K, uint32_t QK, int L, int Q, uint32_t rs, int &out)
+                                            uint32_t flags, int at, int i0, int n, uint32_t K, uint32_t QK, int L, int Q, uint32_t rs, int &out,
+                                            int16_t *pred, long long ldp)
 {
     constexpr bool CLAMP = sizeof(DT) == 4;
     const typename TB::Costs costs = tab.costs(i0);
@@ -226,10 +231,13 @@ __device__ __forceinline__ void walk2_steps(Deque2 &d, const uint32_t (&q)[kPref
         const int ci = tab.cost(costs, i, u);
         const bool noback = tab.noback(flags, i, at + u);
         const uint32_t xi = QK + (uint32_t)i;
+        int p = 0;
         if (!GUARD || i < n)
-            dq2_step<R, T, LTEST, OVF, NOWRAP, CLAMP, true, GENERAL>(d, q[u], i, ci, K, xi, L, Q, rs, noback);
+            dq2_step<R, T, LTEST, OVF, NOWRAP, CLAMP, true, GENERAL, PRED>(d, q[u], i, ci, K, xi, L, Q, rs, noback, &p);
         else
-            out = dq2_step<R, T, LTEST, OVF, NOWRAP, CLAMP, false, GENERAL>(d, q[u], i, ci, K, xi, L, Q, rs, noback);
+            out = dq2_step<R, T, LTEST, OVF, NOWRAP, CLAMP, false, GENERAL, PRED>(d, q[u], i, ci, K, xi, L, Q, rs, noback,
+                                                                                 &p);
+        if (PRED && pred) __stcs(pred + (long long)(i - 1) * ldp, (int16_t)p);
     }
 }
 
@@ -251,28 +259,29 @@ __device__ __forceinline__ bool walk2_exact(const Deque2 &d, int i0, uint32_t K,
 
 // SMOOTH (see smooth_table): the tests of a block that needs the exact
 // positions and those of one holding some C_i <= 0 share one copy of the code.
-template <typename DT, int R, int T, bool LCAP, bool NOWRAP, bool GUARD, bool SMOOTH, typename TB>
+template <typename DT, int R, int T, bool LCAP, bool NOWRAP, bool GUARD, bool SMOOTH, bool PRED, typename TB>
 __device__ __forceinline__ void walk2_block(Deque2 &d, const uint32_t (&q)[kPrefetch2], const TB &tab,
                                             uint32_t flags, int at, int i0, int n, uint32_t K, uint32_t QK, int L, int Q, uint32_t rs,
-                                            bool exact, int &out)
+                                            bool exact, int &out,
+                                            int16_t *pred, long long ldp)
 {
     constexpr bool kBlockOvf = block_ovf<R>();
     const bool general = tab.general(flags, i0, at);
     if (SMOOTH) {
         if (exact || general)
-            walk2_steps<DT, R, T, LCAP, true, NOWRAP, GUARD, true>(d, q, tab, flags, at, i0, n, K, QK, L, Q, rs, out);
+            walk2_steps<DT, R, T, LCAP, true, NOWRAP, GUARD, true, PRED>(d, q, tab, flags, at, i0, n, K, QK, L, Q, rs, out, pred, ldp);
         else
-            walk2_steps<DT, R, T, false, !kBlockOvf, NOWRAP, GUARD, false>(d, q, tab, flags, at, i0, n, K, QK, L, Q, rs, out);
+            walk2_steps<DT, R, T, false, !kBlockOvf, NOWRAP, GUARD, false, PRED>(d, q, tab, flags, at, i0, n, K, QK, L, Q, rs, out, pred, ldp);
     } else if (exact) {
         if (general)
-            walk2_steps<DT, R, T, LCAP, true, NOWRAP, GUARD, true>(d, q, tab, flags, at, i0, n, K, QK, L, Q, rs, out);
+            walk2_steps<DT, R, T, LCAP, true, NOWRAP, GUARD, true, PRED>(d, q, tab, flags, at, i0, n, K, QK, L, Q, rs, out, pred, ldp);
         else
-            walk2_steps<DT, R, T, LCAP, true, NOWRAP, GUARD, false>(d, q, tab, flags, at, i0, n, K, QK, L, Q, rs, out);
+            walk2_steps<DT, R, T, LCAP, true, NOWRAP, GUARD, false, PRED>(d, q, tab, flags, at, i0, n, K, QK, L, Q, rs, out, pred, ldp);
     } else {
         if (general)
-            walk2_steps<DT, R, T, false, !kBlockOvf, NOWRAP, GUARD, true>(d, q, tab, flags, at, i0, n, K, QK, L, Q, rs, out);
+            walk2_steps<DT, R, T, false, !kBlockOvf, NOWRAP, GUARD, true, PRED>(d, q, tab, flags, at, i0, n, K, QK, L, Q, rs, out, pred, ldp);
         else
-            walk2_steps<DT, R, T, false, !kBlockOvf, NOWRAP, GUARD, false>(d, q, tab, flags, at, i0, n, K, QK, L, Q, rs, out);
+            walk2_steps<DT, R, T, false, !kBlockOvf, NOWRAP, GUARD, false, PRED>(d, q, tab, flags, at, i0, n, K, QK, L, Q, rs, out, pred, ldp);
     }
 }
 
@@ -290,7 +299,7 @@ __device__ __forceinline__ void prefetch2(const char *base, const TB &tab, int i
 // The walk of one scenario (column s; a thread past S walks column 0 and
 // reports nothing: every lane takes part in the votes). Returns f(n) or
 // sets *aside.
-template <typename DT, int R, int T, bool LCAP, bool NOWRAP, bool SMOOTH, typename TB>
+template <typename DT, int R, int T, bool LCAP, bool NOWRAP, bool SMOOTH, bool PRED = false, typename TB>
 __device__ __forceinline__ int walk2_scenario(const Walk2Params &p, const TB &tab, long long s,
                                               uint32_t rs, uint32_t slot0, bool &aside)
 {
@@ -310,6 +319,9 @@ __device__ __forceinline__ int walk2_scenario(const Walk2Params &p, const TB &ta
     uint32_t qa[kPrefetch2], qb[kPrefetch2];
     const uint32_t pitch = p.pitch;
     unsigned long long *status = p.status;
+    // A thread without a scenario writes no predecessors.
+    int16_t *pred = PRED && s < p.S ? p.pred + s : nullptr;
+    const long long ldp = PRED ? p.ldp : 0;
     prefetch2<DT, true>(base, tab, 1, n, pitch, status, qa);
     int i0 = 1;
     // One exactness vote covers both prefetch blocks of an iteration; on a
@@ -320,19 +332,19 @@ __device__ __forceinline__ int walk2_scenario(const Walk2Params &p, const TB &ta
         const uint32_t fl = tab.span(i0);
         const bool ex = walk2_exact<R, T, LCAP, NOWRAP, kSpan>(d, i0, K, L);
         const bool ea = SMOOTH ? ex && walk2_exact<R, T, LCAP, NOWRAP, kPrefetch2>(d, i0, K, L) : ex;
-        walk2_block<DT, R, T, LCAP, NOWRAP, false, SMOOTH>(d, qa, tab, fl, 0, i0, n, K, QK, L, Q, rs, ea, out);
+        walk2_block<DT, R, T, LCAP, NOWRAP, false, SMOOTH, PRED>(d, qa, tab, fl, 0, i0, n, K, QK, L, Q, rs, ea, out, pred, ldp);
         prefetch2<DT, false>(base, tab, i0 + 2 * kPrefetch2, n, pitch, status, qa);
         const bool eb = SMOOTH ? ex && walk2_exact<R, T, LCAP, NOWRAP, kPrefetch2>(d, i0 + kPrefetch2, K, L) : ex;
-        walk2_block<DT, R, T, LCAP, NOWRAP, false, SMOOTH>(d, qb, tab, fl, kPrefetch2, i0 + kPrefetch2, n, K, QK, L, Q, rs, eb, out);
+        walk2_block<DT, R, T, LCAP, NOWRAP, false, SMOOTH, PRED>(d, qb, tab, fl, kPrefetch2, i0 + kPrefetch2, n, K, QK, L, Q, rs, eb, out, pred, ldp);
     }
     for (; i0 <= n; i0 += 2 * kPrefetch2) {
         prefetch2<DT, true>(base, tab, i0 + kPrefetch2, n, pitch, status, qb);
         const uint32_t fl = tab.span(i0);
         const bool ex = walk2_exact<R, T, LCAP, NOWRAP, kSpan>(d, i0, K, L);
-        walk2_block<DT, R, T, LCAP, NOWRAP, true, SMOOTH>(d, qa, tab, fl, 0, i0, n, K, QK, L, Q, rs, ex, out);
+        walk2_block<DT, R, T, LCAP, NOWRAP, true, SMOOTH, PRED>(d, qa, tab, fl, 0, i0, n, K, QK, L, Q, rs, ex, out, pred, ldp);
         if (i0 + kPrefetch2 > n) break;
         prefetch2<DT, true>(base, tab, i0 + 2 * kPrefetch2, n, pitch, status, qa);
-        walk2_block<DT, R, T, LCAP, NOWRAP, true, SMOOTH>(d, qb, tab, fl, kPrefetch2, i0 + kPrefetch2, n, K, QK, L, Q, rs, ex, out);
+        walk2_block<DT, R, T, LCAP, NOWRAP, true, SMOOTH, PRED>(d, qb, tab, fl, kPrefetch2, i0 + kPrefetch2, n, K, QK, L, Q, rs, ex, out, pred, ldp);
     }
     aside = d.frozen || d.qmax > (uint32_t)Q;
     return out;
@@ -349,7 +361,7 @@ constexpr int kD2ThreadsPerSM = 2048;
 template <int R, int T>
 constexpr int d2_min_blocks() { return kD2ThreadsPerSM / T; }
 
-template <typename DT, int R, int T, bool LCAP, bool NOWRAP, int CAP, bool SMOOTH>
+template <typename DT, int R, int T, bool LCAP, bool NOWRAP, int CAP, bool SMOOTH, bool PRED>
 __global__ void __launch_bounds__(T, d2_min_blocks<R, T>()) split_deque2_kernel(const Walk2Params p, const __grid_constant__ TabParam<CAP> tab)
 {
     // Rings [R][T] of (g, key) slots: thread t's slot k is at byte
@@ -365,7 +377,7 @@ __global__ void __launch_bounds__(T, d2_min_blocks<R, T>()) split_deque2_kernel(
     for (long long sb = (long long)blockIdx.x * T; sb < p.S; sb += p.stride) {
         const long long s = sb + tid;
         bool aside = false;
-        const int c = walk2_scenario<DT, R, T, LCAP, NOWRAP, SMOOTH>(p, tab, s, rs, slot0, aside);
+        const int c = walk2_scenario<DT, R, T, LCAP, NOWRAP, SMOOTH, PRED>(p, tab, s, rs, slot0, aside);
         if (s < p.S) {
             if (aside) {
                 const unsigned long long idx = atomicAdd(p.acc + ACC_OVERFLOW, 1ull);
