@@ -530,6 +530,25 @@ int split_eval_impl(cvrpsd_ctx *ctx, const int32_t *tour, int32_t n, const int32
                 st.launches = 1;
                 goto launched;
             }
+            // Rows of host memory that straddle its 64-byte lines, from 24,576
+            // scenarios: staged (n = 200, S = 24,577: 115 us direct, 108 staged;
+            // n = 1000: 380 and 327). Below that too few blocks are at work and the
+            // walk's latency counts (n = 1000, S = 8,001: 300 and 305; 32 bits,
+            // S = 12,301: 370 and 412), and aligned rows gain nothing in 32 bits
+            // (S = 100,000: 437 and 440) and little in 16 (260 and 258).
+            if (host_buffers && !pred && !ctx->cfg.threads && S >= 24 * 1024 &&
+                ((uintptr_t)p.demand & 15) == 0 && (((uintptr_t)p.demand | (uintptr_t)(ld * demand_dtype)) & 63) != 0) {
+                if (timed) CK(cudaEventRecord(ctx->ev_t[0], stream), "cudaEventRecord");
+                CK(launch_split_host(p, demand_dtype, stream), "split_host launch");
+                if (timed) CK(cudaEventRecord(ctx->ev_t[1], stream), "cudaEventRecord");
+                st.kernel = CVRPSD_KERNEL_DEQUE;
+                st.threads = 1024 / demand_dtype;
+                st.spt = 1;
+                st.ring = 16;
+                st.variant = CVRPSD_WALK_GLOBAL_TABLE;
+                st.launches = 1;
+                goto launched;
+            }
             if (host_buffers && !ctx->cfg.threads) shape = DequeShape{128, 1, 16};
             if (shape.ring == 8 && (shape.spt != 1 || shape.threads == 64 || pred))
                 shape.ring = 16;   // rings of 8 exist for one scenario per thread, 128 or 256 threads

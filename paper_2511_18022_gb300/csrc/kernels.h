@@ -83,6 +83,14 @@ cudaError_t launch_split_deque_i16_nocap(const SplitParams &p, const DequeShape 
 cudaError_t launch_split_deque_i32_cap(const SplitParams &p, const DequeShape &s, cudaStream_t st);
 cudaError_t launch_split_deque_i32_nocap(const SplitParams &p, const DequeShape &s, cudaStream_t st);
 
+// The same walk for scenarios in page-locked host memory (device addresses of
+// it in p): 1 KB windows of the rows staged through shared memory, rings of 16.
+cudaError_t launch_split_host(const SplitParams &p, int esize, cudaStream_t stream);
+cudaError_t launch_split_host_i16_cap(const SplitParams &p, cudaStream_t st);
+cudaError_t launch_split_host_i16_nocap(const SplitParams &p, cudaStream_t st);
+cudaError_t launch_split_host_i32_cap(const SplitParams &p, cudaStream_t st);
+cudaError_t launch_split_host_i32_nocap(const SplitParams &p, cudaStream_t st);
+
 // Dynamic shared memory of the deque kernel: its rings ([spt][ring][threads] int2).
 inline size_t split_deque_smem(const SplitParams &p, const DequeShape &shape)
 {

@@ -39,18 +39,33 @@ static cudaError_t dispatch_shape(const SplitParams &p, const DequeShape &s, cud
     return cudaErrorInvalidValue;
 }
 
+template <typename DT, bool LCAP>
+static cudaError_t launch_host(const SplitParams &p, cudaStream_t stream)
+{
+    auto kern = split_host_kernel<DT, 16, LCAP>;
+    const size_t smem = split_host_smem<DT, 16>();
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    kern<<<(unsigned)((p.S + kHostThreads<DT> - 1) / kHostThreads<DT>), kHostThreads<DT>, smem, stream>>>(p);
+    return cudaGetLastError();
+}
+
 #if CVRPSD_DEQUE_PART == 0
 cudaError_t launch_split_deque_i16_cap(const SplitParams &p, const DequeShape &s, cudaStream_t st)
 { return dispatch_shape<int16_t, true>(p, s, st); }
+cudaError_t launch_split_host_i16_cap(const SplitParams &p, cudaStream_t st) { return launch_host<int16_t, true>(p, st); }
 #elif CVRPSD_DEQUE_PART == 1
 cudaError_t launch_split_deque_i16_nocap(const SplitParams &p, const DequeShape &s, cudaStream_t st)
 { return dispatch_shape<int16_t, false>(p, s, st); }
+cudaError_t launch_split_host_i16_nocap(const SplitParams &p, cudaStream_t st) { return launch_host<int16_t, false>(p, st); }
 #elif CVRPSD_DEQUE_PART == 2
 cudaError_t launch_split_deque_i32_cap(const SplitParams &p, const DequeShape &s, cudaStream_t st)
 { return dispatch_shape<int32_t, true>(p, s, st); }
+cudaError_t launch_split_host_i32_cap(const SplitParams &p, cudaStream_t st) { return launch_host<int32_t, true>(p, st); }
 #elif CVRPSD_DEQUE_PART == 3
 cudaError_t launch_split_deque_i32_nocap(const SplitParams &p, const DequeShape &s, cudaStream_t st)
 { return dispatch_shape<int32_t, false>(p, s, st); }
+cudaError_t launch_split_host_i32_nocap(const SplitParams &p, cudaStream_t st) { return launch_host<int32_t, false>(p, st); }
 #endif
 
 }  // namespace cvrpsd

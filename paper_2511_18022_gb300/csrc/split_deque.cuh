@@ -431,4 +431,102 @@ __global__ void __launch_bounds__(T, d1_min_blocks<T>()) split_deque_kernel(Spli
     block_finish(p.acc, p.done);
 }
 
+// ---- scenarios in page-locked host memory
+//
+// The same walk with the demands staged through shared memory. What bounds it
+// is the host link, which carries 64-byte lines: where a row does not start on
+// one, the 64 bytes that a warp reads from it straddle two, and every line
+// crosses twice (a call with n = 200 takes 260 us at S = 100,000, whose rows are
+// aligned, and 322 at S = 99,999). So a block copies whole lines of its 1 KB
+// window of each row (16 bytes per cp.async, three groups of eight tour
+// positions in flight), and only the window's two ends cross twice: 267 us at
+// S = 99,999; in 32 bits 518 -> 468.
+constexpr int kHostStages = 4;                 // groups of kPrefetch positions
+template <typename DT> constexpr int kHostThreads = 1024 / (int)sizeof(DT);
+constexpr int kHostRow = 1024 + 128;           // a row's window and the rest of its first and last line
+constexpr int kHostChunks = kHostRow / 16;
+
+template <typename DT, int R>
+inline size_t split_host_smem() { return (size_t)R * kHostThreads<DT> * 8 + (size_t)kHostStages * kPrefetch * kHostRow; }
+
+template <typename DT, int R, bool LCAP>
+__global__ void __launch_bounds__(kHostThreads<DT>) split_host_kernel(SplitParams p)
+{
+    constexpr int T = kHostThreads<DT>;
+    extern __shared__ __align__(128) unsigned char smem[];   // rings, then the stages
+    unsigned char *stages = smem + (size_t)R * T * 8;
+    const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(smem), stage_s = sbase + R * T * 8;
+    const int n = p.n, Q = p.Q, L = p.L, tid = threadIdx.x;
+    const uint32_t K = p.K, QK = (uint32_t)Q * K;
+    const TabGlobal tab{reinterpret_cast<const int *>(p.tab)};
+    const long long s0 = (long long)blockIdx.x * T, s = s0 + tid;
+    const bool valid = s < p.S;
+    const uintptr_t base = (uintptr_t)p.demand + (uintptr_t)s0 * sizeof(DT);
+    const uintptr_t lo = (uintptr_t)p.demand;                // a multiple of 16
+    const uintptr_t hi = lo + ((uintptr_t)(n - 1) * p.ld + p.S) * sizeof(DT);
+    const uintptr_t ldb = (uintptr_t)p.ld * sizeof(DT);
+    const uintptr_t bytes = (uintptr_t)(p.S - s0 < T ? p.S - s0 : T) * sizeof(DT);   // of a row's window
+    const int groups = (n + kPrefetch - 1) / kPrefetch;
+    unsigned long long *status = p.acc + ACC_STATUS;
+    auto row_of = [&](int i) {
+        const int row = tab.row(i) & kRowMask;
+        return (uintptr_t)(index_ok(row < n, status) ? row : 0) * ldb + base;
+    };
+    auto copy = [&](int g) {                                 // group g's windows into stage g mod 4
+        if (g < groups) {
+            for (int c = tid; c < kPrefetch * kHostChunks; c += T) {
+                const int u = c / kHostChunks, k = c % kHostChunks;
+                const uintptr_t a = row_of(min(g * kPrefetch + u + 1, n)), src = (a & ~(uintptr_t)63) + 16 * (uintptr_t)k;
+                if (src >= lo && src < a + bytes) {          // within the matrix; its last bytes by size
+                    const uint32_t dst = stage_s + (uint32_t)(((g % kHostStages) * kPrefetch + u) * kHostRow + 16 * k);
+                    const uint32_t size = hi - src < 16 ? (uint32_t)(hi - src) : 16u;
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(size) : "memory");
+                }
+            }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    Deque d[1];
+    const uint32_t ring[1] = {sbase};
+    int out[1] = {0};
+    d[0].hoff = d[0].boff = (uint32_t)tid * 8u;
+    d[0].fg = d[0].bg = p.g0;
+    d[0].fx = QK;
+    d[0].fe = L + 1;
+    d[0].pk = 0;
+    d[0].qmax = 0;
+    d[0].ovf = false;
+    sts2(sbase + d[0].hoff, p.g0, (int)QK);
+#pragma unroll
+    for (int g = 0; g < kHostStages - 1; ++g) copy(g);
+    for (int g = 0; g < groups; ++g) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(kHostStages - 2) : "memory");
+        __syncthreads();                                     // group g is there; group g - 1 has been read by all
+        int q[kPrefetch][1];
+        const int i0 = g * kPrefetch + 1;
+#pragma unroll
+        for (int u = 0; u < kPrefetch; ++u) {
+            const unsigned char *w = stages + ((g % kHostStages) * kPrefetch + u) * kHostRow + (row_of(min(i0 + u, n)) & 63);
+            q[u][0] = valid ? (int)reinterpret_cast<const DT *>(w)[tid] : 0;
+        }
+        copy(g + kHostStages - 1);
+        if (i0 + kPrefetch - 1 < n)
+            walk_block<DT, 1, R, T, LCAP, false, false>(d, ring, q, tab, i0, n, K, QK, L, Q, out, nullptr, 0);
+        else
+            walk_block<DT, 1, R, T, LCAP, true, false>(d, ring, q, tab, i0, n, K, QK, L, Q, out, nullptr, 0);
+    }
+    long long sum = 0;
+    if (valid) {
+        if (d[0].ovf || d[0].qmax > (uint32_t)Q) {
+            const unsigned long long idx = atomicAdd(p.acc + ACC_OVERFLOW, 1ull);
+            if (index_ok(idx < (unsigned long long)p.S, status)) p.ovf_list[idx] = (int32_t)s;
+        } else {
+            sum = out[0];
+            if (p.out_cost) p.out_cost[s] = out[0];
+        }
+    }
+    block_accumulate(sum, 0u, 0u, p.acc);
+    block_finish(p.acc, p.done);
+}
+
 }  // namespace cvrpsd

@@ -406,4 +406,11 @@ cudaError_t launch_split_deque(const SplitParams &p, int esize, const DequeShape
                : launch_split_deque_i32_nocap(p, shape, stream);
 }
 
+cudaError_t launch_split_host(const SplitParams &p, int esize, cudaStream_t stream)
+{
+    const bool cap = p.L < p.n;
+    if (esize == 2) return cap ? launch_split_host_i16_cap(p, stream) : launch_split_host_i16_nocap(p, stream);
+    return cap ? launch_split_host_i32_cap(p, stream) : launch_split_host_i32_nocap(p, stream);
+}
+
 }  // namespace cvrpsd
