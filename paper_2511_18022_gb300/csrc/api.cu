@@ -389,8 +389,10 @@ int split_eval_impl(cvrpsd_ctx *ctx, const int32_t *tour, int32_t n, const int32
     //   1000  4096    152    80
     //   1000  8192    161   139
     //   4000    37    581   121     75
-    // so one warp per scenario up to 8192 scenarios, and the
-    // sequence-parallel kernel for a few dozen on a long tour. Below 64
+    // (whole calls, S = 37: n = 1000 71 warp, 76 seqpar; 1200 78, 79.5; 1400
+    // 86.5, 84.5; S = 1: 1100 74, 76; 1200 78.5, 77.2), so one warp per
+    // scenario up to 8192 scenarios, and the sequence-parallel kernel for a few
+    // dozen on a long tour. Below 64
     // positions the deque kernel stays (15 us against 9 at n = 50: its walk
     // is short, and callers read the kernel back). Scenarios in host memory
     // keep the kernels whose warps read whole sectors of a row.
@@ -400,7 +402,7 @@ int split_eval_impl(cvrpsd_ctx *ctx, const int32_t *tour, int32_t n, const int32
         if (!pred && host_buffers) {
             if (S <= 256 && n >= 128) kernel = CVRPSD_KERNEL_SEQPAR;
         } else if (!pred && n >= 64 && S <= 8192) {
-            kernel = S <= 48 && n >= 900 ? CVRPSD_KERNEL_SEQPAR : CVRPSD_KERNEL_WARP;
+            kernel = S <= 48 && n >= 1200 ? CVRPSD_KERNEL_SEQPAR : CVRPSD_KERNEL_WARP;
         }
     }
     DequeShape shape{128, 1, 16};
@@ -410,8 +412,8 @@ int split_eval_impl(cvrpsd_ctx *ctx, const int32_t *tour, int32_t n, const int32
     // thread, no predecessor output, n <= 4032, ...).
     // Host buffers keep the global-table walk: its prefetch runs twice
     // as far ahead, which the host link's latency wants.
-    // Predecessors too, in the library's own shape (n = 200, S = 100,000: 103
-    // against 96 us per call; the other shapes are the first walk's).
+    // Predecessors too, in the library's own shape (n = 200, S = 100,000: 100.4
+    // against 92.3 us per call; the other shapes are the first walk's).
     const bool v2_ok = deque2_supported(p, demand_dtype) && !host_buffers && !(pred && ctx->cfg.threads);
     const bool param_walk = kernel == CVRPSD_KERNEL_DEQUE && v2_ok && ctx->cfg.variant != CVRPSD_WALK_GLOBAL_TABLE &&
                             (ctx->cfg.variant == CVRPSD_WALK_PARAM_TABLE || !ctx->cfg.threads || shape.spt == 1);
