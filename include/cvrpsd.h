@@ -67,7 +67,7 @@ extern "C" {
 
 /* Kernel choice for the Split (see cvrpsd_config). AUTO takes, for device
  * buffers and no predecessors, WARP for S <= 8192 scenarios on tours of
- * n >= 64 (SEQPAR for S <= 48 where n >= 1200), for host buffers SEQPAR for
+ * n >= 64 (SEQPAR for S <= 48 where n >= 3000), for host buffers SEQPAR for
  * S <= 256 where n >= 128, and DEQUE otherwise (lowest latency each). */
 #define CVRPSD_KERNEL_AUTO   0
 #define CVRPSD_KERNEL_DEQUE  1   /* one thread per scenario, monotone deque */

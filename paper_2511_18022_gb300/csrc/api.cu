@@ -389,10 +389,10 @@ int split_eval_impl(cvrpsd_ctx *ctx, const int32_t *tour, int32_t n, const int32
     //   1000  4096    152    80
     //   1000  8192    161   139
     //   4000    37    581   121     75
-    // (whole calls, S = 37: n = 1000 71 warp, 76 seqpar; 1200 78, 79.5; 1400
-    // 86.5, 84.5; S = 1: 1100 74, 76; 1200 78.5, 77.2), so one warp per
-    // scenario up to 8192 scenarios, and the sequence-parallel kernel for a few
-    // dozen on a long tour. Below 64
+    // (whole calls by the walk in pairs and by seqpar: n = 2000, S = 1 88, 90,
+    // S = 37 91, 101; 3000, S = 1 121, 115, S = 37 123, 128; 4000, S = 37 150,
+    // 140), so one warp per scenario up to 8192 scenarios, and the
+    // sequence-parallel kernel for a few dozen on a very long tour. Below 64
     // positions the deque kernel stays (15 us against 9 at n = 50: its walk
     // is short, and callers read the kernel back). Scenarios in host memory
     // keep the kernels whose warps read whole sectors of a row.
@@ -402,7 +402,7 @@ int split_eval_impl(cvrpsd_ctx *ctx, const int32_t *tour, int32_t n, const int32
         if (!pred && host_buffers) {
             if (S <= 256 && n >= 128) kernel = CVRPSD_KERNEL_SEQPAR;
         } else if (!pred && n >= 64 && S <= 8192) {
-            kernel = S <= 48 && n >= 1200 ? CVRPSD_KERNEL_SEQPAR : CVRPSD_KERNEL_WARP;
+            kernel = S <= 48 && n >= 3000 ? CVRPSD_KERNEL_SEQPAR : CVRPSD_KERNEL_WARP;
         }
     }
     DequeShape shape{128, 1, 16};
@@ -500,7 +500,7 @@ int split_eval_impl(cvrpsd_ctx *ctx, const int32_t *tour, int32_t n, const int32
             st.launches = 4;
         } else if (kernel == CVRPSD_KERNEL_WARP && !pred) {
             if (timed) CK(cudaEventRecord(ctx->ev_t[0], stream), "cudaEventRecord");
-            CK(launch_split_walk(p, demand_dtype, stream), "split_walk launch");
+            CK(launch_split_walk(p, demand_dtype, ctx->sm_count, stream), "split_walk launch");
             if (timed) CK(cudaEventRecord(ctx->ev_t[1], stream), "cudaEventRecord");
             st.kernel = CVRPSD_KERNEL_WARP;
             st.launches = 1;

@@ -106,7 +106,7 @@ cudaError_t launch_split_warp(const SplitParams &p, int esize, const int32_t *li
                               cudaStream_t stream);
 // One scenario per warp by the register walk; scenarios with a window longer
 // than 64 go on p.ovf_list (count in ACC_OVERFLOW) for launch_split_warp.
-cudaError_t launch_split_walk(const SplitParams &p, int esize, cudaStream_t stream);
+cudaError_t launch_split_walk(const SplitParams &p, int esize, int sm_count, cudaStream_t stream);
 inline size_t split_warp_smem_per_warp(int n) { return (size_t)2 * (n + 1) * sizeof(int); }
 
 // ---- batches of tours (one persistent launch) ----

@@ -49,13 +49,13 @@ struct __align__(16) WalkSmem {
 // step itself are added on uniform registers. PLAIN: no window of the chunk
 // is longer than 32 positions or starts inside its own step.
 template <bool PLAIN>
-__device__ __forceinline__ void walk_chunk(const WalkSmem &w, int n, int i0, int &v0, int &v1, int &pl)
+__device__ __forceinline__ void walk_chunk(const int *lo32, const int *c32, int n, int i0, int &v0, int &v1, int &pl)
 {
     constexpr int kNone = INT32_MAX;
     constexpr unsigned kAll = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const bool odd = lane & 1, high = lane & 2;
-    const int4 *lo = reinterpret_cast<const int4 *>(w.lo), *c = reinterpret_cast<const int4 *>(w.c);
+    const int4 *lo = reinterpret_cast<const int4 *>(lo32), *c = reinterpret_cast<const int4 *>(c32);
     int4 l4 = lo[0], c4 = c[0];
 #pragma unroll
     for (int b = 0; b < 8; ++b) {
@@ -93,11 +93,97 @@ __device__ __forceinline__ void walk_chunk(const WalkSmem &w, int n, int i0, int
     }
 }
 
-// Evaluates scenario s of one tour with the calling (full) warp, 32
-// positions (one per lane) to a chunk: the chunk's demands (loaded a chunk
-// ahead) are scanned to prefix loads, each lane finds its position's window
-// start by bisection over the prefix loads kept in shared memory, and the
-// recursion follows.
+// One scenario's positions prepared by a (full) warp, 32 at a time, one per
+// lane: demands (loaded a chunk ahead) are scanned to prefix loads, and each
+// lane finds its position's window start by bisection over the prefix loads
+// kept in shared memory.
+template <typename DT>
+struct WalkPrep {
+    static constexpr unsigned kAll = 0xffffffffu;
+    const TourStep *__restrict__ tab;
+    int n, Q, L;
+    const DT *__restrict__ dem;
+    long long ld, s;
+    unsigned long long *status;
+    int *P;                                                    // kWalkRing prefix loads, this warp's
+    TourStep t0, t1;                                           // table entries of this chunk and the next
+    int q, carry;
+    bool neg, bad;
+
+    __device__ __forceinline__ TourStep step_of(int i) const
+    {
+        const TourStep none{0, 0};
+        return i <= n ? tab[i - 1] : none;
+    }
+    __device__ __forceinline__ int demand_of(const TourStep &t, int i) const
+    {
+        const int row = t.row & kRowMask;
+        return i <= n && index_ok(row < n && s >= 0 && s < ld, status) ? (int)__ldg(dem + (long long)row * ld + s) : 0;
+    }
+    __device__ __forceinline__ void start()
+    {
+        const int lane = threadIdx.x & 31;
+        t0 = step_of(1 + lane);
+        t1 = step_of(33 + lane);
+        q = demand_of(t0, 1 + lane);
+        carry = 0;
+        neg = bad = false;
+        __syncwarp();                                          // the previous scenario's readers are done
+        if (lane == 0) P[0] = 0;
+    }
+    // The chunk from i0: window starts to lo, C_i to c. False (uniformly) if the
+    // scenario has no cost (bad) or a window longer than kWalkWidth.
+    __device__ __forceinline__ bool chunk(int i0, int *lo_out, int *c_out, bool &plain)
+    {
+        const int lane = threadIdx.x & 31, i = i0 + lane;
+        const TourStep t2 = step_of(i + 64);
+        const int qn = demand_of(t1, i + 32);
+        neg |= q < 0;
+        bad |= q > Q;
+        int p = max(q, 0);
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int u = __shfl_up_sync(kAll, p, o);
+            if (lane >= o) p += u;
+        }
+        p += carry;
+        carry = __shfl_sync(kAll, p, 31);
+        P[i & (kWalkRing - 1)] = p;
+        __syncwarp();
+        const int first = max(0, i - L);                       // the route-length limit's start
+        const int before = i - kWalkWidth - 1;
+        const bool wide = i <= n && before >= first && p - P[before & (kWalkRing - 1)] <= Q;
+        // a scenario with a demand above Q has no cost; one with a longer window is not for this walk
+        if (__any_sync(kAll, wide | bad)) return false;
+        int lo = max(first, i - kWalkWidth), hi = i - 1;       // hi is always in the window
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+            const int mid = (lo + hi) >> 1;
+            const bool in = p - P[mid & (kWalkRing - 1)] <= Q;
+            hi = in ? mid : hi;
+            lo = in ? lo : mid + 1;
+        }
+        // positions past n (the last chunk) have an empty window
+        lo_out[lane] = i <= n ? lo : INT32_MAX;
+        c_out[lane] = t0.c;
+        plain = __all_sync(kAll, i > n || (i - lo <= 32 && lo <= i - (lane & 3)));
+        t0 = t1;
+        t1 = t2;
+        q = qn;
+        return true;
+    }
+    // After the last chunk, or the one that ended the walk.
+    __device__ __forceinline__ void finish(bool ended, bool &any_neg, bool &any_bad)
+    {
+        any_bad = __any_sync(kAll, bad);
+        if (ended && any_bad)                                  // a negative demand anywhere is still reported
+            for (int i = 1 + (threadIdx.x & 31); i <= n; i += 32) neg |= demand_of(step_of(i), i) < 0;
+        any_neg = __any_sync(kAll, neg);
+    }
+};
+
+// Evaluates scenario s of one tour with the calling (full) warp: 32 positions
+// are prepared, then walked.
 //
 // What bounds it: the chain of a step (select, 18 clocks of reduction, four
 // additions and minima, insertion) while few warps run, issue of the ALU pipe
@@ -107,71 +193,26 @@ __device__ __forceinline__ WarpResult warp_walk_scenario(const TourStep *__restr
                                                          const DT *__restrict__ dem, long long ld, long long s,
                                                          WalkSmem &w, unsigned long long *status)
 {
-    constexpr unsigned kAll = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     WarpResult r{INT32_MAX, false, false, false};
-    const TourStep none{0, 0};
-    auto step_of = [&](int i) { return i <= n ? tab[i - 1] : none; };
-    auto demand_of = [&](const TourStep &t, int i) {
-        const int row = t.row & kRowMask;
-        return i <= n && index_ok(row < n && s >= 0 && s < ld, status) ? (int)__ldg(dem + (long long)row * ld + s) : 0;
-    };
-    TourStep t0 = step_of(1 + lane), t1 = step_of(33 + lane);
-    int q = demand_of(t0, 1 + lane);
+    WalkPrep<DT> pr{tab, n, Q, L, dem, ld, s, status, w.P};
+    pr.start();
     int v0 = lane == 31 ? g0 : INT32_MAX, v1 = INT32_MAX, pl = lane == 31 ? 0 : -kWalkWidth;
-    int carry = 0;
-    bool neg = false, bad = false;
-    __syncwarp();                                              // the previous scenario's readers are done
-    if (lane == 0) w.P[0] = 0;
+    bool ended = false;
     for (int i0 = 1; i0 <= n; i0 += 32) {
-        const int i = i0 + lane;
-        const TourStep t2 = step_of(i + 64);
-        const int qn = demand_of(t1, i + 32);
-        neg |= q < 0;
-        bad |= q > Q;
-        int P = max(q, 0);
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int u = __shfl_up_sync(kAll, P, o);
-            if (lane >= o) P += u;
-        }
-        P += carry;
-        carry = __shfl_sync(kAll, P, 31);
-        w.P[i & (kWalkRing - 1)] = P;
-        __syncwarp();
-        const int first = max(0, i - L);                       // the route-length limit's start
-        const int before = i - kWalkWidth - 1;
-        const bool wide = i <= n && before >= first && P - w.P[before & (kWalkRing - 1)] <= Q;
-        // a scenario with a demand above Q has no cost; one with a longer window is not for this walk
-        if (__any_sync(kAll, wide | bad)) {
-            r.bad = __any_sync(kAll, bad);
-            r.wide = !r.bad;
+        bool plain;
+        if (!pr.chunk(i0, w.lo, w.c, plain)) {
+            ended = true;
             break;
         }
-        int lo = max(first, i - kWalkWidth), hi = i - 1;       // hi is always in the window
-#pragma unroll
-        for (int k = 0; k < 6; ++k) {
-            const int mid = (lo + hi) >> 1;
-            const bool in = P - w.P[mid & (kWalkRing - 1)] <= Q;
-            hi = in ? mid : hi;
-            lo = in ? lo : mid + 1;
-        }
-        const bool plain = i > n || (i - lo <= 32 && lo <= i - (lane & 3));
-        // positions past n (the last chunk) have an empty window
-        w.lo[lane] = i <= n ? lo : INT32_MAX;
-        w.c[lane] = t0.c;
         __syncwarp();
-        if (__all_sync(kAll, plain)) walk_chunk<true>(w, n, i0, v0, v1, pl);
-        else walk_chunk<false>(w, n, i0, v0, v1, pl);
-        t0 = t1;
-        t1 = t2;
-        q = qn;
+        if (plain) walk_chunk<true>(w.lo, w.c, n, i0, v0, v1, pl);
+        else walk_chunk<false>(w.lo, w.c, n, i0, v0, v1, pl);
     }
-    if (r.bad)                                                 // a negative demand anywhere is still reported
-        for (int i = 1 + lane; i <= n; i += 32) neg |= demand_of(step_of(i), i) < 0;
-    r.neg = __any_sync(kAll, neg);
-    const int cost = __shfl_sync(kAll, v0, (n - 1) & 31);
-    if (!r.bad && !r.wide) r.cost = cost;
+    pr.finish(ended, r.neg, r.bad);
+    r.wide = ended && !r.bad;
+    const int cost = __shfl_sync(0xffffffffu, v0, (n - 1) & 31);
+    if (!ended) r.cost = cost;
     return r;
 }
 
@@ -309,8 +350,82 @@ __global__ void __launch_bounds__(32 * kWalkWarps) split_walk_kernel(SplitParams
     block_finish(p.acc, p.done);
 }
 
-cudaError_t launch_split_walk(const SplitParams &p, int esize, cudaStream_t stream)
+// The register walk with a second warp that prepares the next 32 positions
+// while the first walks these: a block is one scenario, and the two meet at a
+// barrier per chunk.
+//
+// What bounds it: the walking warp's chain (see above), which one warp alone
+// interrupts for the 37 % of its time that a chunk's preparation takes. A call
+// with n = 1000, S = 37 takes 67 us, 78 without the second warp.
+__device__ __forceinline__ void pair_sync() { asm volatile("bar.sync 1, 64;" ::: "memory"); }
+
+template <typename DT>
+__global__ void __launch_bounds__(64) split_walk_pair_kernel(SplitParams p)
 {
+    __shared__ int s_prefix[kWalkRing];
+    __shared__ __align__(16) int s_lo[2][32], s_c[2][32];
+    __shared__ int s_mode[2];                                  // 0 ended, 1 general, 2 plain
+    __shared__ int s_flags;                                    // 1 negative demand, 2 demand above Q
+    const int lane = threadIdx.x & 31, n = p.n;
+    const long long s = blockIdx.x;
+    const bool prepares = threadIdx.x >= 32;
+    const int chunks = (n + 31) >> 5;
+    int v0 = lane == 31 ? p.g0 : INT32_MAX, v1 = INT32_MAX, pl = lane == 31 ? 0 : -kWalkWidth;
+    bool ended = false;
+    if (prepares) {
+        WalkPrep<DT> pr{p.tab, n, p.Q, p.L, reinterpret_cast<const DT *>(p.demand), p.ld, s, p.acc + ACC_STATUS, s_prefix};
+        pr.start();
+        for (int k = 0; k < chunks && !ended; ++k) {
+            bool plain = false;
+            ended = !pr.chunk(1 + 32 * k, s_lo[k & 1], s_c[k & 1], plain);
+            if (lane == 0) s_mode[k & 1] = ended ? 0 : plain ? 2 : 1;
+            pair_sync();                                       // chunk k is there, chunk k - 1 walked
+        }
+        bool neg, bad;
+        pr.finish(ended, neg, bad);
+        if (lane == 0) s_flags = (neg ? 1 : 0) | (bad ? 2 : 0);
+    } else {
+        for (int k = 0; k < chunks; ++k) {
+            pair_sync();
+            const int mode = s_mode[k & 1];
+            if (mode == 2) walk_chunk<true>(s_lo[k & 1], s_c[k & 1], n, 1 + 32 * k, v0, v1, pl);
+            else if (mode == 1) walk_chunk<false>(s_lo[k & 1], s_c[k & 1], n, 1 + 32 * k, v0, v1, pl);
+            else {
+                ended = true;
+                break;
+            }
+        }
+    }
+    __syncthreads();
+    const int cost = __shfl_sync(0xffffffffu, v0, (n - 1) & 31);
+    long long sum = 0;
+    unsigned inf = 0, status = 0;
+    if (threadIdx.x == 0) {
+        const int flags = s_flags;
+        if (ended && !(flags & 2)) {                           // a long window: set aside
+            const unsigned long long idx = atomicAdd(p.acc + ACC_OVERFLOW, 1ull);
+            if (index_ok(idx < (unsigned long long)p.S, p.acc + ACC_STATUS)) p.ovf_list[idx] = (int32_t)s;
+        } else {
+            if (flags & 1) status = ST_NEGATIVE_DEMAND;
+            if (ended) inf = 1; else sum = cost;
+            if (p.out_cost) p.out_cost[s] = ended ? INT32_MAX : cost;
+        }
+    }
+    if (status) atomicOr(p.sticky, (unsigned long long)status);
+    block_accumulate(sum, inf, status, p.acc);
+    block_finish(p.acc, p.done);
+}
+
+cudaError_t launch_split_walk(const SplitParams &p, int esize, int sm_count, cudaStream_t stream)
+{
+    // Pairs while each scenario can have a walking warp's scheduler to itself;
+    // more of them fill the preparation's gaps with other scenarios (n = 1000, us
+    // per call alone / in pairs: S = 600 78.9, 69.9; 1000 82, 82; 2000 96.7, 100).
+    if (p.S <= 4LL * sm_count) {
+        if (esize == 2) split_walk_pair_kernel<int16_t><<<(unsigned)p.S, 64, 0, stream>>>(p);
+        else split_walk_pair_kernel<int32_t><<<(unsigned)p.S, 64, 0, stream>>>(p);
+        return cudaGetLastError();
+    }
     const unsigned grid = (unsigned)((p.S + kWalkWarps - 1) / kWalkWarps);
     if (esize == 2) split_walk_kernel<int16_t><<<grid, 32 * kWalkWarps, 0, stream>>>(p);
     else split_walk_kernel<int32_t><<<grid, 32 * kWalkWarps, 0, stream>>>(p);

@@ -66,3 +66,34 @@ def test_automatic_choice_is_exact(cv, n, S):
     r, got = split(cv, sp, inst, D, 200, 60)
     assert np.array_equal(got, want) and (r.sum, r.infeasible) == (ws, wi)
     sp.close()
+
+
+@pytest.mark.parametrize("more", [-1, 0, 1])                 # around four scenarios per SM: pairs, then lone warps
+@pytest.mark.parametrize("n,Q", [(1, 30), (32, 60), (33, 60), (200, 150), (200, 700)])
+@pytest.mark.parametrize("dtype", [np.int16, np.int32])
+def test_pairs_and_lone_warps(cv, more, n, Q, dtype):
+    S = 4 * torch.cuda.get_device_properties(0).multi_processor_count + more
+    rng = np.random.default_rng([n, S])
+    inst = make_instance(n, 1, 10, seed=n + S, Q=Q)
+    D = rng.integers(0, 20, size=(n, S)).astype(dtype)
+    D[:, 1] = 0                                              # a window of the whole tour, after short ones
+    D[: n // 2, 2] = 5
+    D[n // 2:, 2] = 0
+    D[n - 1, 3] = Q + 1
+    D[0, S - 1] = Q + 1
+    sp = cv.Splitter(0)
+    sp.configure(kernel=cv.KERNEL_WARP)
+    want, ws, wi, _ = oracle.split_costs(inst.tour, inst.dist, D, Q, n, nthreads=4)
+    for _ in range(2):                                       # the second call finds the first one's totals
+        r, got = split(cv, sp, inst, D, Q, n)
+        assert np.array_equal(got, want)
+        assert (r.sum, r.infeasible) == (ws, wi) and wi >= 2
+    D[0, 3] = -1                                             # beside a demand above Q (n = 1: alone)
+    with pytest.raises(cv.CvrpsdError):
+        split(cv, sp, inst, D, Q, n)
+    sp.close()
+
+
+@pytest.mark.parametrize("n,S", [(2999, 48), (3000, 48), (3000, 49)])
+def test_automatic_choice_of_long_tours_is_exact(cv, n, S):
+    test_automatic_choice_is_exact(cv, n, S)
