@@ -1,10 +1,8 @@
 // Surrogate network for screening local-search neighbours: training and
 // inference kernels. BF16 weights, per-position features as BF16 hi + lo
 // pairs (about 16 significant bits), FP32 activations and accumulation.
-// The products of layers 1 and 2, forward and backward, run on the tensor
-// cores (mlp_tc.cu, with the output layer and the loss in their epilogue); this
-// file holds the rest: the output layer's gradient, the layer-2 bias gradient
-// and Adam.
+// The layers run on the tensor cores, forward and backward (mlp_tc.cu); this
+// file holds Adam, the BF16 copies and the order of the launches.
 //
 // Architecture (width H = 256):
 //   per position k of a tour:  phi_k = (x, y, mu / Q, sd / Q, frac(cum_k / Q))
@@ -26,37 +24,6 @@
 #include "tcgen05.h"
 
 namespace cvrpsd {
-
-// ---------------------------------------------------------------- layer 3 backward
-
-// dU[b][j] = dy_b w3_j [u_bj > 0]; g_w3[j] += sum_b dy_b u_bj; g_b3 += sum_b
-// dy_b; g_b2[j] += sum_b dU[b][j]. A block takes 16 rows, eight at a time in
-// flight, and one atomic per column and sum (with two rows a block and the
-// last sum in a kernel of its own: 7.4 + 6.8 us for 1024 rows).
-constexpr int kOutRows = 16;
-
-__global__ void __launch_bounds__(kMlpH) mlp_out_backward_kernel(const float *U, int B, const float *dy,
-                                                                 const __nv_bfloat16 *w3, float *dU, float *gw3,
-                                                                 float *gb3, float *gb2)
-{
-    const int j = threadIdx.x;                // kMlpH threads
-    float acc = 0.0f, accb = 0.0f, accu = 0.0f;
-    const float wj = __bfloat162float(w3[j]);
-    const int b0 = blockIdx.x * kOutRows, b1 = min(B, b0 + kOutRows);
-#pragma unroll 8
-    for (int b = b0; b < b1; ++b) {
-        const float u = U[(long long)b * kMlpH + j];
-        const float d = dy[b];
-        acc += d * u;
-        accb += d;
-        const float du = u > 0.0f ? d * wj : 0.0f;
-        accu += du;
-        dU[(long long)b * kMlpH + j] = du;
-    }
-    atomicAdd(gw3 + j, acc);
-    atomicAdd(gb2 + j, accu);
-    if (j == 0) atomicAdd(gb3, accb);
-}
 
 // ---------------------------------------------------------------- Adam
 
@@ -95,7 +62,6 @@ __global__ void to_bf16_kernel(const float *p, __nv_bfloat16 *q, unsigned char *
 
 // ---------------------------------------------------------------- host launchers
 
-
 cudaError_t mlp_forward(const MlpLayer1Args &l1, const MlpWeights &wt, float *U, float *y, const float *target,
                         float *dy, float *loss, cudaStream_t st)
 {
@@ -105,24 +71,17 @@ cudaError_t mlp_forward(const MlpLayer1Args &l1, const MlpWeights &wt, float *U,
     return mlp_head(MlpHeadArgs{l1.z_hi, l1.z_lo, wt.w2b, wt.w3, wt.b3, T, U, y, target, dy, loss, l1.err}, st);
 }
 
-cudaError_t mlp_backward(const MlpLayer1Args &l1, const MlpWeights &wt, const float *U, const float *dy, float *dU,
-                         float *dzt, float *grad, cudaStream_t st)
+cudaError_t mlp_backward(const MlpLayer1Args &l1, const MlpWeights &wt, const float *U, const float *dy, float *dzt,
+                         float *grad, cudaStream_t st)
 {
-    const int T = l1.T;
-    float *gw1 = grad + kOffW1, *gb1 = grad + kOffB1, *gw2 = grad + kOffW2, *gb2 = grad + kOffB2;
-    float *gw3 = grad + kOffW3, *gb3 = grad + kOffB3;
-    mlp_out_backward_kernel<<<(unsigned)((T + kOutRows - 1) / kOutRows), kMlpH, 0, st>>>(U, T, dy, wt.w3, dU, gw3, gb3, gb2);
-    cudaError_t e = mlp_grad_w2_tc(dU, l1.zt, T, gw2, l1.err, st);
-    if (e != cudaSuccess) return e;
-    e = mlp_grad_zt_tc(dU, T, wt.w2, dzt, l1.err, st);
+    cudaError_t e = mlp_grad(MlpGradArgs{U, dy, wt.w3, wt.w2, l1.zt, l1.T, dzt, grad + kOffW2, grad + kOffW3,
+                                         grad + kOffB2, grad + kOffB3, l1.err}, st);
     if (e != cudaSuccess) return e;
     MlpLayer1Args b = l1;
     b.dzt = dzt;
-    b.gw1 = gw1;
-    b.gb1 = gb1;
-    e = mlp_layer1_bwd_tc(b, l1.sm_count > 0 ? l1.sm_count : 1, st);
-    if (e != cudaSuccess) return e;
-    return cudaGetLastError();
+    b.gw1 = grad + kOffW1;
+    b.gb1 = grad + kOffB1;
+    return mlp_layer1_bwd_tc(b, l1.sm_count > 0 ? l1.sm_count : 1, st);
 }
 
 cudaError_t mlp_adam(float *p, const float *g, float *m, float *v, __nv_bfloat16 *pb, unsigned char *w2b, float lr,

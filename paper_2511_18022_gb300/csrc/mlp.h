@@ -48,6 +48,7 @@ struct MlpLayer1Args {
     unsigned char *z_hi, *z_lo;            // device: the same as the head's operands (mlp_tile_bytes(T) each)
     const float *dzt;                      // backward: gradient of the pooled features, [T][H]
     float *gw1, *gb1;                      // backward: accumulated gradients
+    float *loss;                           // forward: cleared for the head that follows, or nullptr
     unsigned int *err;                     // device word: set if a tensor-core wait gave up
     int sm_count;                          // SMs of the device (grid of the tensor-core kernel)
 };
@@ -73,16 +74,22 @@ cudaError_t mlp_layer1_bwd_tc(const MlpLayer1Args &l1, int sm_count, cudaStream_
 // (mlp_tc.cu).
 cudaError_t mlp_head(const MlpHeadArgs &a, cudaStream_t st);
 
-// Backward products on the tensor cores (mlp_tc.cu): dZ = dU W2 and
-// gW2 += dU^T ZT (FP32 operands as BF16 hi/lo pairs, FP32 accumulation).
-cudaError_t mlp_grad_zt_tc(const float *dU, int T, const __nv_bfloat16 *w2, float *dzt, unsigned int *err,
-                           cudaStream_t st);
-cudaError_t mlp_grad_w2_tc(const float *dU, const float *zt, int T, float *gw2, unsigned int *err, cudaStream_t st);
+// Gradients of layers 2 and 3 from U and dy, and dZ for layer 1.
+struct MlpGradArgs {
+    const float *U, *dy;                       // T x 256 (rows 16-byte aligned), T
+    const __nv_bfloat16 *w3, *w2;
+    const float *zt;                           // T x 257: pooled features and tour length
+    int T;
+    float *dzt;                                // T x 256, written
+    float *gw2, *gw3, *gb2, *gb3;              // added to
+    unsigned int *err;
+};
+cudaError_t mlp_grad(const MlpGradArgs &g, cudaStream_t st);
 
 cudaError_t mlp_forward(const MlpLayer1Args &l1, const MlpWeights &wt, float *U, float *y, const float *target,
                         float *dy, float *loss, cudaStream_t st);
-cudaError_t mlp_backward(const MlpLayer1Args &l1, const MlpWeights &wt, const float *U, const float *dy, float *dU,
-                         float *dzt, float *grad, cudaStream_t st);
+cudaError_t mlp_backward(const MlpLayer1Args &l1, const MlpWeights &wt, const float *U, const float *dy, float *dzt,
+                         float *grad, cudaStream_t st);
 // Both write the BF16 copies: pb (flat) and W2' in w2b (whose padding the
 // caller has zeroed once).
 cudaError_t mlp_adam(float *p, const float *g, float *m, float *v, __nv_bfloat16 *pb, unsigned char *w2b, float lr,

@@ -169,6 +169,7 @@ __global__ void __launch_bounds__(kF1Threads, 1) mlp_layer1_tc_kernel(MlpLayer1A
 
     stage_w1(a, s_w1, tid, kF1Threads);
     if (tid == 0) {
+        if (!BWD && a.loss && blockIdx.x == 0) *a.loss = 0.0f;
         for (int l = 0; l < kF1Lines; ++l) {
             for (int p = 0; p < kF1Prod; ++p)
                 for (int k = 0; k < kF1Depth; ++k) {
@@ -550,181 +551,263 @@ __global__ void __launch_bounds__(kTcThreads, 1) mlp_head_kernel(MlpHeadArgs a)
     if (w == 0) tc::tmem_dealloc(tmem, kHeadTmemCols);
 }
 
-// ---------------------------------------------------------------- backward GEMMs
+// ---------------------------------------------------------------- gradients behind layer 1
 //
-// C (M x N) = A (M x K) B (N x K)^T on the tensor cores, stored or added
-// atomically (split-K over blockIdx.z). One CTA computes a 128 x 96 tile of C
-// in tensor memory, K in chunks of 128 staged in shared memory in the K-major
-// layout of the forward kernels. FP32 operands are split into BF16 hi and
-// lo parts (hi = bf16(v), lo = bf16(v - hi)); a product of two split
-// operands takes hi*hi + hi*lo + lo*hi (the lo*lo term, at most 2^-18 of
-// the product, is the order of the pair's own rounding and is left out),
-// one with an exact BF16 operand hi*B + lo*B. Operands
-// are read through an element rule: A(m, k) at a[m * lda + k], or at
-// a[k * lda + m] when transposed (AT); B likewise (BT), FP32 or BF16.
-constexpr int kGM = 128;                       // rows of C per CTA
-constexpr int kGN = 96;                        // columns of C per CTA (3 x 32)
+// With dU[b][j] = dy_b w3_j [u_bj > 0], formed from U where it is staged:
+//   dZ (T x 256) = dU (T x 256) W2[:, 0..255]   (the tour length has no
+//                                                gradient to pass on)
+//   gW2 (256 x 257) += dU^T (256 x T) ZT (T x 257), in slabs of 128 tours
+//   gw3_j += sum_b dy_b u_bj, gb2_j += sum_b dU[b][j], gb3 += sum_b dy_b
+// in one launch, whose first blocks take 128 x 64 tiles of dZ and the others 128 x
+// 80 tiles of gW2; those of the first columns also add up the three sums, over the
+// slab that they stage anyway. FP32 operands are split into BF16 hi and lo parts
+// (hi = bf16(v), lo = bf16(v - hi)); a product of two split operands takes
+// hi*hi + hi*lo + lo*hi (the lo*lo term, at most 2^-18 of the product, is the
+// order of the pair's own rounding and is left out), one with an exact BF16
+// operand hi*B + lo*B.
+//
+// What bounds it: latency. A tile's chain is two rounds of loads per operand and
+// chunk of K = 128, the MMAs, their commit and the epilogue, and there are
+// fewer tiles than SMs at the usual 1024 tours; so a thread has 32 words and
+// more in flight, and the accumulators go through shared memory to full rows.
+// 13.3 us for 1024 tours; as an elementwise kernel and two products, one after
+// the other: 10.9 + 17.3 + 23.2. 80 columns, not 96: two blocks fit an SM.
+constexpr int kGM = 128;                       // rows of a tile
+constexpr int kGNz = 64, kGNw = 80;            // its columns: dZ, gW2
 constexpr int kGK = 128;                       // K per staged chunk
 constexpr int kGKc = kGK / 8;                  // 16-byte core-matrix columns per row group
 constexpr size_t kGA = (size_t)kGM * kGK * 2;  // one BF16 A part
-constexpr size_t kGB = (size_t)kGN * kGK * 2;  // one BF16 B part
-constexpr size_t kGSmem = 2 * kGA + 2 * kGB;   // A hi, A lo, B hi, B lo
-// Requested dynamic shared memory: the operands plus padding so that one CTA
-// of this kernel runs on an SM.
-constexpr size_t kGSmemReq = 120 * 1024;
-static_assert(kGSmem <= kGSmemReq, "GEMM operands exceed the requested shared memory");
+constexpr size_t kGB = (size_t)kGNw * kGK * 2; // one BF16 B part
+constexpr size_t kGSmem = 2 * kGA + 2 * kGB;   // A hi, A lo, B hi, B lo; then the tile of C
+static_assert((size_t)kGM * (kGNw + 1) * 4 <= kGSmem, "the tile of C takes the operands' place");
 constexpr uint32_t kGTmemCols = 128;
+constexpr int kGwTiles = (kMlpIn2 + kGNw - 1) / kGNw;
+static_assert(kMlpH == 2 * kGM && kMlpH == kTcThreads && kMlpH % kGNz == 0, "tiles of the two products");
 
-struct TcGemm {
-    const float *a;          // FP32 A
-    int lda;
-    const float *bf;         // FP32 B (or nullptr)
-    const __nv_bfloat16 *bh; // BF16 B (or nullptr)
-    int ldb;
-    int M, N, K;
-    int k_slab;              // K per blockIdx.z
-    float *out;
-    int ldo;
-    unsigned int *err;
-};
-
-template <bool AT, bool BT, bool BBF16, bool ATOMIC>
-__global__ void __launch_bounds__(kTcThreads, 1) tc_gemm_kernel(TcGemm g)
+// Eight values along K as BF16 hi and lo parts.
+__device__ __forceinline__ void split8(const float (&v)[8], uint4 &hi, uint4 &lo)
 {
-    extern __shared__ __align__(128) unsigned char smem[];   // A hi | A lo | B hi | B lo
-    __shared__ __align__(8) unsigned long long s_mbar;
-    __shared__ uint32_t s_tmem;
-    unsigned char *a_hi = smem, *a_lo = smem + kGA, *b_hi = smem + 2 * kGA, *b_lo = smem + 2 * kGA + kGB;
+    uint32_t h[4], l[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const __nv_bfloat16 h0 = __float2bfloat16_rn(v[2 * q]), h1 = __float2bfloat16_rn(v[2 * q + 1]);
+        h[q] = pack_bf16x2(h0, h1);
+        l[q] = pack_bf16x2(__float2bfloat16_rn(v[2 * q] - __bfloat162float(h0)),
+                           __float2bfloat16_rn(v[2 * q + 1] - __bfloat162float(h1)));
+    }
+    hi = make_uint4(h[0], h[1], h[2], h[3]);
+    lo = make_uint4(l[0], l[1], l[2], l[3]);
+}
+
+__device__ __forceinline__ float relu_grad(float u, float d, float w) { return u > 0.0f ? d * w : 0.0f; }
+
+// dZ: rows m0.. of A, all K in two chunks. s_d holds dy of the tile's rows.
+__device__ __forceinline__ void stage_dz(const MlpGradArgs &g, unsigned char *smem, const float *s_d, const float *s_w3,
+                                         int m0, int n0, int kc0)
+{
+    unsigned char *a_hi = smem, *a_lo = smem + kGA, *b_hi = smem + 2 * kGA;
     const int j = threadIdx.x, lane = j & 31, w = j >> 5;
-    const int m0 = blockIdx.x * kGM, n0 = blockIdx.y * kGN;
-    const int k_begin = blockIdx.z * g.k_slab, k_end = min(g.K, k_begin + g.k_slab);
-    const uint32_t mbar = (uint32_t)__cvta_generic_to_shared(&s_mbar);
-    if (j == 0) tc::mbar_init(mbar);
-    if (w == 0) tc::tmem_alloc((uint32_t)__cvta_generic_to_shared(&s_tmem), kGTmemCols);
-    tc::fence_before_sync();
+    // an eighth of a warp reads a whole line of a row, and eight rows make a core matrix
+#pragma unroll
+    for (int half = 0; half < 2; ++half) {
+        float4 x[4][2];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int it = w * 8 + half * 4 + i, m = m0 + (it >> 2) * 8 + (lane & 7), gk = (it & 3) * 4 + (lane >> 3);
+            const float4 *src = reinterpret_cast<const float4 *>(g.U + (long long)m * kMlpH + kc0 + 8 * gk);
+            const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+            x[i][0] = m < g.T ? __ldg(src) : zero;
+            x[i][1] = m < g.T ? __ldg(src + 1) : zero;
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int it = w * 8 + half * 4 + i, r = (it >> 2) * 8 + (lane & 7), gk = (it & 3) * 4 + (lane >> 3);
+            const float d = s_d[r], *w3 = s_w3 + kc0 + 8 * gk;
+            const float u[8] = {x[i][0].x, x[i][0].y, x[i][0].z, x[i][0].w, x[i][1].x, x[i][1].y, x[i][1].z, x[i][1].w};
+            float v[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) v[q] = relu_grad(u[q], d, w3[q]);
+            uint4 hi, lo;
+            split8(v, hi, lo);
+            const uint32_t off = tc::kmajor_offset(r, 8 * gk, kGKc);
+            *reinterpret_cast<uint4 *>(a_hi + off) = hi;
+            *reinterpret_cast<uint4 *>(a_lo + off) = lo;
+        }
+    }
+    // B(n, k) = W2[k][n0 + n], neighbouring threads on neighbouring columns
+    const int r = j % kGNz;
+    unsigned short b[4][8];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+            b[i][q] = __ldg(reinterpret_cast<const unsigned short *>(g.w2) +
+                            (kc0 + 8 * (j / kGNz + 4 * i) + q) * kMlpIn2 + n0 + r);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        uint32_t p[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) p[q] = (uint32_t)b[i][2 * q] | (uint32_t)b[i][2 * q + 1] << 16;
+        *reinterpret_cast<uint4 *>(b_hi + tc::kmajor_offset(r, 8 * (j / kGNz + 4 * i), kGKc)) =
+            make_uint4(p[0], p[1], p[2], p[3]);
+    }
+}
+
+// gW2: hidden units m0.. over the slab of tours from kc0. s_d holds the slab's dy (0 past T).
+__device__ __forceinline__ void stage_gw2(const MlpGradArgs &g, unsigned char *smem, const float *s_d, const float *s_w3,
+                                          int m0, int n0, int kc0)
+{
+    unsigned char *a_hi = smem, *a_lo = smem + kGA, *b_hi = smem + 2 * kGA, *b_lo = smem + 2 * kGA + kGB;
+    const int j = threadIdx.x, r = j % kGM;
+    const float w3 = s_w3[m0 + r];
+    float sum = 0.0f, sumu = 0.0f;
+#pragma unroll
+    for (int half = 0; half < 2; ++half) {
+        float x[4][8];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                const int b = kc0 + 8 * (j / kGM + 2 * (half * 4 + i)) + q;
+                x[i][q] = b < g.T ? __ldg(g.U + (long long)b * kMlpH + m0 + r) : 0.0f;
+            }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int gk = j / kGM + 2 * (half * 4 + i);
+            float v[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                const float d = s_d[8 * gk + q];
+                v[q] = relu_grad(x[i][q], d, w3);
+                sum += d * x[i][q];
+                sumu += v[q];
+            }
+            uint4 hi, lo;
+            split8(v, hi, lo);
+            const uint32_t off = tc::kmajor_offset(r, 8 * gk, kGKc);
+            *reinterpret_cast<uint4 *>(a_hi + off) = hi;
+            *reinterpret_cast<uint4 *>(a_lo + off) = lo;
+        }
+    }
+    if (n0 == 0) {
+        atomicAdd(g.gw3 + m0 + r, sum);
+        atomicAdd(g.gb2 + m0 + r, sumu);
+        if (m0 == 0 && j < 32) {
+            float d = (s_d[j] + s_d[j + 32]) + (s_d[j + 64] + s_d[j + 96]);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+            if (j == 0) atomicAdd(g.gb3, d);
+        }
+    }
+    float x[5][8];
+#pragma unroll
+    for (int i = 0; i < 5; ++i)
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const int e = j + i * kTcThreads, n = n0 + e % kGNw, b = kc0 + 8 * (e / kGNw) + q;
+            x[i][q] = n < kMlpIn2 && b < g.T ? __ldg(g.zt + (long long)b * kMlpIn2 + n) : 0.0f;
+        }
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+        const int e = j + i * kTcThreads;
+        uint4 hi, lo;
+        split8(x[i], hi, lo);
+        const uint32_t off = tc::kmajor_offset(e % kGNw, 8 * (e / kGNw), kGKc);
+        *reinterpret_cast<uint4 *>(b_hi + off) = hi;
+        *reinterpret_cast<uint4 *>(b_lo + off) = lo;
+    }
+}
+static_assert(kGNw * kGKc == 5 * kTcThreads && kGNz * kGKc == 4 * kTcThreads && kGM * kGKc == 8 * kTcThreads,
+              "items per thread of the staging loops");
+
+template <bool DZ>
+__device__ __forceinline__ void grad_tile(const MlpGradArgs &g, unsigned char *smem, uint32_t tmem, uint32_t mbar,
+                                          float *s_d, const float *s_w3, int m0, int n0, int b0)
+{
+    constexpr int N = DZ ? kGNz : kGNw, kChunks = DZ ? kMlpH / kGK : 1;
+    const int j = threadIdx.x, lane = j & 31, w = j >> 5;
+    if (j < kGM) s_d[j] = b0 + j < g.T ? __ldg(g.dy + b0 + j) : 0.0f;
     __syncthreads();
-    tc::fence_after_sync();
-    const uint32_t tmem = s_tmem;
-    uint32_t parity = 0;
-    bool ok = true, any = false;
-    for (int kc0 = k_begin; kc0 < k_end; kc0 += kGK) {
-        // A: item = (row, group of 8 K columns); transposed operands read the
-        // row index fastest, so neighbouring threads read neighbouring words
-#pragma unroll 4
-        for (int e = j; e < kGM * kGKc; e += kTcThreads) {
-            const int r = AT ? e % kGM : e / kGKc, gk = AT ? e / kGM : e % kGKc;
-            const int m = m0 + r;
-            uint32_t ph[4], pl[4];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                __nv_bfloat16 hi[2], lo[2];
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const int k = kc0 + 8 * gk + 2 * q + h;
-                    float v = 0.0f;
-                    if (m < g.M && k < k_end) v = AT ? g.a[(long long)k * g.lda + m] : g.a[(long long)m * g.lda + k];
-                    hi[h] = __float2bfloat16_rn(v);
-                    lo[h] = __float2bfloat16_rn(v - __bfloat162float(hi[h]));
-                }
-                ph[q] = pack_bf16x2(hi[0], hi[1]);
-                pl[q] = pack_bf16x2(lo[0], lo[1]);
-            }
-            const uint32_t off = tc::kmajor_offset(r, 8 * gk, kGKc);
-            *reinterpret_cast<uint4 *>(a_hi + off) = make_uint4(ph[0], ph[1], ph[2], ph[3]);
-            *reinterpret_cast<uint4 *>(a_lo + off) = make_uint4(pl[0], pl[1], pl[2], pl[3]);
-        }
-#pragma unroll 3
-        for (int e = j; e < kGN * kGKc; e += kTcThreads) {
-            const int r = BT ? e % kGN : e / kGKc, gk = BT ? e / kGN : e % kGKc;
-            const int nn = n0 + r;
-            uint32_t ph[4], pl[4];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                __nv_bfloat16 hi[2], lo[2];
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const int k = kc0 + 8 * gk + 2 * q + h;
-                    const bool in = nn < g.N && k < k_end;
-                    if (BBF16) {
-                        hi[h] = in ? (BT ? g.bh[(long long)k * g.ldb + nn] : g.bh[(long long)nn * g.ldb + k])
-                                   : __float2bfloat16_rn(0.0f);
-                        lo[h] = __float2bfloat16_rn(0.0f);
-                    } else {
-                        const float v = in ? (BT ? g.bf[(long long)k * g.ldb + nn] : g.bf[(long long)nn * g.ldb + k])
-                                           : 0.0f;
-                        hi[h] = __float2bfloat16_rn(v);
-                        lo[h] = __float2bfloat16_rn(v - __bfloat162float(hi[h]));
-                    }
-                }
-                ph[q] = pack_bf16x2(hi[0], hi[1]);
-                pl[q] = pack_bf16x2(lo[0], lo[1]);
-            }
-            const uint32_t off = tc::kmajor_offset(r, 8 * gk, kGKc);
-            *reinterpret_cast<uint4 *>(b_hi + off) = make_uint4(ph[0], ph[1], ph[2], ph[3]);
-            if (!BBF16) *reinterpret_cast<uint4 *>(b_lo + off) = make_uint4(pl[0], pl[1], pl[2], pl[3]);
-        }
+    bool ok = true;
+#pragma unroll 1
+    for (int c = 0; c < kChunks && ok; ++c) {
+        if (DZ) stage_dz(g, smem, s_d, s_w3, m0, n0, c * kGK);
+        else stage_gw2(g, smem, s_d, s_w3, m0, n0, b0);
         tc::fence_operands();
         tc::fence_before_sync();
         __syncthreads();
         tc::fence_after_sync();
         if (j == 0) {
-            const uint32_t idesc = tc::instr_desc(kGN);
-            const uint32_t sah = (uint32_t)__cvta_generic_to_shared(a_hi), sal = (uint32_t)__cvta_generic_to_shared(a_lo);
-            const uint32_t sbh = (uint32_t)__cvta_generic_to_shared(b_hi), sbl = (uint32_t)__cvta_generic_to_shared(b_lo);
-            const uint32_t sbo = kGKc * 128;
+            const uint32_t idesc = tc::instr_desc(N), sbo = kGKc * 128;
+            const uint32_t ah = (uint32_t)__cvta_generic_to_shared(smem), al = ah + kGA, bh = al + kGA, bl = bh + kGB;
             for (int step = 0; step < kGK / 16; ++step) {
-                const uint32_t koff = (uint32_t)step * 256;
-                const uint64_t ah = tc::smem_desc(sah + koff, 128, sbo), al = tc::smem_desc(sal + koff, 128, sbo);
-                const uint64_t bh = tc::smem_desc(sbh + koff, 128, sbo);
-                tc::mma_bf16(tmem, ah, bh, idesc, any || step > 0);
-                tc::mma_bf16(tmem, al, bh, idesc, true);
-                if (!BBF16) tc::mma_bf16(tmem, ah, tc::smem_desc(sbl + koff, 128, sbo), idesc, true);
+                const uint32_t ko = (uint32_t)step * 256;
+                const uint64_t dah = tc::smem_desc(ah + ko, 128, sbo), dal = tc::smem_desc(al + ko, 128, sbo);
+                const uint64_t dbh = tc::smem_desc(bh + ko, 128, sbo);
+                tc::mma_bf16(tmem, dah, dbh, idesc, c > 0 || step > 0);
+                tc::mma_bf16(tmem, dal, dbh, idesc, true);
+                if (!DZ) tc::mma_bf16(tmem, dah, tc::smem_desc(bl + ko, 128, sbo), idesc, true);
             }
             tc::mma_commit(mbar);
         }
-        any = true;
-        // the operands are overwritten next chunk: wait for the MMAs
-        ok = tc::mbar_wait(mbar, parity);
-        parity ^= 1u;
+        // the operands are overwritten next (by the next chunk, then by the tile): wait for the MMAs
+        ok = tc::mbar_wait(mbar, (uint32_t)c & 1u);
         if (!ok && lane == 0) atomicOr(g.err, 1u);
         tc::fence_after_sync();
-        __syncthreads();
-        if (!ok) break;
+        ok = __syncthreads_and(ok);
     }
-    if (ok && any && w < 4) {
-        const int m = m0 + 32 * w + lane;
-        const uint32_t row = tmem + ((uint32_t)(32 * w) << 16);
-#pragma unroll 1
-        for (int c = 0; c < kGN; c += 32) {
-            float r[32];
-            tc::tmem_ld32(row + c, r);
-            if (m < g.M) {
-                float *out = g.out + (long long)m * g.ldo + n0 + c;
+    float *tile = reinterpret_cast<float *>(smem);
+    if (ok && w < 4) {
 #pragma unroll
-                for (int q = 0; q < 32; ++q) {
-                    if (n0 + c + q < g.N) {
-                        if (ATOMIC) atomicAdd(out + q, r[q]);
-                        else out[q] = r[q];
-                    }
-                }
-            }
+        for (int c = 0; c < N; c += 32) {                     // the last load may run past N, within the allocation
+            float r[32];
+            tc::tmem_ld32(tmem + ((uint32_t)(32 * w) << 16) + c, r);
+#pragma unroll
+            for (int q = 0; q < 32; ++q)
+                if (c + q < N) tile[(32 * w + lane) * (N + 1) + c + q] = r[q];
         }
+    }
+    __syncthreads();
+    if (!ok) return;
+#pragma unroll 4
+    for (int e = j; e < kGM * N; e += kTcThreads) {
+        const int r = e / N, c = e % N;
+        const float v = tile[r * (N + 1) + c];
+        if (DZ) {
+            if (m0 + r < g.T) g.dzt[(long long)(m0 + r) * kMlpH + n0 + c] = v;
+        } else if (n0 + c < kMlpIn2) {
+            atomicAdd(g.gw2 + (long long)(m0 + r) * kMlpIn2 + n0 + c, v);
+        }
+    }
+}
+
+__global__ void __launch_bounds__(kTcThreads, 2) mlp_grad_kernel(MlpGradArgs g)
+{
+    extern __shared__ __align__(128) unsigned char smem[];
+    __shared__ __align__(8) unsigned long long s_mbar;
+    __shared__ uint32_t s_tmem;
+    __shared__ float s_w3[kMlpH], s_d[kGM];
+    const int j = threadIdx.x, w = j >> 5;
+    const uint32_t mbar = (uint32_t)__cvta_generic_to_shared(&s_mbar);
+    if (j == 0) tc::mbar_init(mbar);
+    if (w == 0) tc::tmem_alloc((uint32_t)__cvta_generic_to_shared(&s_tmem), kGTmemCols);
+    s_w3[j] = __bfloat162float(g.w3[j]);
+    tc::fence_before_sync();
+    __syncthreads();
+    tc::fence_after_sync();
+    const uint32_t tmem = s_tmem;
+    const int slabs = (g.T + kGM - 1) / kGM;                   // of 128 tours, in both products
+    const int b = blockIdx.x, dz = slabs * (kMlpH / kGNz);
+    if (b < dz) {
+        const int m0 = b / (kMlpH / kGNz) * kGM, n0 = b % (kMlpH / kGNz) * kGNz;
+        grad_tile<true>(g, smem, tmem, mbar, s_d, s_w3, m0, n0, m0);
+    } else {
+        const int t = b - dz, m0 = (t & 1) * kGM, n0 = (t >> 1) % kGwTiles * kGNw, b0 = (t >> 1) / kGwTiles * kGM;
+        grad_tile<false>(g, smem, tmem, mbar, s_d, s_w3, m0, n0, b0);
     }
     tc::fence_before_sync();
     __syncthreads();
     if (w == 0) tc::tmem_dealloc(tmem, kGTmemCols);
-}
-
-template <bool AT, bool BT, bool BBF16, bool ATOMIC>
-cudaError_t tc_gemm(const TcGemm &g, cudaStream_t st)
-{
-    auto kern = tc_gemm_kernel<AT, BT, BBF16, ATOMIC>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGSmemReq);
-    if (e != cudaSuccess) return e;
-    const int slabs = (g.K + g.k_slab - 1) / g.k_slab;
-    const dim3 grid((unsigned)((g.M + kGM - 1) / kGM), (unsigned)((g.N + kGN - 1) / kGN), (unsigned)slabs);
-    kern<<<grid, kTcThreads, kGSmemReq, st>>>(g);
-    return cudaGetLastError();
 }
 
 }  // namespace
@@ -751,44 +834,13 @@ static cudaError_t layer1(const MlpLayer1Args &l1, int sm_count, cudaStream_t st
 cudaError_t mlp_layer1_tc(const MlpLayer1Args &l1, int sm_count, cudaStream_t st) { return layer1<false>(l1, sm_count, st); }
 cudaError_t mlp_layer1_bwd_tc(const MlpLayer1Args &l1, int sm_count, cudaStream_t st) { return layer1<true>(l1, sm_count, st); }
 
-// dZ (T x 256) = dU (T x 256) W2[:, 0..255]: A = dU, B(n, k) = W2[k][n] (the
-// tour length has no gradient to pass on).
-cudaError_t mlp_grad_zt_tc(const float *dU, int T, const __nv_bfloat16 *w2, float *dzt, unsigned int *err,
-                           cudaStream_t st)
+cudaError_t mlp_grad(const MlpGradArgs &g, cudaStream_t st)
 {
-    TcGemm g{};
-    g.a = dU;
-    g.lda = kMlpH;
-    g.bh = w2;
-    g.ldb = kMlpIn2;
-    g.M = T;
-    g.N = kMlpH;
-    g.K = kMlpH;
-    g.k_slab = kMlpH;
-    g.out = dzt;
-    g.ldo = kMlpH;
-    g.err = err;
-    return tc_gemm<false, true, true, false>(g, st);
-}
-
-// gW2 (256 x 257) += dU^T (256 x T) ZT (T x 257): A(m, k) = dU[k][m],
-// B(n, k) = ZT[k][n]; split-K over slabs of 128 tours (a CTA per slab and
-// tile fills the GPU), added atomically.
-cudaError_t mlp_grad_w2_tc(const float *dU, const float *zt, int T, float *gw2, unsigned int *err, cudaStream_t st)
-{
-    TcGemm g{};
-    g.a = dU;
-    g.lda = kMlpH;
-    g.bf = zt;
-    g.ldb = kMlpIn2;
-    g.M = kMlpH;
-    g.N = kMlpIn2;
-    g.K = T;
-    g.k_slab = 128;
-    g.out = gw2;
-    g.ldo = kMlpIn2;
-    g.err = err;
-    return tc_gemm<true, true, false, true>(g, st);
+    cudaError_t e = cudaFuncSetAttribute(mlp_grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGSmem);
+    if (e != cudaSuccess) return e;
+    const long long slabs = ((long long)g.T + kGM - 1) / kGM;
+    mlp_grad_kernel<<<(unsigned)(slabs * (kMlpH / kGNz + 2 * kGwTiles)), kTcThreads, kGSmem, st>>>(g);
+    return cudaGetLastError();
 }
 
 }  // namespace cvrpsd

@@ -259,7 +259,7 @@ struct cvrpsd_surrogate {
     unsigned char *ws_infer = nullptr;
     float *ws_train = nullptr;
     long long cap_infer = 0, cap_train = 0;   // rows
-    float *d_zt = nullptr, *d_U = nullptr, *d_y = nullptr, *d_dy = nullptr, *d_dU = nullptr, *d_dzt = nullptr;
+    float *d_zt = nullptr, *d_U = nullptr, *d_y = nullptr, *d_dy = nullptr, *d_dzt = nullptr;
     float *d_loss = nullptr;
     unsigned int *d_err = nullptr;  // set by a tensor-core kernel whose wait gave up
     int step = 0;
@@ -297,11 +297,10 @@ int sur_workspace(cvrpsd_surrogate *s, long long T, bool train)
         if (s->ws_train) cudaFree(s->ws_train);
         s->ws_train = nullptr;
         // the rows that are written four floats at a time come first
-        CK(dev_alloc(ctx, &s->ws_train, sizeof(float) * T * (3 * kMlpH + kMlpIn2 + 2)), "surrogate workspace");
+        CK(dev_alloc(ctx, &s->ws_train, sizeof(float) * T * (2 * kMlpH + kMlpIn2 + 2)), "surrogate workspace");
         s->cap_train = T;
         s->d_U = s->ws_train;
-        s->d_dU = s->d_U + T * kMlpH;
-        s->d_dzt = s->d_dU + T * kMlpH;
+        s->d_dzt = s->d_U + T * kMlpH;
         s->d_zt = s->d_dzt + T * kMlpH;
         s->d_y = s->d_zt + T * kMlpIn2;
         s->d_dy = s->d_y + T;
@@ -471,11 +470,11 @@ static int sur_grad(cvrpsd_surrogate *s, const int32_t *d_tours, int32_t T, cons
 {
     cvrpsd_ctx *ctx = s->ctx;
     CK(cudaMemsetAsync(s->d_g, 0, sizeof(float) * kMlpParams, st), "clear gradient");
-    CK(cudaMemsetAsync(s->d_loss, 0, sizeof(float), st), "clear loss");
-    const MlpLayer1Args l1 = layer1_of(s, d_tours, T);
+    MlpLayer1Args l1 = layer1_of(s, d_tours, T);
+    l1.loss = s->d_loss;
     const MlpWeights w = weights_of(s);
     CK(mlp_forward(l1, w, s->d_U, s->d_y, d_target, s->d_dy, s->d_loss, st), "surrogate forward");
-    CK(mlp_backward(l1, w, s->d_U, s->d_dy, s->d_dU, s->d_dzt, s->d_g, st), "surrogate backward");
+    CK(mlp_backward(l1, w, s->d_U, s->d_dy, s->d_dzt, s->d_g, st), "surrogate backward");
     return CVRPSD_OK;
 }
 
