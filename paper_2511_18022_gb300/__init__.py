@@ -38,8 +38,10 @@ def _i32(a) -> np.ndarray:
 
 def _stream_ptr(stream):
     if stream is None:
+        # the raw handle: building a Stream object around it takes 3 us of a
+        # 40 us call
         import torch
-        return torch.cuda.current_stream().cuda_stream
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream

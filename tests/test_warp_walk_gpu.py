@@ -97,3 +97,11 @@ def test_pairs_and_lone_warps(cv, more, n, Q, dtype):
 @pytest.mark.parametrize("n,S", [(2999, 48), (3000, 48), (3000, 49)])
 def test_automatic_choice_of_long_tours_is_exact(cv, n, S):
     test_automatic_choice_is_exact(cv, n, S)
+
+
+def test_calls_without_a_stream_take_the_current_one(cv):
+    s = torch.cuda.Stream()
+    assert cv._stream_ptr(None) == torch.cuda.current_stream().cuda_stream
+    with torch.cuda.stream(s):
+        assert cv._stream_ptr(None) == s.cuda_stream
+    assert cv._stream_ptr(s) == s.cuda_stream and cv._stream_ptr(7) == 7
