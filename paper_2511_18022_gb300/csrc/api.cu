@@ -609,14 +609,33 @@ launched:
     if (one_launch && a[ACC_OVERFLOW]) {
         if (param_walk) CK(upload_table(), "upload tour table");
         if (timed) CK(cudaEventRecord(ctx->ev_t[1], stream), "cudaEventRecord");
-        CK(aside_pass(), "split_warp (set-aside scenarios) launch");
+        const auto read_totals = [&]() {
+            return cudaMemcpyAsync(a, p.acc, ACC_ALLOC_WORDS * sizeof(unsigned long long), cudaMemcpyDeviceToHost, stream);
+        };
+        // A long list left by rings of 16 or 8 goes to rings of 32, one thread
+        // per scenario: one walk's latency and a twelfth of the warp kernel's
+        // time per scenario (n = 1000: 26 ns). Whole calls, n = 200: 39,108
+        // listed 646 us by warps, 529 by threads; 19,737 396, 349; they meet
+        // near 12,000.
+        bool warps = true;
+        ctx->stats.launches = 1;
+        if (a[ACC_OVERFLOW] >= 16384 && kernel == CVRPSD_KERNEL_DEQUE && !pred && st.ring < 32) {
+            p.done = nullptr;
+            CK(launch_split_list(p, (long long)a[ACC_OVERFLOW], demand_dtype, stream), "split_list launch");
+            CK(read_totals(), "read accumulators");
+            CK(cudaStreamSynchronize(stream), "cudaStreamSynchronize");
+            warps = a[ACC_TICKET] != 0;
+            ++ctx->stats.launches;
+        }
+        if (warps) {
+            CK(aside_pass(), "split_warp (set-aside scenarios) launch");
+            CK(read_totals(), "read accumulators");
+            ++ctx->stats.launches;
+        }
         if (timed) CK(cudaEventRecord(ctx->ev_t[2], stream), "cudaEventRecord");
-        CK(cudaMemcpyAsync(a, p.acc, ACC_WORDS * sizeof(unsigned long long), cudaMemcpyDeviceToHost, stream),
-           "read accumulators");
         CK(cudaMemsetAsync(p.acc, 0, ACC_ALLOC_WORDS * sizeof(unsigned long long), stream), "clear accumulators");
         CK(cudaStreamSynchronize(stream), "cudaStreamSynchronize");
         ctx->tab_use = cvrpsd_ctx::TAB_FREE;
-        ctx->stats.launches = 2;
         fallback_launched = true;
     }
     if (one_launch) ctx->acc_dirty = false;

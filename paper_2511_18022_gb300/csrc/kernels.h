@@ -83,6 +83,14 @@ cudaError_t launch_split_deque_i16_nocap(const SplitParams &p, const DequeShape 
 cudaError_t launch_split_deque_i32_cap(const SplitParams &p, const DequeShape &s, cudaStream_t st);
 cudaError_t launch_split_deque_i32_nocap(const SplitParams &p, const DequeShape &s, cudaStream_t st);
 
+// The scenarios of p.ovf_list (count of them, known to the host) by rings of 32;
+// entries that are settled become -1, and ACC_TICKET (0 before) counts the others.
+cudaError_t launch_split_list(const SplitParams &p, long long count, int esize, cudaStream_t stream);
+cudaError_t launch_split_list_i16_cap(const SplitParams &p, long long count, cudaStream_t st);
+cudaError_t launch_split_list_i16_nocap(const SplitParams &p, long long count, cudaStream_t st);
+cudaError_t launch_split_list_i32_cap(const SplitParams &p, long long count, cudaStream_t st);
+cudaError_t launch_split_list_i32_nocap(const SplitParams &p, long long count, cudaStream_t st);
+
 // The same walk for scenarios in page-locked host memory (device addresses of
 // it in p): 1 KB windows of the rows staged through shared memory, rings of 16.
 cudaError_t launch_split_host(const SplitParams &p, int esize, cudaStream_t stream);

@@ -44,7 +44,7 @@ __global__ void __launch_bounds__(T) split_batch_kernel(BatchParams b)
         const long long cap = b.list_cap;
         long long sum = split_thread<DT, SPT, R, T, LCAP>(
             td.demand, td.ld, b.S, s_first, td.n, td.Q, td.L, td.K, td.g0, sbase, tabref, tid, td.out_cost,
-            [acc, list, cap, t](long long s) {
+            [acc, list, cap, t](long long s, uint32_t) {
                 const unsigned long long idx = atomicAdd(acc + BACC_LIST, 1ull);
                 if ((long long)idx < cap) list[idx] = make_int2(t, (int)s);
                 else atomicOr(acc + BACC_STATUS, (unsigned long long)BST_LIST_FULL);

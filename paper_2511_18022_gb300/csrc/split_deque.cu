@@ -50,22 +50,37 @@ static cudaError_t launch_host(const SplitParams &p, cudaStream_t stream)
     return cudaGetLastError();
 }
 
+template <typename DT, bool LCAP>
+static cudaError_t launch_list(const SplitParams &p, long long count, cudaStream_t stream)
+{
+    split_list_kernel<DT, LCAP><<<(unsigned)((count + kListThreads - 1) / kListThreads), kListThreads, 0, stream>>>(p, count);
+    return cudaGetLastError();
+}
+
 #if CVRPSD_DEQUE_PART == 0
 cudaError_t launch_split_deque_i16_cap(const SplitParams &p, const DequeShape &s, cudaStream_t st)
 { return dispatch_shape<int16_t, true>(p, s, st); }
 cudaError_t launch_split_host_i16_cap(const SplitParams &p, cudaStream_t st) { return launch_host<int16_t, true>(p, st); }
+cudaError_t launch_split_list_i16_cap(const SplitParams &p, long long count, cudaStream_t st)
+{ return launch_list<int16_t, true>(p, count, st); }
 #elif CVRPSD_DEQUE_PART == 1
 cudaError_t launch_split_deque_i16_nocap(const SplitParams &p, const DequeShape &s, cudaStream_t st)
 { return dispatch_shape<int16_t, false>(p, s, st); }
 cudaError_t launch_split_host_i16_nocap(const SplitParams &p, cudaStream_t st) { return launch_host<int16_t, false>(p, st); }
+cudaError_t launch_split_list_i16_nocap(const SplitParams &p, long long count, cudaStream_t st)
+{ return launch_list<int16_t, false>(p, count, st); }
 #elif CVRPSD_DEQUE_PART == 2
 cudaError_t launch_split_deque_i32_cap(const SplitParams &p, const DequeShape &s, cudaStream_t st)
 { return dispatch_shape<int32_t, true>(p, s, st); }
 cudaError_t launch_split_host_i32_cap(const SplitParams &p, cudaStream_t st) { return launch_host<int32_t, true>(p, st); }
+cudaError_t launch_split_list_i32_cap(const SplitParams &p, long long count, cudaStream_t st)
+{ return launch_list<int32_t, true>(p, count, st); }
 #elif CVRPSD_DEQUE_PART == 3
 cudaError_t launch_split_deque_i32_nocap(const SplitParams &p, const DequeShape &s, cudaStream_t st)
 { return dispatch_shape<int32_t, false>(p, s, st); }
 cudaError_t launch_split_host_i32_nocap(const SplitParams &p, cudaStream_t st) { return launch_host<int32_t, false>(p, st); }
+cudaError_t launch_split_list_i32_nocap(const SplitParams &p, long long count, cudaStream_t st)
+{ return launch_list<int32_t, false>(p, count, st); }
 #endif
 
 }  // namespace cvrpsd

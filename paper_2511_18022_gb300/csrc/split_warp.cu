@@ -297,6 +297,7 @@ __global__ void __launch_bounds__(128) split_warp_kernel(SplitParams p, const in
     for (long long item = (long long)blockIdx.x * wpb + w; item < total;
          item += (long long)gridDim.x * wpb) {
         const long long s = list ? (long long)list[item] : item;
+        if (list && s < 0) continue;                         // settled by split_list_kernel (warp-uniform)
         if (!index_ok(s >= 0 && s < p.S, p.acc + ACC_STATUS)) continue;   // warp-uniform
         WarpResult r{};
         r.wide = true;
@@ -526,6 +527,13 @@ cudaError_t launch_split_host(const SplitParams &p, int esize, cudaStream_t stre
     const bool cap = p.L < p.n;
     if (esize == 2) return cap ? launch_split_host_i16_cap(p, stream) : launch_split_host_i16_nocap(p, stream);
     return cap ? launch_split_host_i32_cap(p, stream) : launch_split_host_i32_nocap(p, stream);
+}
+
+cudaError_t launch_split_list(const SplitParams &p, long long count, int esize, cudaStream_t stream)
+{
+    const bool cap = p.L < p.n;
+    if (esize == 2) return cap ? launch_split_list_i16_cap(p, count, stream) : launch_split_list_i16_nocap(p, count, stream);
+    return cap ? launch_split_list_i32_cap(p, count, stream) : launch_split_list_i32_nocap(p, count, stream);
 }
 
 }  // namespace cvrpsd
