@@ -216,6 +216,27 @@ __device__ __forceinline__ WarpResult warp_walk_scenario(const TourStep *__restr
     return r;
 }
 
+// A set-aside scenario with the calling (full) warp: a demand above Q, which
+// takes no walk, is looked for first, with its loads in flight together (n = 200,
+// 108,613 of 120,000 infeasible: 451 -> 267 us per call; 3 % more where a batch
+// sets many feasible ones aside, 1529 -> 1575 us).
+template <typename DT>
+__device__ __forceinline__ WarpResult warp_aside_scenario(const TourStep *__restrict__ tab, int n, int Q, int L, int g0,
+                                                          const DT *__restrict__ dem, long long ld, long long s,
+                                                          WalkSmem &w, unsigned long long *status)
+{
+    bool neg = false, bad = false;
+#pragma unroll 4
+    for (int i = threadIdx.x & 31; i < n; i += 32) {
+        const int row = tab[i].row & kRowMask;
+        const int q = index_ok(row < n && s >= 0 && s < ld, status) ? (int)__ldg(dem + (long long)row * ld + s) : 0;
+        neg |= q < 0;
+        bad |= q > Q;
+    }
+    if (__any_sync(0xffffffffu, bad)) return WarpResult{INT32_MAX, true, (bool)__any_sync(0xffffffffu, neg), false};
+    return warp_walk_scenario<DT>(tab, n, Q, L, g0, dem, ld, s, w, status);
+}
+
 // Evaluates scenario s of one tour with the calling (full) warp. P and g are
 // this warp's shared arrays of n + 1 ints each.
 template <typename DT>
@@ -301,7 +322,7 @@ __global__ void __launch_bounds__(128) split_warp_kernel(SplitParams p, const in
         if (!index_ok(s >= 0 && s < p.S, p.acc + ACC_STATUS)) continue;   // warp-uniform
         WarpResult r{};
         r.wide = true;
-        if (!p.pred) r = warp_walk_scenario<DT>(p.tab, n, p.Q, p.L, p.g0, dem, p.ld, s, s_walk[w], p.acc + ACC_STATUS);
+        if (!p.pred) r = warp_aside_scenario<DT>(p.tab, n, p.Q, p.L, p.g0, dem, p.ld, s, s_walk[w], p.acc + ACC_STATUS);
         if (r.wide)
             r = warp_split_scenario<DT>(p.tab, n, p.Q, p.L, p.g0, dem, p.ld, s, P, g, p.acc + ACC_STATUS, p.pred,
                                         p.ldp);
@@ -452,8 +473,8 @@ __global__ void __launch_bounds__(128) split_warp_batch_kernel(BatchParams b)
         if (!index_ok(e.x >= 0 && e.y >= 0 && e.y < b.S, b.acc + BACC_STATUS)) continue;   // warp-uniform
         const TourDev td = b.tours[e.x];
         const DT *dem = reinterpret_cast<const DT *>(td.demand);
-        WarpResult r = warp_walk_scenario<DT>(td.tab, td.n, td.Q, td.L, td.g0, dem, td.ld, e.y, s_walk[w],
-                                              b.acc + BACC_STATUS);
+        WarpResult r = warp_aside_scenario<DT>(td.tab, td.n, td.Q, td.L, td.g0, dem, td.ld, e.y, s_walk[w],
+                                               b.acc + BACC_STATUS);
         if (r.wide)
             r = warp_split_scenario<DT>(td.tab, td.n, td.Q, td.L, td.g0, dem, td.ld, e.y, P, g, b.acc + BACC_STATUS);
         if (lane == 0) {
