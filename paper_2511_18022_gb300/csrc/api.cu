@@ -1053,7 +1053,7 @@ int cvrpsd_batch_create(cvrpsd_ctx *ctx, int32_t T, const cvrpsd_tour_desc *tour
         smooth += smooth_table(rises, hd[t].n);
     }
     bp.smooth = 2 * smooth > T;
-    bp.walk2 = demand_dtype == CVRPSD_I16;
+    bp.walk2 = 1;
     for (int t = 0; t < T; ++t) bp.walk2 &= batch2_keys_fit(hd[t].n, hd[t].Q, hd[t].K);
     int per_sm = 0;
     BK(launch_split_batch(bp, demand_dtype, lcap, shape, 0, true, &per_sm, nullptr), "configure batch kernel");

@@ -146,7 +146,7 @@ struct BatchParams {
     int2 *list;                   // device [list_cap]: set-aside (tour, scenario)
     long long list_cap;
     int max_n;                    // largest tour
-    int walk2;                    // int16 demands and keys that cannot wrap in every tour: the
+    int walk2;                    // keys that cannot wrap in every tour (and 32-bit pitches): the
                                   // second walk runs the one-scenario-per-thread shapes
     int T;                        // tours
     int smooth;                   // second walk: 1 if most tours are smooth (smooth_table), 0 if not, -1 if only
@@ -190,13 +190,20 @@ cudaError_t launch_split_batch(const BatchParams &b, int esize, bool lcap, const
 // The batch kernel on the second walk (split_batch2.cu), which
 // launch_split_batch picks where b.walk2 is set and the shape has one
 // scenario per thread.
-bool batch2_shape_compiled(const DequeShape &s);
+bool batch2_shape_compiled(const DequeShape &s, int esize);
+cudaError_t launch_split_batch2(const BatchParams &b, int esize, bool lcap, const DequeShape &shape, int grid,
+                                bool configure_only, int *blocks_per_sm, cudaStream_t stream);
 cudaError_t launch_split_batch2_cap(const BatchParams &b, const DequeShape &shape, int grid, bool configure_only,
                                     int *blocks_per_sm, cudaStream_t stream);
 cudaError_t launch_split_batch2_nocap(const BatchParams &b, const DequeShape &shape, int grid, bool configure_only,
                                       int *blocks_per_sm, cudaStream_t stream);
-// Whether every key K (P + Q) + p of an int16 walk stays below 2^31 (demands
-// read unclamped: one bad demand may add up to 65535 before the walk freezes).
+cudaError_t launch_split_batch2_i32_cap(const BatchParams &b, const DequeShape &shape, int grid, bool configure_only,
+                                        int *blocks_per_sm, cudaStream_t stream);
+cudaError_t launch_split_batch2_i32_nocap(const BatchParams &b, const DequeShape &shape, int grid, bool configure_only,
+                                          int *blocks_per_sm, cudaStream_t stream);
+// Whether every key K (P + Q) + p of a walk stays below 2^31 (int16 demands are
+// read unclamped: one bad demand may add up to 65535 before the walk freezes;
+// int32 ones add Q at most).
 inline bool batch2_keys_fit(long long n, long long Q, long long K)
 {
     return K * (n * Q + 65535 + Q) + n < (1LL << 31);

@@ -8,15 +8,16 @@
 // bits and a vote-free first back step. The table differs from the
 // single-tour walk's only in where it lives: shared memory instead of the
 // launch parameters, with the skip bit and the block flag derived while it
-// is copied. One scenario per thread, int16 demands, rings of 16 or more,
-// keys that cannot wrap (the host checks every tour).
+// is copied. One scenario per thread, rings of 16 or more,
+// keys that cannot wrap (the host checks every tour). int32 demands keep the
+// second walk's clamp and running maximum.
 #include "split_deque2.cuh"
 
 namespace cvrpsd {
 
 // The tour's table in shared memory: the demand rows of its positions, their
 // C_i, both up to the next multiple of 4 (the last row and 0 again), so that a
-// prefetch block of 4 positions reads each in one load (1124 -> 1068 us for 64
+// prefetch block of 4 positions reads each in one load (1084 -> 1048 us for 64
 // tours of n = 200 under 65,536 scenarios against pairs read per position); and
 // a word of flags for every span of two prefetch blocks (8 positions): bit u
 // where no scenario can pop the back at the span's position u (kTab2NoBack of
@@ -78,7 +79,7 @@ constexpr int b2_min_blocks()
 // under 8192 scenarios 434 -> 443 us; out of line worse). Where the host has
 // the tables it launches one of the two; where they were built on the device
 // both are launched and the blocks of the one that does not apply exit.
-template <int R, int T, bool LCAP, bool SMOOTH>
+template <typename DT, int R, int T, bool LCAP, bool SMOOTH>
 __global__ void __launch_bounds__(T, b2_min_blocks<R, T>()) split_batch2_kernel(BatchParams b)
 {
     if (b.smooth < 0 && (2 * b.acc[BACC_SMOOTH] > (unsigned long long)b.T) != SMOOTH) return;
@@ -135,11 +136,11 @@ __global__ void __launch_bounds__(T, b2_min_blocks<R, T>()) split_batch2_kernel(
         p.L = (int)uniform((uint32_t)td.L);
         p.g0 = td.g0;
         p.K = uniform(td.K);
-        p.pitch = uniform((uint32_t)(td.ld * 2));
+        p.pitch = uniform((uint32_t)(td.ld * (int)sizeof(DT)));
         p.status = status;
         const long long s = (long long)it.y * T + tid;
         bool aside = false;
-        const int c = walk2_scenario<int16_t, R, T, LCAP, true, SMOOTH>(p, tab, s, rs, (uint32_t)tid * 8u, aside);
+        const int c = walk2_scenario<DT, R, T, LCAP, true, SMOOTH>(p, tab, s, rs, (uint32_t)tid * 8u, aside);
         long long sum = 0;
         if (s < b.S) {
             if (aside) {
@@ -164,11 +165,11 @@ __global__ void __launch_bounds__(T, b2_min_blocks<R, T>()) split_batch2_kernel(
     }
 }
 
-template <int R, int T, bool LCAP, bool SMOOTH>
+template <typename DT, int R, int T, bool LCAP, bool SMOOTH>
 static cudaError_t launch2_one(const BatchParams &b, const DequeShape &shape, int grid, bool configure_only,
                                int *blocks_per_sm, cudaStream_t stream)
 {
-    auto kern = split_batch2_kernel<R, T, LCAP, SMOOTH>;
+    auto kern = split_batch2_kernel<DT, R, T, LCAP, SMOOTH>;
     const size_t smem = split_batch_smem(b.max_n, shape);
     if (configure_only) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -185,7 +186,11 @@ static cudaError_t launch2_one(const BatchParams &b, const DequeShape &shape, in
     X(32, 16) X(32, 32) X(32, 64) X(64, 16) X(64, 32) X(64, 64) X(128, 16) X(128, 32)            \
     X(128, 64) X(256, 16) X(256, 32) X(512, 16)
 
-template <bool LCAP>
+// 32-bit demands: the library's own shapes (64 tours of n = 200 under 65,536
+// scenarios 1451 us by the first walk, 1152; in strips 1703, 1553).
+#define CVRPSD_BATCH2_SHAPES_I32(X) X(64, 16) X(128, 16) X(256, 16) X(512, 16)
+
+template <typename DT, bool LCAP>
 static cudaError_t dispatch2(BatchParams b, const DequeShape &s, int grid, bool configure_only,
                              int *blocks_per_sm, cudaStream_t st)
 {
@@ -193,39 +198,69 @@ static cudaError_t dispatch2(BatchParams b, const DequeShape &s, int grid, bool 
     // one a tuner picks.
     if (b.smooth != 0 && s.spt == 1 && s.ring == 16 && (s.threads == 256 || s.threads == 512)) {
         const cudaError_t e = s.threads == 256
-            ? launch2_one<16, 256, LCAP, true>(b, s, grid, configure_only, blocks_per_sm, st)
-            : launch2_one<16, 512, LCAP, true>(b, s, grid, configure_only, blocks_per_sm, st);
+            ? launch2_one<DT, 16, 256, LCAP, true>(b, s, grid, configure_only, blocks_per_sm, st)
+            : launch2_one<DT, 16, 512, LCAP, true>(b, s, grid, configure_only, blocks_per_sm, st);
         if (e != cudaSuccess || b.smooth > 0) return e;
     } else {
         b.smooth = 0;
     }
 #define CVRPSD_CASE(T_, R_)                                                            \
     if (s.threads == T_ && s.spt == 1 && s.ring == R_)                                \
-        return launch2_one<R_, T_, LCAP, false>(b, s, grid, configure_only, blocks_per_sm, st);
-    CVRPSD_BATCH2_SHAPES(CVRPSD_CASE)
+        return launch2_one<DT, R_, T_, LCAP, false>(b, s, grid, configure_only, blocks_per_sm, st);
+    if constexpr (sizeof(DT) == 2) {
+        CVRPSD_BATCH2_SHAPES(CVRPSD_CASE)
+    } else {
+        CVRPSD_BATCH2_SHAPES_I32(CVRPSD_CASE)
+    }
 #undef CVRPSD_CASE
     return cudaErrorInvalidValue;
 }
 
 #if CVRPSD_BATCH2_PART == 0
-bool batch2_shape_compiled(const DequeShape &s)
+bool batch2_shape_compiled(const DequeShape &s, int esize)
 {
 #define CVRPSD_CASE(T_, R_) if (s.threads == T_ && s.spt == 1 && s.ring == R_) return true;
-    CVRPSD_BATCH2_SHAPES(CVRPSD_CASE)
+    if (esize == 2) {
+        CVRPSD_BATCH2_SHAPES(CVRPSD_CASE)
+    } else {
+        CVRPSD_BATCH2_SHAPES_I32(CVRPSD_CASE)
+    }
 #undef CVRPSD_CASE
     return false;
+}
+
+cudaError_t launch_split_batch2(const BatchParams &b, int esize, bool lcap, const DequeShape &shape, int grid,
+                                bool configure_only, int *blocks_per_sm, cudaStream_t stream)
+{
+    if (esize == 2)
+        return lcap ? launch_split_batch2_cap(b, shape, grid, configure_only, blocks_per_sm, stream)
+                    : launch_split_batch2_nocap(b, shape, grid, configure_only, blocks_per_sm, stream);
+    return lcap ? launch_split_batch2_i32_cap(b, shape, grid, configure_only, blocks_per_sm, stream)
+                : launch_split_batch2_i32_nocap(b, shape, grid, configure_only, blocks_per_sm, stream);
 }
 
 cudaError_t launch_split_batch2_cap(const BatchParams &b, const DequeShape &shape, int grid, bool configure_only,
                                     int *blocks_per_sm, cudaStream_t stream)
 {
-    return dispatch2<true>(b, shape, grid, configure_only, blocks_per_sm, stream);
+    return dispatch2<int16_t, true>(b, shape, grid, configure_only, blocks_per_sm, stream);
 }
-#else
+#elif CVRPSD_BATCH2_PART == 1
 cudaError_t launch_split_batch2_nocap(const BatchParams &b, const DequeShape &shape, int grid, bool configure_only,
                                       int *blocks_per_sm, cudaStream_t stream)
 {
-    return dispatch2<false>(b, shape, grid, configure_only, blocks_per_sm, stream);
+    return dispatch2<int16_t, false>(b, shape, grid, configure_only, blocks_per_sm, stream);
+}
+#elif CVRPSD_BATCH2_PART == 2
+cudaError_t launch_split_batch2_i32_cap(const BatchParams &b, const DequeShape &shape, int grid, bool configure_only,
+                                        int *blocks_per_sm, cudaStream_t stream)
+{
+    return dispatch2<int32_t, true>(b, shape, grid, configure_only, blocks_per_sm, stream);
+}
+#else
+cudaError_t launch_split_batch2_i32_nocap(const BatchParams &b, const DequeShape &shape, int grid, bool configure_only,
+                                          int *blocks_per_sm, cudaStream_t stream)
+{
+    return dispatch2<int32_t, false>(b, shape, grid, configure_only, blocks_per_sm, stream);
 }
 #endif
 
