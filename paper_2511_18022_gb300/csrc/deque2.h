@@ -45,7 +45,6 @@ struct TabParam {
     static constexpr int kCap = CAP;
 #ifdef __CUDACC__
     // The walk's view of a table (see TabShared2 for the batch kernel's).
-    __device__ __forceinline__ uint2 entry(int i) const { return e[i - 1]; }
     __device__ __forceinline__ uint32_t row(int i) const { return e[i - 1].x & kTab2RowMask; }
     // Flags of the span of two prefetch blocks from i0: read where they are used.
     __device__ __forceinline__ uint32_t span(int i0) const { return 0; }
