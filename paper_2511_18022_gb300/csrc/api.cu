@@ -449,7 +449,7 @@ int split_eval_impl(cvrpsd_ctx *ctx, const int32_t *tour, int32_t n, const int32
     st.kernel_ms = st.fallback_ms = -1.0f;
     const bool timed = ctx->profiling && (out_sum || out_infeasible || out_mean || host_buffers) && S > 0;
     bool fallback_launched = false;
-    const int warp_grid = 2 * (ctx->sm_count > 0 ? ctx->sm_count : 152);
+    const int warp_grid = kAsideBlocks * (ctx->sm_count > 0 ? ctx->sm_count : 152);
     const auto aside_pass = [&]() {
         return launch_split_warp(p, demand_dtype, p.ovf_list, p.acc + ACC_OVERFLOW, warp_grid, ctx->max_smem, stream);
     };
@@ -506,7 +506,7 @@ int split_eval_impl(cvrpsd_ctx *ctx, const int32_t *tour, int32_t n, const int32
             st.launches = 1;
         } else if (kernel == CVRPSD_KERNEL_WARP) {
             long long need = (S + 3) / 4;
-            const int grid = (int)(need < 8LL * warp_grid ? need : 8LL * warp_grid);
+            const int grid = (int)(need < 2LL * warp_grid ? need : 2LL * warp_grid);
             if (timed) CK(cudaEventRecord(ctx->ev_t[0], stream), "cudaEventRecord");
             CK(launch_split_warp(p, demand_dtype, nullptr, nullptr, grid, ctx->max_smem, stream),
                "split_warp launch");
@@ -1059,7 +1059,7 @@ int cvrpsd_batch_create(cvrpsd_ctx *ctx, int32_t T, const cvrpsd_tour_desc *tour
     BK(launch_split_batch(bp, demand_dtype, lcap, shape, 0, true, &per_sm, nullptr), "configure batch kernel");
     if (per_sm < 1) per_sm = 1;
     const int grid = ctx->sm_count * per_sm;
-    const int warp_grid = 2 * ctx->sm_count;
+    const int warp_grid = kAsideBlocks * ctx->sm_count;
     BK(launch_split_warp_batch(bp, demand_dtype, warp_grid, ctx->max_smem, true, nullptr), "configure warp kernel");
 
     BK(cudaStreamCreateWithFlags(&b->cap_stream, cudaStreamNonBlocking), "cudaStreamCreate");

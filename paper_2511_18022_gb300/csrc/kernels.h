@@ -106,6 +106,12 @@ inline size_t split_deque_smem(const SplitParams &p, const DequeShape &shape)
     return (size_t)shape.spt * shape.ring * shape.threads * 8;
 }
 
+// Blocks per SM of the pass over set-aside scenarios (four warps each; its
+// registers and tours of a few hundred positions let eight be resident). 64
+// tours of n = 200 in strips under 65,536 scenarios, many set aside: two blocks
+// 2579 us, four 2145, eight 2024; none set aside: 0.3 us more to start them.
+constexpr int kAsideBlocks = 8;
+
 // Warp-per-scenario kernel. If `list` is non-null it evaluates the scenarios
 // named in list[0 .. *count) (count lives on the device); otherwise all S.
 // `max_smem` is the device's opt-in shared memory per block.

@@ -164,8 +164,8 @@ int cvrpsd_split_eval_tours(cvrpsd_ctx *ctx, const int32_t *d_tours, int32_t T, 
     CK(launch_split_batch(bp, demand_dtype, L < n, shape, ctx->sm_count * (per_sm > 0 ? per_sm : 1), false, nullptr,
                           stream),
        "split kernel");
-    CK(launch_split_warp_batch(bp, demand_dtype, 2 * ctx->sm_count, ctx->max_smem, true, stream), "configure warp");
-    CK(launch_split_warp_batch(bp, demand_dtype, 2 * ctx->sm_count, ctx->max_smem, false, stream), "warp kernel");
+    CK(launch_split_warp_batch(bp, demand_dtype, kAsideBlocks * ctx->sm_count, ctx->max_smem, true, stream), "configure warp");
+    CK(launch_split_warp_batch(bp, demand_dtype, kAsideBlocks * ctx->sm_count, ctx->max_smem, false, stream), "warp kernel");
     CK(launch_tour_means(ctx->mt_acc, T, S, d_mean, reinterpret_cast<long long *>(d_sum),
                          reinterpret_cast<long long *>(d_infeasible), stream),
        "tour means");
