@@ -1,8 +1,7 @@
 """The surrogate's kernels at the edges of their tiles (128 positions per stage
-and 32 per step in layer 1, 128 tours per head tile, 16 rows per block of the
-output layer's gradient, 96 x 128 tiles of the other gradients; more tours than
-two lines of 152 CTAs take in one turn), against the FP64 reference with the
-tolerances of the other surrogate tests."""
+and 32 per step in layer 1, 128 tours per head tile and per slab of the gradient
+kernel; more tours than two lines of 152 CTAs take in one turn), against the
+FP64 reference with the tolerances of the other surrogate tests."""
 import numpy as np
 import pytest
 
