@@ -192,7 +192,9 @@ int cvrpsd_debug_fail_alloc(cvrpsd_ctx *ctx, int32_t after);
  *  stream                  cudaStream_t.
  *
  * If any host output is requested the call waits for `stream` to finish its
- * work; otherwise it returns once the work is enqueued. Rejects device
+ * work; otherwise it returns once the work is enqueued (recorded into a CUDA
+ * graph, with the tour as it is now, where `stream` is being captured and the
+ * context has split as many scenarios before). Rejects device
  * buffers too small for [n][ld] / [S] with CVRPSD_ERR_ARG, and inputs whose
  * costs could overflow int32 with CVRPSD_ERR_OVERFLOW.
  */

@@ -432,7 +432,13 @@ int split_eval_impl(cvrpsd_ctx *ctx, const int32_t *tour, int32_t n, const int32
     } else {
         CK(cudaMemsetAsync(ctx->d_acc, 0, ACC_WORDS * sizeof(unsigned long long), stream), "clear accumulators");
     }
+    // Into a graph the table goes by value: a recorded copy would read the
+    // pinned table when the graph runs, after later calls have changed it, and
+    // an event recorded there could not be waited for by them.
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (!want_host && cudaStreamIsCapturing(stream, &capture) != cudaSuccess) cudaGetLastError();
     const auto upload_table = [&]() {
+        if (capture != cudaStreamCaptureStatusNone) return launch_store_table(ctx->h_tab, n, ctx->d_tab, stream);
         ctx->tab_use = cvrpsd_ctx::TAB_UNKNOWN;
         cudaError_t e = cudaMemcpyAsync(ctx->d_tab, ctx->h_tab, (size_t)n * sizeof(TourStep), cudaMemcpyHostToDevice,
                                         stream);

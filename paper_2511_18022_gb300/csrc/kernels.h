@@ -99,6 +99,10 @@ cudaError_t launch_split_host_i16_nocap(const SplitParams &p, cudaStream_t st);
 cudaError_t launch_split_host_i32_cap(const SplitParams &p, cudaStream_t st);
 cudaError_t launch_split_host_i32_nocap(const SplitParams &p, cudaStream_t st);
 
+// Writes a tour table of n entries to d_tab, from the launches' own parameters:
+// `tab` is free again when this returns, also under stream capture.
+cudaError_t launch_store_table(const TourStep *tab, int n, TourStep *d_tab, cudaStream_t stream);
+
 // Dynamic shared memory of the deque kernel: its rings ([spt][ring][threads] int2).
 inline size_t split_deque_smem(const SplitParams &p, const DequeShape &shape)
 {

@@ -533,6 +533,29 @@ cudaError_t launch_split_warp_batch(const BatchParams &b, int esize, int grid_ct
     return cudaGetLastError();
 }
 
+// A part of a tour table as a launch's parameters (at most 32764 bytes).
+constexpr int kTabPart = 2040;
+struct TabPart {
+    TourStep e[kTabPart];
+};
+
+__global__ void store_table_kernel(const __grid_constant__ TabPart part, TourStep *out, int count)
+{
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k < count) out[k] = part.e[k];
+}
+
+cudaError_t launch_store_table(const TourStep *tab, int n, TourStep *d_tab, cudaStream_t stream)
+{
+    static thread_local TabPart part;
+    for (int at = 0; at < n; at += kTabPart) {
+        const int count = n - at < kTabPart ? n - at : kTabPart;
+        for (int k = 0; k < count; ++k) part.e[k] = tab[at + k];
+        store_table_kernel<<<(count + 127) / 128, 128, 0, stream>>>(part, d_tab + at, count);
+    }
+    return cudaGetLastError();
+}
+
 cudaError_t launch_split_deque(const SplitParams &p, int esize, const DequeShape &shape,
                                cudaStream_t stream)
 {
