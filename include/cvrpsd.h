@@ -67,12 +67,14 @@ extern "C" {
 
 /* Kernel choice for the Split (see cvrpsd_config). AUTO takes, for device
  * buffers and no predecessors, WARP for S <= 8192 scenarios on tours of
- * n >= 64 (SEQPAR for S <= 48 where n >= 3000), for host buffers SEQPAR for
- * S <= 256 where n >= 128, and DEQUE otherwise (lowest latency each). */
+ * n >= 64 (SEQPAR for S <= 48 where n >= 3000) if the walk's memory holds
+ * windows of min(n, L) candidates: any up to n = 1000, and longer ones the
+ * fewer the scenarios. Otherwise, and for host buffers, SEQPAR for S <= 256
+ * where n >= 128 (no predecessors), and DEQUE. */
 #define CVRPSD_KERNEL_AUTO   0
 #define CVRPSD_KERNEL_DEQUE  1   /* one thread per scenario, monotone deque */
-#define CVRPSD_KERNEL_WARP   2   /* one warp per scenario, parallel window min (windows of up to 64
-                                    candidates in registers, longer ones in shared memory) */
+#define CVRPSD_KERNEL_WARP   2   /* one warp per scenario, parallel window min (the last 64
+                                    candidates in registers, older ones in shared memory) */
 #define CVRPSD_KERNEL_SEQPAR 3   /* few scenarios: min-plus matrix products over blocks of
                                     positions, parallel along the tour (S <= 4096) */
 

@@ -396,13 +396,22 @@ int split_eval_impl(cvrpsd_ctx *ctx, const int32_t *tour, int32_t n, const int32
     // positions the deque kernel stays (15 us against 9 at n = 50: its walk
     // is short, and callers read the kernel back). Scenarios in host memory
     // keep the kernels whose warps read whole sectors of a row.
+    // The walk is taken where it holds every window that n and L allow, so its
+    // time does not hang on the demands. Whole calls with L = n and a Q of 70
+    // mean demands, by the deque (S <= 256: sequence-parallel) kernel and by the walk:
+    //   n      S     deque  warp          n      S     deque  warp
+    //   200    37    131    42            1000   37    421    77
+    //   200    1000  75     46            1000   1000  178    88
+    //   200    4096  77     57            1000   4096  181    142
+    //   200    8192  76     68            1000   8192  188    199
     int kernel = ctx->cfg.kernel;
     if (kernel == CVRPSD_KERNEL_AUTO) {
         kernel = CVRPSD_KERNEL_DEQUE;
-        if (!pred && host_buffers) {
-            if (S <= 256 && n >= 128) kernel = CVRPSD_KERNEL_SEQPAR;
-        } else if (!pred && n >= 64 && S <= 8192) {
+        const bool held = walk_ring(n, L, S, ctx->sm_count).width >= (n < L ? n : L);
+        if (!pred && !host_buffers && n >= 64 && S <= 8192 && held) {
             kernel = S <= 48 && n >= 3000 ? CVRPSD_KERNEL_SEQPAR : CVRPSD_KERNEL_WARP;
+        } else if (!pred && S <= 256 && n >= 128) {
+            kernel = CVRPSD_KERNEL_SEQPAR;
         }
     }
     DequeShape shape{128, 1, 16};

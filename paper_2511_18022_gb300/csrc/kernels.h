@@ -122,8 +122,14 @@ constexpr int kAsideBlocks = 8;
 cudaError_t launch_split_warp(const SplitParams &p, int esize, const int32_t *list,
                               const unsigned long long *count, int grid_ctas, int max_smem,
                               cudaStream_t stream);
+// The register walk's memory of older positions: entries of its two rings (0:
+// none, no window can be longer than 64), a slot's mask, the longest window.
+struct WalkRing {
+    int size, mask, width;
+};
+WalkRing walk_ring(int n, int L, long long S, int sm_count);
 // One scenario per warp by the register walk; scenarios with a window longer
-// than 64 go on p.ovf_list (count in ACC_OVERFLOW) for launch_split_warp.
+// than walk_ring's go on p.ovf_list (count in ACC_OVERFLOW) for launch_split_warp.
 cudaError_t launch_split_walk(const SplitParams &p, int esize, int sm_count, cudaStream_t stream);
 inline size_t split_warp_smem_per_warp(int n) { return (size_t)2 * (n + 1) * sizeof(int); }
 

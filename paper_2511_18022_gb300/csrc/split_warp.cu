@@ -17,6 +17,10 @@
 // starts do not depend on g, so the minima of the four windows over the
 // values already known are four independent warp reductions, and what is
 // left in sequence is three minima and four additions on uniform values.
+// Where L and n allow longer windows, the walk of a whole call (split_walk_*)
+// also keeps the prefix loads and values of older positions in shared memory,
+// the values as suffix minima of their 32 positions, and adds the minimum of
+// a window's older part to each reduction (see WalkPrep).
 #include <stdint.h>
 
 #include "kernels.h"
@@ -29,7 +33,7 @@ struct WarpResult {
     int cost;      // f(n), INT32_MAX if infeasible
     bool bad;      // some demand > Q
     bool neg;      // some demand < 0
-    bool wide;     // register walk only: a window longer than kWalkWidth, no cost
+    bool wide;     // register walk only: a window longer than it holds, no cost
 };
 
 constexpr int kWalkWidth = 64;       // candidates held in registers
@@ -41,27 +45,44 @@ struct __align__(16) WalkSmem {
     int lo[32], c[32];               // window start and C_i of the chunk's positions
 };
 
+// What a walk reads and writes there. FAR walks, whose windows may be longer
+// than kWalkWidth, have rings of `ring` prefix loads and values (slot i & mask),
+// and the minima of the chunk's windows before the values in registers.
+struct WalkStore {
+    int *P, *lo, *c;
+    int *a, *g;
+    WalkRing ring;
+};
+
+// How a prepared chunk is walked.
+enum WalkMode { WALK_ENDED, WALK_GENERAL, WALK_PLAIN, WALK_FAR, WALK_SCAN };
+
 // The recursion over the positions i0 .. min(n, i0 + 31) of a chunk, four to
 // a step. The value of position p lives in lane (p - 1) mod 32: v0 the latest
 // there (position pl), v1 the one 32 positions earlier. The window starts do
 // not depend on g, so the minima of a step's four windows over the values
 // known before it are four independent warp reductions; the values of the
 // step itself are added on uniform registers. PLAIN: no window of the chunk
-// is longer than 32 positions or starts inside its own step.
-template <bool PLAIN>
-__device__ __forceinline__ void walk_chunk(const int *lo32, const int *c32, int n, int i0, int &v0, int &v1, int &pl)
+// is longer than 32 positions or starts inside its own step. FAR: some window
+// is longer than kWalkWidth; a32 holds the minima of the positions' windows
+// up to i0 - 33, and the registers always reach back to i0 - 36 or further.
+template <int MODE>
+__device__ __forceinline__ void walk_chunk(const int *lo32, const int *c32, const int *a32, int n, int i0, int &v0,
+                                           int &v1, int &pl)
 {
+    constexpr bool PLAIN = MODE == WALK_PLAIN, FAR = MODE == WALK_FAR;
     constexpr int kNone = INT32_MAX;
     constexpr unsigned kAll = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const bool odd = lane & 1, high = lane & 2;
     const int4 *lo = reinterpret_cast<const int4 *>(lo32), *c = reinterpret_cast<const int4 *>(c32);
-    int4 l4 = lo[0], c4 = c[0];
+    const int4 *a = reinterpret_cast<const int4 *>(a32);
+    int4 l4 = lo[0], c4 = c[0], a4 = FAR ? a[0] : make_int4(0, 0, 0, 0);
 #pragma unroll
     for (int b = 0; b < 8; ++b) {
         const int ib = i0 + 4 * b;
         if (b > 0 && ib > n) break;
-        const int4 ln = lo[(b + 1) & 7], cn = c[(b + 1) & 7];
+        const int4 ln = lo[(b + 1) & 7], cn = c[(b + 1) & 7], an = FAR ? a[(b + 1) & 7] : a4;
         int m0 = pl >= l4.x ? v0 : kNone, m1 = pl >= l4.y ? v0 : kNone;
         int m2 = pl >= l4.z ? v0 : kNone, m3 = pl >= l4.w ? v0 : kNone;
         if (!PLAIN) {
@@ -75,6 +96,12 @@ __device__ __forceinline__ void walk_chunk(const int *lo32, const int *c32, int 
         m1 = __reduce_min_sync(kAll, m1);
         m2 = __reduce_min_sync(kAll, m2);
         m3 = __reduce_min_sync(kAll, m3);
+        if (FAR) {
+            m0 = min(m0, a4.x);
+            m1 = min(m1, a4.y);
+            m2 = min(m2, a4.z);
+            m3 = min(m3, a4.w);
+        }
         // the previous position is always in the window
         const int ga = c4.x + m0;
         const int gb = c4.y + min(m1, ga);
@@ -90,14 +117,66 @@ __device__ __forceinline__ void walk_chunk(const int *lo32, const int *c32, int 
         }
         l4 = ln;
         c4 = cn;
+        a4 = an;
     }
+}
+
+// The same for a chunk whose windows all start at i0 or before: with A_i the
+// minimum of position i's window before i0 and m_i that of the chunk's values up
+// to i, m_i = min(m_{i-1} + min(C_i, 0), A_i + C_i): a warp scan of such pairs
+// gives all positions at once, for a fifth of the instructions of eight steps
+// (calls with n = 1000, windows of 70: S = 8192 288 us by steps, 199 by scans;
+// S = 1000 108, 88; S = 37, where the preparing warp is the slower one, 81, 77).
+__device__ __forceinline__ void scan_chunk(const WalkStore &w, int i0, int &v0, int &v1, int &pl)
+{
+    constexpr int kFar = 1 << 30;                              // above all values; sums with C_i stay in range
+    constexpr unsigned kAll = 0xffffffffu;
+    const int lane = threadIdx.x & 31, lo = w.lo[lane], c = w.c[lane];
+    int m = v0;                                                // position i0 - 32 + lane
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int u = __shfl_down_sync(kAll, m, o);
+        if (lane + o < 32) m = min(m, u);
+    }
+    m = __shfl_sync(kAll, m, max(lo - (i0 - 32), 0) & 31);
+    const int A = min(kFar, min(w.a[lane], lo < i0 ? m : kFar));
+    int shift = min(c, 0), best = A + c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int us = __shfl_up_sync(kAll, shift, o), ub = __shfl_up_sync(kAll, best, o);
+        if (lane >= o) {
+            best = min(best, ub + shift);
+            shift += us;
+        }
+    }
+    const int before = __shfl_up_sync(kAll, best, 1);
+    v1 = v0;
+    v0 = c + (lane ? min(A, before) : A);
+    pl = i0 + lane;
+}
+
+// A chunk in the mode its preparation found, and (FAR) its values to the ring.
+template <bool FAR>
+__device__ __forceinline__ void walk_chunk(int mode, const WalkStore &w, int n, int i0, int &v0, int &v1, int &pl)
+{
+    if (mode == WALK_PLAIN) walk_chunk<WALK_PLAIN>(w.lo, w.c, w.a, n, i0, v0, v1, pl);
+    else if (!FAR || mode == WALK_GENERAL) walk_chunk<WALK_GENERAL>(w.lo, w.c, w.a, n, i0, v0, v1, pl);
+    else if (mode == WALK_SCAN) scan_chunk(w, i0, v0, v1, pl);
+    else walk_chunk<WALK_FAR>(w.lo, w.c, w.a, n, i0, v0, v1, pl);
+    if (FAR) w.g[(i0 + (int)(threadIdx.x & 31)) & w.ring.mask] = v0;
 }
 
 // One scenario's positions prepared by a (full) warp, 32 at a time, one per
 // lane: demands (loaded a chunk ahead) are scanned to prefix loads, and each
 // lane finds its position's window start by bisection over the prefix loads
 // kept in shared memory.
-template <typename DT>
+//
+// FAR: where a chunk holds a window longer than kWalkWidth, the values of
+// positions up to i0 - 33 (the walk of the chunk before this one may still be
+// under way) are turned into suffix minima of their chunks of 32, each chunk
+// once, and a lane's minimum over its window there is the suffix from the
+// window's start and the minima of the whole chunks after it.
+template <typename DT, bool FAR>
 struct WalkPrep {
     static constexpr unsigned kAll = 0xffffffffu;
     const TourStep *__restrict__ tab;
@@ -105,11 +184,13 @@ struct WalkPrep {
     const DT *__restrict__ dem;
     long long ld, s;
     unsigned long long *status;
-    int *P;                                                    // kWalkRing prefix loads, this warp's
+    WalkStore w;
     TourStep t0, t1;                                           // table entries of this chunk and the next
     int q, carry;
+    int suffixes;                                              // chunks before this one hold suffix minima
     bool neg, bad;
 
+    __device__ __forceinline__ int slot(int p) const { return p & (FAR ? w.ring.mask : kWalkRing - 1); }
     __device__ __forceinline__ TourStep step_of(int i) const
     {
         const TourStep none{0, 0};
@@ -127,13 +208,38 @@ struct WalkPrep {
         t1 = step_of(33 + lane);
         q = demand_of(t0, 1 + lane);
         carry = 0;
+        suffixes = -1;
         neg = bad = false;
         __syncwarp();                                          // the previous scenario's readers are done
-        if (lane == 0) P[0] = 0;
+        if (lane == 0) w.P[0] = 0;
     }
-    // The chunk from i0: window starts to lo, C_i to c. False (uniformly) if the
-    // scenario has no cost (bad) or a window longer than kWalkWidth.
-    __device__ __forceinline__ bool chunk(int i0, int *lo_out, int *c_out, bool &plain)
+    // Minimum of the window from lo (INT32_MAX: none) over the positions up to i0 - 33.
+    __device__ __forceinline__ int older(int i0, int lo)
+    {
+        const int lane = threadIdx.x & 31, last = ((i0 - 1) >> 5) - 2;
+        const int from = (__shfl_sync(kAll, lo, 0) - 1) >> 5;  // window starts never move back
+        for (int k = max(suffixes, from); k <= last; ++k) {
+            const int p = 32 * k + 1 + lane;                   // chunk -1 holds position 0 alone
+            int v = p >= 0 ? w.g[slot(p)] : INT32_MAX;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int u = __shfl_down_sync(kAll, v, o);
+                if (lane + o < 32) v = min(v, u);
+            }
+            if (p >= 0) w.g[slot(p)] = v;
+        }
+        suffixes = last + 1;
+        __syncwarp();
+        int m = lo <= i0 - 33 ? w.g[slot(lo)] : INT32_MAX;
+        for (int k = from + 1; k <= last; ++k) {
+            const int whole = w.g[slot(32 * k + 1)];
+            if (k > (lo - 1) >> 5) m = min(m, whole);
+        }
+        return m;
+    }
+    // The chunk from i0: window starts, C_i and (FAR) older minima to shared memory.
+    // WALK_ENDED (uniformly) if the scenario has no cost (bad) or a window too long.
+    __device__ __forceinline__ int chunk(int i0)
     {
         const int lane = threadIdx.x & 31, i = i0 + lane;
         const TourStep t2 = step_of(i + 64);
@@ -148,29 +254,39 @@ struct WalkPrep {
         }
         p += carry;
         carry = __shfl_sync(kAll, p, 31);
-        P[i & (kWalkRing - 1)] = p;
+        w.P[slot(i)] = p;
         __syncwarp();
         const int first = max(0, i - L);                       // the route-length limit's start
-        const int before = i - kWalkWidth - 1;
-        const bool wide = i <= n && before >= first && p - P[before & (kWalkRing - 1)] <= Q;
+        const auto beyond = [&](int width) {                   // the window is longer than width
+            const int before = i - width - 1;
+            return i <= n && before >= first && p - w.P[slot(before)] <= Q;
+        };
+        const bool wide = beyond(kWalkWidth);
         // a scenario with a demand above Q has no cost; one with a longer window is not for this walk
-        if (__any_sync(kAll, wide | bad)) return false;
-        int lo = max(first, i - kWalkWidth), hi = i - 1;       // hi is always in the window
-#pragma unroll
-        for (int k = 0; k < 6; ++k) {
+        bool far = __any_sync(kAll, wide | bad);
+        if (far && (!FAR || __any_sync(kAll, bad || beyond(w.ring.width)))) return WALK_ENDED;
+        int lo = max(first, i - (far ? w.ring.width : kWalkWidth)), hi = i - 1;       // hi is always in the window
+        const auto halve = [&]() {
             const int mid = (lo + hi) >> 1;
-            const bool in = p - P[mid & (kWalkRing - 1)] <= Q;
+            const bool in = p - w.P[slot(mid)] <= Q;
             hi = in ? mid : hi;
             lo = in ? lo : mid + 1;
-        }
+        };
+        if (far)
+            for (int k = 32 - __clz(w.ring.width); k > 6; --k) halve();
+#pragma unroll
+        for (int k = 0; k < 6; ++k) halve();
         // positions past n (the last chunk) have an empty window
-        lo_out[lane] = i <= n ? lo : INT32_MAX;
-        c_out[lane] = t0.c;
-        plain = __all_sync(kAll, i > n || (i - lo <= 32 && lo <= i - (lane & 3)));
+        if (i > n) lo = INT32_MAX;
+        w.lo[lane] = lo;
+        w.c[lane] = t0.c;
+        const bool plain = __all_sync(kAll, i > n || (i - lo <= 32 && lo <= i - (lane & 3)));
+        const bool scan = FAR && !plain && __all_sync(kAll, i > n || lo <= i0);
+        if (far || scan) w.a[lane] = older(i0, lo);
         t0 = t1;
         t1 = t2;
         q = qn;
-        return true;
+        return scan ? WALK_SCAN : far ? WALK_FAR : plain ? WALK_PLAIN : WALK_GENERAL;
     }
     // After the last chunk, or the one that ended the walk.
     __device__ __forceinline__ void finish(bool ended, bool &any_neg, bool &any_bad)
@@ -188,26 +304,26 @@ struct WalkPrep {
 // What bounds it: the chain of a step (select, 18 clocks of reduction, four
 // additions and minima, insertion) while few warps run, issue of the ALU pipe
 // when many do.
-template <typename DT>
+template <typename DT, bool FAR>
 __device__ __forceinline__ WarpResult warp_walk_scenario(const TourStep *__restrict__ tab, int n, int Q, int L, int g0,
                                                          const DT *__restrict__ dem, long long ld, long long s,
-                                                         WalkSmem &w, unsigned long long *status)
+                                                         const WalkStore &w, unsigned long long *status)
 {
     const int lane = threadIdx.x & 31;
     WarpResult r{INT32_MAX, false, false, false};
-    WalkPrep<DT> pr{tab, n, Q, L, dem, ld, s, status, w.P};
+    WalkPrep<DT, FAR> pr{tab, n, Q, L, dem, ld, s, status, w};
     pr.start();
+    if (FAR && lane == 0) w.g[0] = g0;
     int v0 = lane == 31 ? g0 : INT32_MAX, v1 = INT32_MAX, pl = lane == 31 ? 0 : -kWalkWidth;
     bool ended = false;
     for (int i0 = 1; i0 <= n; i0 += 32) {
-        bool plain;
-        if (!pr.chunk(i0, w.lo, w.c, plain)) {
+        const int mode = pr.chunk(i0);
+        if (mode == WALK_ENDED) {
             ended = true;
             break;
         }
         __syncwarp();
-        if (plain) walk_chunk<true>(w.lo, w.c, n, i0, v0, v1, pl);
-        else walk_chunk<false>(w.lo, w.c, n, i0, v0, v1, pl);
+        walk_chunk<FAR>(mode, w, n, i0, v0, v1, pl);
     }
     pr.finish(ended, r.neg, r.bad);
     r.wide = ended && !r.bad;
@@ -234,7 +350,7 @@ __device__ __forceinline__ WarpResult warp_aside_scenario(const TourStep *__rest
         bad |= q > Q;
     }
     if (__any_sync(0xffffffffu, bad)) return WarpResult{INT32_MAX, true, (bool)__any_sync(0xffffffffu, neg), false};
-    return warp_walk_scenario<DT>(tab, n, Q, L, g0, dem, ld, s, w, status);
+    return warp_walk_scenario<DT, false>(tab, n, Q, L, g0, dem, ld, s, WalkStore{w.P, w.lo, w.c}, status);
 }
 
 // Evaluates scenario s of one tour with the calling (full) warp. P and g are
@@ -343,20 +459,25 @@ __global__ void __launch_bounds__(128) split_warp_kernel(SplitParams p, const in
 }
 
 // The register walk alone, one scenario per warp: a scenario with a window
-// longer than kWalkWidth goes on the list (for split_warp_kernel).
+// longer than it holds goes on the list (for split_warp_kernel). FAR: windows
+// of up to ring.width, with the rings in dynamic shared memory.
 constexpr int kWalkWarps = 4;
 
-template <typename DT>
-__global__ void __launch_bounds__(32 * kWalkWarps) split_walk_kernel(SplitParams p)
+template <typename DT, bool FAR>
+__global__ void __launch_bounds__(32 * kWalkWarps) split_walk_kernel(SplitParams p, WalkRing ring)
 {
-    __shared__ WalkSmem s_walk[kWalkWarps];
+    extern __shared__ __align__(16) int wsmem[];
+    __shared__ __align__(16) int s_P[FAR ? 1 : kWalkWarps][FAR ? 4 : kWalkRing];
+    __shared__ __align__(16) int s_lo[kWalkWarps][32], s_c[kWalkWarps][32], s_a[FAR ? kWalkWarps : 1][32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const long long s = (long long)blockIdx.x * kWalkWarps + w;
+    int *far = wsmem + (FAR ? w * 2 * ring.size : 0);
+    const WalkStore store{FAR ? far : s_P[FAR ? 0 : w], s_lo[w], s_c[w], s_a[FAR ? w : 0], far + ring.size, ring};
     long long sum = 0;
     unsigned inf = 0, status = 0;
     if (s < p.S) {
-        const WarpResult r = warp_walk_scenario<DT>(p.tab, p.n, p.Q, p.L, p.g0, reinterpret_cast<const DT *>(p.demand),
-                                                    p.ld, s, s_walk[w], p.acc + ACC_STATUS);
+        const WarpResult r = warp_walk_scenario<DT, FAR>(p.tab, p.n, p.Q, p.L, p.g0, reinterpret_cast<const DT *>(p.demand),
+                                                         p.ld, s, store, p.acc + ACC_STATUS);
         if (lane == 0) {
             if (r.wide) {
                 p.ovf_list[atomicAdd(p.acc + ACC_OVERFLOW, 1ull)] = (int32_t)s;
@@ -381,41 +502,47 @@ __global__ void __launch_bounds__(32 * kWalkWarps) split_walk_kernel(SplitParams
 // with n = 1000, S = 37 takes 67 us, 78 without the second warp.
 __device__ __forceinline__ void pair_sync() { asm volatile("bar.sync 1, 64;" ::: "memory"); }
 
-template <typename DT>
-__global__ void __launch_bounds__(64) split_walk_pair_kernel(SplitParams p)
+template <typename DT, bool FAR>
+__global__ void __launch_bounds__(64) split_walk_pair_kernel(SplitParams p, WalkRing ring)
 {
-    __shared__ int s_prefix[kWalkRing];
-    __shared__ __align__(16) int s_lo[2][32], s_c[2][32];
-    __shared__ int s_mode[2];                                  // 0 ended, 1 general, 2 plain
+    extern __shared__ __align__(16) int wsmem[];
+    __shared__ int s_prefix[FAR ? 1 : kWalkRing];
+    __shared__ __align__(16) int s_lo[2][32], s_c[2][32], s_a[FAR ? 2 : 1][32];
+    __shared__ int s_mode[2];                                  // WalkMode
     __shared__ int s_flags;                                    // 1 negative demand, 2 demand above Q
     const int lane = threadIdx.x & 31, n = p.n;
     const long long s = blockIdx.x;
     const bool prepares = threadIdx.x >= 32;
     const int chunks = (n + 31) >> 5;
+    const auto store = [&](int k) {
+        return WalkStore{FAR ? wsmem : s_prefix, s_lo[k & 1], s_c[k & 1], s_a[FAR ? k & 1 : 0], wsmem + ring.size, ring};
+    };
     int v0 = lane == 31 ? p.g0 : INT32_MAX, v1 = INT32_MAX, pl = lane == 31 ? 0 : -kWalkWidth;
     bool ended = false;
     if (prepares) {
-        WalkPrep<DT> pr{p.tab, n, p.Q, p.L, reinterpret_cast<const DT *>(p.demand), p.ld, s, p.acc + ACC_STATUS, s_prefix};
+        WalkPrep<DT, FAR> pr{p.tab, n, p.Q, p.L, reinterpret_cast<const DT *>(p.demand), p.ld, s, p.acc + ACC_STATUS,
+                             store(0)};
         pr.start();
         for (int k = 0; k < chunks && !ended; ++k) {
-            bool plain = false;
-            ended = !pr.chunk(1 + 32 * k, s_lo[k & 1], s_c[k & 1], plain);
-            if (lane == 0) s_mode[k & 1] = ended ? 0 : plain ? 2 : 1;
+            pr.w = store(k);
+            const int mode = pr.chunk(1 + 32 * k);
+            ended = mode == WALK_ENDED;
+            if (lane == 0) s_mode[k & 1] = mode;
             pair_sync();                                       // chunk k is there, chunk k - 1 walked
         }
         bool neg, bad;
         pr.finish(ended, neg, bad);
         if (lane == 0) s_flags = (neg ? 1 : 0) | (bad ? 2 : 0);
     } else {
+        if (FAR && lane == 0) wsmem[ring.size] = p.g0;
         for (int k = 0; k < chunks; ++k) {
             pair_sync();
             const int mode = s_mode[k & 1];
-            if (mode == 2) walk_chunk<true>(s_lo[k & 1], s_c[k & 1], n, 1 + 32 * k, v0, v1, pl);
-            else if (mode == 1) walk_chunk<false>(s_lo[k & 1], s_c[k & 1], n, 1 + 32 * k, v0, v1, pl);
-            else {
+            if (mode == WALK_ENDED) {
                 ended = true;
                 break;
             }
+            walk_chunk<FAR>(mode, store(k), n, 1 + 32 * k, v0, v1, pl);
         }
     }
     __syncthreads();
@@ -438,20 +565,54 @@ __global__ void __launch_bounds__(64) split_walk_pair_kernel(SplitParams p)
     block_finish(p.acc, p.done);
 }
 
+// Pairs while each scenario can have a walking warp's scheduler to itself;
+// more of them fill the preparation's gaps with other scenarios (n = 1000, us
+// per call alone / in pairs: S = 600 78.9, 69.9; 1000 82, 82; 2000 96.7, 100).
+static bool walk_in_pairs(long long S, int sm_count) { return S <= 4LL * sm_count; }
+
+// All positions (no slot is used twice) or a power of two that holds a window,
+// the chunk being prepared and the one being walked, whichever is less; where
+// that leaves fewer than kWalkResident scenarios resident, the largest power of two
+// that does not. Six blocks of four warps hold 1004 positions: n = 1000, L = n and
+// windows of 13 then take 131 us at S = 4096 (120 with the registers alone, whose
+// 13 resident blocks cannot finish a longer window) and 194 (182) at S = 8192.
+constexpr int kWalkResident = 3600;
+
+WalkRing walk_ring(int n, int L, long long S, int sm_count)
+{
+    const int reach = n < L ? n : L, all = (n + 31) / 32 * 32 + 4, warps = walk_in_pairs(S, sm_count) ? 1 : kWalkWarps;
+    if (reach <= kWalkWidth) return WalkRing{0, 0, kWalkWidth};
+    const auto fits = [&](int size) {
+        const size_t block = warps * 2 * (size_t)size * sizeof(int) + 3072;
+        return (long long)(233472 / block) * sm_count * warps >= (S < kWalkResident ? S : kWalkResident);
+    };
+    int size = kWalkRing;
+    while (size < reach + kWalkWidth) size *= 2;
+    if (all <= size && fits(all)) return WalkRing{all, -1, n};
+    while (size > kWalkRing && !fits(size)) size /= 2;
+    return WalkRing{size, size - 1, size - kWalkWidth};
+}
+
+template <bool FAR>
+static cudaError_t launch_walk(const SplitParams &p, int esize, const WalkRing &ring, bool pairs, cudaStream_t stream)
+{
+    const size_t smem = FAR ? (pairs ? 1 : kWalkWarps) * 2 * (size_t)ring.size * sizeof(int) : 0;
+    const unsigned grid = pairs ? (unsigned)p.S : (unsigned)((p.S + kWalkWarps - 1) / kWalkWarps);
+    auto k = pairs ? (esize == 2 ? split_walk_pair_kernel<int16_t, FAR> : split_walk_pair_kernel<int32_t, FAR>)
+                   : (esize == 2 ? split_walk_kernel<int16_t, FAR> : split_walk_kernel<int32_t, FAR>);
+    if (smem > 40 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+    }
+    k<<<grid, pairs ? 64 : 32 * kWalkWarps, smem, stream>>>(p, ring);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_split_walk(const SplitParams &p, int esize, int sm_count, cudaStream_t stream)
 {
-    // Pairs while each scenario can have a walking warp's scheduler to itself;
-    // more of them fill the preparation's gaps with other scenarios (n = 1000, us
-    // per call alone / in pairs: S = 600 78.9, 69.9; 1000 82, 82; 2000 96.7, 100).
-    if (p.S <= 4LL * sm_count) {
-        if (esize == 2) split_walk_pair_kernel<int16_t><<<(unsigned)p.S, 64, 0, stream>>>(p);
-        else split_walk_pair_kernel<int32_t><<<(unsigned)p.S, 64, 0, stream>>>(p);
-        return cudaGetLastError();
-    }
-    const unsigned grid = (unsigned)((p.S + kWalkWarps - 1) / kWalkWarps);
-    if (esize == 2) split_walk_kernel<int16_t><<<grid, 32 * kWalkWarps, 0, stream>>>(p);
-    else split_walk_kernel<int32_t><<<grid, 32 * kWalkWarps, 0, stream>>>(p);
-    return cudaGetLastError();
+    const WalkRing ring = walk_ring(p.n, p.L, p.S, sm_count);
+    const bool pairs = walk_in_pairs(p.S, sm_count);
+    return ring.size ? launch_walk<true>(p, esize, ring, pairs, stream) : launch_walk<false>(p, esize, ring, pairs, stream);
 }
 
 // Set-aside (tour, scenario) pairs of a batch; per-tour sums, infeasible
