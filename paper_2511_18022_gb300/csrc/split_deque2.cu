@@ -20,10 +20,22 @@ static_assert(sizeof(TabParam<kTab2Large>) + sizeof(Walk2Params) <= 32764, "tour
 template <typename DT, int R, int T, bool LCAP, bool NOWRAP, int CAP, bool SMOOTH = false, bool PRED = false>
 static cudaError_t launch2(const Walk2Params &p, const void *tab, long long grid, cudaStream_t st)
 {
-    split_deque2_kernel<DT, R, T, LCAP, NOWRAP, CAP, SMOOTH, PRED>
-        <<<(unsigned)grid, T, 0, st>>>(p, *static_cast<const TabParam<CAP> *>(tab));
+    auto kern = split_deque2_kernel<DT, R, T, LCAP, NOWRAP, CAP, SMOOTH, PRED>;
+    constexpr int smem = d2_rings<R, T>() > 48 * 1024 ? d2_rings<R, T>() : 0;
+    if (smem) {
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return e;
+    }
+    kern<<<(unsigned)grid, T, smem, st>>>(p, *static_cast<const TabParam<CAP> *>(tab));
     return cudaGetLastError();
 }
+
+// Blocks of the library's own shapes with rings of 32, by the scenarios that an
+// SM's shared memory holds with them: 13 blocks of 64 threads (each 1 KB beside
+// its rings for the system), or two of 448 for the last of an SM's rings.
+constexpr int kRing32Small = 64, kRing32Large = 448;
+template <int T> constexpr int d2_ring32_resident() { return 233472 / (d2_rings<32, T>() + 512 + 1024) * T; }
+static_assert(d2_ring32_resident<kRing32Small>() == 832 && d2_ring32_resident<kRing32Large>() == 896, "resident scenarios");
 
 // One instantiation class: demand type, route-length cap, key range, table
 // capacity. `shapes` lists the (threads, ring) pairs compiled for it; others
@@ -37,13 +49,15 @@ static cudaError_t dispatch_wide(const Walk2Params &p, const void *tab, const De
 {
     if (p.pred && s.threads == 64 && s.ring == 32)
         return launch2<DT, 32, 64, LCAP, NOWRAP, CAP, false, true>(p, tab, grid, st);
+    if (p.pred && s.threads == kRing32Large && s.ring == 32)
+        return launch2<DT, 32, kRing32Large, LCAP, NOWRAP, CAP, false, true>(p, tab, grid, st);
     if (p.pred && s.threads == 128 && s.ring == 16)
         return launch2<DT, 16, 128, LCAP, NOWRAP, CAP, false, true>(p, tab, grid, st);
     if (p.pred) return cudaErrorInvalidValue;
     if (smooth && s.threads == 128 && s.ring == 16)
         return launch2<DT, 16, 128, LCAP, NOWRAP, CAP, true>(p, tab, grid, st);
     CVRPSD_D2_SHAPE(64, 8) CVRPSD_D2_SHAPE(64, 16) CVRPSD_D2_SHAPE(128, 8) CVRPSD_D2_SHAPE(128, 16)
-    CVRPSD_D2_SHAPE(256, 8) CVRPSD_D2_SHAPE(256, 16) CVRPSD_D2_SHAPE(64, 32)
+    CVRPSD_D2_SHAPE(256, 8) CVRPSD_D2_SHAPE(256, 16) CVRPSD_D2_SHAPE(64, 32) CVRPSD_D2_SHAPE(kRing32Large, 32)
     return cudaErrorInvalidValue;
 }
 
@@ -91,18 +105,19 @@ cudaError_t route(const Walk2Params &w, const void *tab, const SplitParams &p, i
 // (128, 16): 13 blocks fill an SM's shared memory; rings of 8 need a
 // ring-overflow test on every push and set aside more scenarios, and measured
 // 20 % slower at n = 1000. Without a request, rings of 32 where all scenarios
-// are resident with them too (14 blocks of 64 on an SM): they cost nothing
-// there (n = 200, S = 100,000 in random order 50.6 against 51.5 us) and hold
-// the long deques of smooth tours (in strips 60.8 against 70.7 us; n = 1000
-// without a route-length cap 271 us against 286 and 2026 more for the 76 % of
-// scenarios that outgrow rings of 16).
-constexpr int kRing32Blocks = 14;
+// are resident with them too: they cost nothing there (n = 200, S = 100,000 in
+// random order 50.6 against 51.5 us) and hold the long deques of smooth tours
+// (in strips 60.8 against 70.7 us; n = 1000 without a route-length cap 271 us
+// against 286 and 2026 more for the 76 % of scenarios that outgrow rings of 16).
+// A block more than fits starts when the first ones end and doubles the time
+// (n = 1000, S = 136,192 by blocks of 64 428 us, by 448 270, rings of 16 264).
 DequeShape compiled_shape(const SplitParams &p, int esize, const DequeShape &s, int sm_count)
 {
     const bool wide = esize == 2 && keys_fit(p, esize) && p.n <= kTab2Small;
     if (!s.threads) {
-        const bool fits = p.S <= 64LL * kRing32Blocks * sm_count;
-        return wide && fits ? DequeShape{64, 1, 32} : DequeShape{128, 1, 16};
+        if (wide && p.S <= (long long)d2_ring32_resident<kRing32Small>() * sm_count) return DequeShape{kRing32Small, 1, 32};
+        if (wide && p.S <= (long long)d2_ring32_resident<kRing32Large>() * sm_count) return DequeShape{kRing32Large, 1, 32};
+        return DequeShape{128, 1, 16};
     }
     const bool listed = (s.threads == 64 || s.threads == 128 || s.threads == 256) && (s.ring == 8 || s.ring == 16);
     if (wide && listed) return DequeShape{s.threads, 1, s.ring};

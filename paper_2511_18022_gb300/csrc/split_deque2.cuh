@@ -361,15 +361,23 @@ constexpr int kD2ThreadsPerSM = 2048;
 template <int R, int T>
 constexpr int d2_min_blocks() { return kD2ThreadsPerSM / T; }
 
+// Threads that share a set of rings (a power of two: slots wrap by a mask), and
+// what the rings of a block take. Above 48 KB, dynamic.
+template <int T> __host__ __device__ constexpr int d2_ring_threads() { return (T & (T - 1)) ? 32 : T; }
+template <int R, int T> __host__ __device__ constexpr int d2_rings() { return R * T * (int)sizeof(int2); }
+
 template <typename DT, int R, int T, bool LCAP, bool NOWRAP, int CAP, bool SMOOTH, bool PRED>
 __global__ void __launch_bounds__(T, d2_min_blocks<R, T>()) split_deque2_kernel(const Walk2Params p, const __grid_constant__ TabParam<CAP> tab)
 {
-    // Rings [R][T] of (g, key) slots: thread t's slot k is at byte
-    // (k * T + t) * 8, so a warp's accesses never conflict.
-    __shared__ __align__(16) int2 rings[R * T];
+    // Rings [R][TR] of (g, key) slots for every TR threads: thread t's slot k is at
+    // byte (k * TR + t) * 8 of them, so a warp's accesses never conflict.
+    constexpr int TR = d2_ring_threads<T>();
+    constexpr bool kStatic = d2_rings<R, T>() <= 48 * 1024;
+    __shared__ __align__(16) int2 rings[kStatic ? R * T : 1];
+    extern __shared__ __align__(16) int2 more_rings[];
     const int tid = threadIdx.x;
-    const uint32_t rs = (uint32_t)__cvta_generic_to_shared(rings);
-    const uint32_t slot0 = (uint32_t)tid * 8u;
+    const uint32_t rs = (uint32_t)__cvta_generic_to_shared(kStatic ? rings : more_rings) + (uint32_t)(tid / TR * d2_rings<R, TR>());
+    const uint32_t slot0 = (uint32_t)(tid % TR) * 8u;
     long long sum = 0;
     // Every thread of a block runs the same number of rounds (the test is
     // on the block's first scenario), so block-wide code after the loop is
@@ -377,7 +385,7 @@ __global__ void __launch_bounds__(T, d2_min_blocks<R, T>()) split_deque2_kernel(
     for (long long sb = (long long)blockIdx.x * T; sb < p.S; sb += p.stride) {
         const long long s = sb + tid;
         bool aside = false;
-        const int c = walk2_scenario<DT, R, T, LCAP, NOWRAP, SMOOTH, PRED>(p, tab, s, rs, slot0, aside);
+        const int c = walk2_scenario<DT, R, TR, LCAP, NOWRAP, SMOOTH, PRED>(p, tab, s, rs, slot0, aside);
         if (s < p.S) {
             if (aside) {
                 const unsigned long long idx = atomicAdd(p.acc + ACC_OVERFLOW, 1ull);
