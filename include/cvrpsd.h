@@ -88,7 +88,8 @@ typedef struct cvrpsd_ctx cvrpsd_ctx;
 #define CVRPSD_WALK_AUTO          0   /* PARAM_TABLE where it applies, else GLOBAL_TABLE */
 #define CVRPSD_WALK_GLOBAL_TABLE  1   /* tour table in global memory; any n, spt 1 or 2 */
 #define CVRPSD_WALK_PARAM_TABLE   2   /* tour table in the launch's parameters: n <= 4032, spt 1,
-                                         int16 demands need Q < 32768; rings of 8 or 16 */
+                                         int16 demands need Q < 32768; rings of 8 or 16,
+                                         of 32 with 64 threads */
 
 /* Launch shape of the Split. threads in {64,128,256} per block (512 for the
  * batched path; single-tour calls then run 256), spt
@@ -276,10 +277,13 @@ typedef struct {
 } cvrpsd_tune_result;
 
 /*
- * Time every launch shape of the scenario-parallel kernel (threads x spt x
+ * Time the library's own choice and every launch shape of the
+ * scenario-parallel kernel (threads x spt x
  * ring, see cvrpsd_config) on this workload with CUDA events on `stream`,
- * check that each shape gives exactly the sum and infeasible count of the
- * default shape (CVRPSD_ERR_DEVICE_STATUS otherwise), and keep the fastest.
+ * check that each gives exactly the sum and infeasible count of the
+ * default shape (CVRPSD_ERR_DEVICE_STATUS otherwise), and keep the fastest:
+ * a shape whose calls beat the library's own choice by more than 5 %, else that
+ * choice (a zero cvrpsd_config: no forced kernel or shape).
  * Arguments as for cvrpsd_split_eval; out_cost is not written. With
  * cache_path != NULL, a result stored under the same key (GPU name, n rounded
  * up to a power of two, S rounded down to a power of two, demand type,

@@ -119,7 +119,8 @@ DequeShape compiled_shape(const SplitParams &p, int esize, const DequeShape &s, 
         if (wide && p.S <= (long long)d2_ring32_resident<kRing32Large>() * sm_count) return DequeShape{kRing32Large, 1, 32};
         return DequeShape{128, 1, 16};
     }
-    const bool listed = (s.threads == 64 || s.threads == 128 || s.threads == 256) && (s.ring == 8 || s.ring == 16);
+    const bool listed = ((s.threads == 64 || s.threads == 128 || s.threads == 256) && (s.ring == 8 || s.ring == 16)) ||
+                        (s.threads == 64 && s.ring == 32);
     if (wide && listed) return DequeShape{s.threads, 1, s.ring};
     return DequeShape{128, 1, 16};
 }
