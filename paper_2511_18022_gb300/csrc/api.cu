@@ -2,6 +2,7 @@
 // the per-tour position table, the launch plan and the exact host outputs.
 #include <cuda.h>
 #include <cuda_runtime.h>
+#include <limits.h>
 #include <stdarg.h>
 #include <stdio.h>
 #include <string.h>
@@ -466,8 +467,9 @@ int split_eval_impl(cvrpsd_ctx *ctx, const int32_t *tour, int32_t n, const int32
     const bool timed = ctx->profiling && (out_sum || out_infeasible || out_mean || host_buffers) && S > 0;
     bool fallback_launched = false;
     const int warp_grid = kAsideBlocks * (ctx->sm_count > 0 ? ctx->sm_count : 152);
-    const auto aside_pass = [&]() {
-        return launch_split_warp(p, demand_dtype, p.ovf_list, p.acc + ACC_OVERFLOW, warp_grid, ctx->max_smem, stream);
+    const auto aside_pass = [&](unsigned long long listed = ULLONG_MAX) {   // four to a block, at most warp_grid blocks
+        const int grid = listed / 4 < (unsigned long long)warp_grid ? (int)(listed / 4) + 1 : warp_grid;
+        return launch_split_warp(p, demand_dtype, p.ovf_list, p.acc + ACC_OVERFLOW, grid, ctx->max_smem, stream);
     };
     if (S > 0) {
         if (kernel == CVRPSD_KERNEL_SEQPAR && !pred) {
@@ -625,31 +627,37 @@ launched:
     if (one_launch && a[ACC_OVERFLOW]) {
         if (param_walk) CK(upload_table(), "upload tour table");
         if (timed) CK(cudaEventRecord(ctx->ev_t[1], stream), "cudaEventRecord");
-        const auto read_totals = [&]() {
-            return cudaMemcpyAsync(a, p.acc, ACC_ALLOC_WORDS * sizeof(unsigned long long), cudaMemcpyDeviceToHost, stream);
-        };
         // A long list left by rings of 16 or 8 goes to rings of 32, one thread
         // per scenario: one walk's latency and a twelfth of the warp kernel's
         // time per scenario (n = 1000: 26 ns). Whole calls, n = 200: 39,108
         // listed 646 us by warps, 529 by threads; 19,737 396, 349; they meet
-        // near 12,000.
-        bool warps = true;
+        // near 12,000. The warp pass hands its totals over and clears them as the
+        // main kernel does, and has as many blocks as the list needs: with a copy,
+        // a memset and a full grid one infeasible scenario cost a call 31 us
+        // (n = 200, S = 12,000), 19 now, and such calls were slower (101 us) than
+        // with the pass launched every time (91).
         ctx->stats.launches = 1;
         if (a[ACC_OVERFLOW] >= 16384 && kernel == CVRPSD_KERNEL_DEQUE && !pred && st.ring < 32) {
             p.done = nullptr;
             CK(launch_split_list(p, (long long)a[ACC_OVERFLOW], demand_dtype, stream), "split_list launch");
+            const auto read_totals = [&]() {
+                return cudaMemcpyAsync(a, p.acc, ACC_ALLOC_WORDS * sizeof(unsigned long long), cudaMemcpyDeviceToHost, stream);
+            };
             CK(read_totals(), "read accumulators");
             CK(cudaStreamSynchronize(stream), "cudaStreamSynchronize");
-            warps = a[ACC_TICKET] != 0;
             ++ctx->stats.launches;
-        }
-        if (warps) {
-            CK(aside_pass(), "split_warp (set-aside scenarios) launch");
-            CK(read_totals(), "read accumulators");
+            if (a[ACC_TICKET] != 0) {
+                CK(aside_pass(), "split_warp (set-aside scenarios) launch");
+                CK(read_totals(), "read accumulators");
+                ++ctx->stats.launches;
+            }
+            if (timed) CK(cudaEventRecord(ctx->ev_t[2], stream), "cudaEventRecord");
+            CK(cudaMemsetAsync(p.acc, 0, ACC_ALLOC_WORDS * sizeof(unsigned long long), stream), "clear accumulators");
+        } else {
+            CK(aside_pass(a[ACC_OVERFLOW]), "split_warp (set-aside scenarios) launch");
             ++ctx->stats.launches;
+            if (timed) CK(cudaEventRecord(ctx->ev_t[2], stream), "cudaEventRecord");
         }
-        if (timed) CK(cudaEventRecord(ctx->ev_t[2], stream), "cudaEventRecord");
-        CK(cudaMemsetAsync(p.acc, 0, ACC_ALLOC_WORDS * sizeof(unsigned long long), stream), "clear accumulators");
         CK(cudaStreamSynchronize(stream), "cudaStreamSynchronize");
         ctx->tab_use = cvrpsd_ctx::TAB_FREE;
         fallback_launched = true;

@@ -243,15 +243,15 @@ __device__ __forceinline__ void block_accumulate(long long sum, unsigned inf, un
 // totals to page-locked host memory and clears them for the next call, unless
 // scenarios were set aside (the host then launches the pass over them, which
 // adds to the totals left here). It takes the place of a clearing memset and
-// a copy back around the kernel.
-__device__ __forceinline__ void block_finish(unsigned long long *acc, unsigned long long *done)
+// a copy back around the kernel. `last`: no such pass follows.
+__device__ __forceinline__ void block_finish(unsigned long long *acc, unsigned long long *done, bool last = false)
 {
     if (!done || threadIdx.x != 0) return;   // thread 0 did the block's atomics
     __threadfence();
     if (atomicAdd(acc + ACC_TICKET, 1ull) != (unsigned long long)gridDim.x - 1) return;
     __threadfence();
     volatile unsigned long long *a = acc, *d = done;
-    const bool aside = a[ACC_OVERFLOW] != 0;
+    const bool aside = !last && a[ACC_OVERFLOW] != 0;
 #pragma unroll
     for (int k = 0; k < ACC_WORDS; ++k) {
         d[k] = a[k];

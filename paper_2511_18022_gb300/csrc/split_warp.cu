@@ -456,6 +456,10 @@ __global__ void __launch_bounds__(128) split_warp_kernel(SplitParams p, const in
             atomicOr(p.sticky, (unsigned long long)status);
         }
     }
+    if (p.done) {
+        __syncthreads();                                     // the block's additions are done
+        block_finish(p.acc, p.done, true);
+    }
 }
 
 // The register walk alone, one scenario per warp: a scenario with a window
