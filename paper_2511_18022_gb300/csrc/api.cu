@@ -1385,7 +1385,8 @@ int cvrpsd_gen_demand(cvrpsd_ctx *ctx, uint64_t seed, int32_t kind, const int32_
     CK(cudaMemcpyAsync(ctx->d_gen, ctx->h_gen, 2 * (size_t)n * sizeof(int32_t), cudaMemcpyHostToDevice, stream),
        "upload mu/region");
     CK(cudaEventRecord(ctx->ev_gen, stream), "cudaEventRecord");
-    GenParams g{seed, kind, ctx->d_gen, ctx->d_gen + n, n, S, ld, out};
+    GenParams g{seed, kind, ctx->d_gen, ctx->d_gen + n, n, S, ld, out, *std::min_element(mu, mu + n),
+                *std::max_element(mu, mu + n)};
     CK(launch_gen_demand(g, dtype, stream), "gen_demand launch");
     return CVRPSD_OK;
 }

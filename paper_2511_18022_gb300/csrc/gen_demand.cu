@@ -157,10 +157,10 @@ struct PhiloxColumn {
 // n = 200, S = 100,000, 10.6 GB/s of output). So each entry is evaluated in
 // float32 with a rigorous error bound first; when both ends of the bound
 // round to the same integer that integer is the float64 result. The others
-// (about 2e-4 of the entries at means of 5 to 30; all of them above about
-// 1e5, where float32 cannot decide) go through the float64 recipe: collected
-// in shared memory and evaluated densely after the block's rows, or on the
-// spot when the list is full. What bounds it now: issue of the Philox rounds
+// (about 2e-4 of the entries at means of 5 to 30) go through the float64
+// recipe: collected in shared memory and evaluated densely after the block's
+// rows, or on the spot when the list is full. SKIP: rows of means from `dense`
+// on are left to gen_dense_kernel. What bounds it now: issue of the Philox rounds
 // (14 wide multiplies) and the four special functions of an entry, 153 clocks
 // of a scheduler per 32 entries. 110 us at n = 200, S = 100,000 (1.01 ms at
 // n = 1000, S = 2^18); 132 us before the draws' common Philox rounds, the
@@ -172,8 +172,8 @@ constexpr int kGenRows = 64;                     // most rows of a block
 constexpr float kGenMax = 1.0e6f;                // float32 decides nothing above
 constexpr float kGenMagic = 12582912.0f;         // 1.5 * 2^23: adding it rounds to an integer
 
-template <typename DT, int KIND>
-__global__ void __launch_bounds__(kGenThreads, 4) gen_demand_kernel(GenParams g, int rows_per_block)
+template <typename DT, int KIND, bool SKIP>
+__global__ void __launch_bounds__(kGenThreads, 4) gen_demand_kernel(GenParams g, int rows_per_block, float dense)
 {
     __shared__ uint32_t s_list[kGenList];
     __shared__ int s_count;
@@ -212,6 +212,7 @@ __global__ void __launch_bounds__(kGenThreads, 4) gen_demand_kernel(GenParams g,
         for (int k = 0; k < rows; ++k, out += g.ld) {
             const float2 rw = s_row[k];
             const float mu = rw.x;
+            if (SKIP && mu >= dense) continue;               // the same for all threads
             const uint2 w = px.at((uint32_t)(r0 + k));
             float e, x, err;
             bool ok;
@@ -262,6 +263,37 @@ __global__ void __launch_bounds__(kGenThreads, 4) gen_demand_kernel(GenParams g,
     }
 }
 
+// Rows of large means, where float32 decides so few of a warp's entries that
+// the draws behind the others (two normals for each of a correlated matrix)
+// take longer: the recipe in float64 for every entry, a column's four factors
+// once per block. Bound by the float64 pipe.
+template <typename DT, int KIND>
+__global__ void __launch_bounds__(kGenThreads) gen_dense_kernel(GenParams g, int rows_per_block, float dense)
+{
+    const long long s = (long long)blockIdx.x * kGenThreads + threadIdx.x;
+    if (s >= g.S) return;
+    const uint32_t k0 = (uint32_t)g.seed, k1 = (uint32_t)(g.seed >> 32);
+    const int r0 = blockIdx.y * rows_per_block, r1 = min(g.n, r0 + rows_per_block);
+    DT *out = reinterpret_cast<DT *>(g.out) + (long long)r0 * g.ld + s;
+    double f[4] = {0.0, 0.0, 0.0, 0.0};
+    bool drawn = false;
+    for (int row = r0; row < r1; ++row, out += g.ld) {
+        if ((float)g.mu[row] < dense) continue;              // the same for all threads
+        const double mu = (double)g.mu[row], z = std_normal((uint32_t)s, (uint32_t)row, KIND == 1 ? 0u : 2u, k0, k1);
+        if (KIND == 1) {
+            if (!drawn) {
+#pragma unroll
+                for (int r = 0; r < 4; ++r) f[r] = std_normal((uint32_t)s, (uint32_t)r, 1u, k0, k1);
+                drawn = true;
+            }
+            const int reg = g.region[row] & 3;
+            *out = round_demand<DT>(correlated_f64(mu, reg == 0 ? f[0] : reg == 1 ? f[1] : reg == 2 ? f[2] : f[3], z));
+        } else {
+            *out = round_demand<DT>(__dadd_rn(mu, __dmul_rn(__dmul_rn(0.3, mu), z)));
+        }
+    }
+}
+
 template <typename TI, typename TO>
 __global__ void convert_demand_kernel(const TI *in, long long ld_in, TO *out, long long ld_out, int n, long long S,
                                       unsigned int *saturated)
@@ -296,23 +328,40 @@ cudaError_t launch_convert_demand(const void *in, int esize_in, long long ld_in,
     return cudaGetLastError();
 }
 
+template <typename DT, int KIND>
+static cudaError_t launch_gen(const GenParams &g, cudaStream_t stream)
+{
+    const long long bx = (g.S + kGenThreads - 1) / kGenThreads;
+    // 64 rows a block spread the four factor draws of a column thin; fewer
+    // where that leaves less than four blocks of 256 for each of 152 SMs (two in float64).
+    const auto block_rows = [&](int blocks) {
+        int rows = kGenRows;
+        while (rows > 8 && bx * ((g.n + rows - 1) / rows) < blocks) rows >>= 1;
+        return rows;
+    };
+    const int rows = block_rows(4 * 152), rows64 = block_rows(2 * 152);
+    // Means from here on go through float64 throughout. By float32 first and in
+    // float64, us: correlated, n = 200, S = 100,000, means of 10,000 3565 and 3775,
+    // 14,000 4365 and 3777, 10^6 6076 and 3772; in shorter blocks more of a row's
+    // entries fit the list (n = 200, S = 4000, 8 rows a block: 50,000 217 and 239,
+    // 10^5 295 and 238). Normal: 10^5 2902 and 2937, 10^6 3010 and 2937.
+    const float dense = KIND == 1 ? 7.0e5f / (float)rows : 1.0e5f;
+    const dim3 grid((unsigned)bx, (unsigned)((g.n + rows - 1) / rows));
+    if ((float)g.mu_max < dense) {
+        gen_demand_kernel<DT, KIND, false><<<grid, kGenThreads, 0, stream>>>(g, rows, dense);
+        return cudaGetLastError();
+    }
+    if ((float)g.mu_min < dense) gen_demand_kernel<DT, KIND, true><<<grid, kGenThreads, 0, stream>>>(g, rows, dense);
+    gen_dense_kernel<DT, KIND><<<dim3((unsigned)bx, (unsigned)((g.n + rows64 - 1) / rows64)), kGenThreads, 0, stream>>>(
+        g, rows64, dense);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_gen_demand(const GenParams &g, int esize, cudaStream_t stream)
 {
     if (g.S == 0 || g.n == 0) return cudaSuccess;
-    const long long bx = (g.S + kGenThreads - 1) / kGenThreads;
-    // 64 rows a block spread the four factor draws of a column thin; fewer
-    // where that leaves less than four blocks of 256 for each of 152 SMs.
-    int rows = kGenRows;
-    while (rows > 8 && bx * ((g.n + rows - 1) / rows) < 4 * 152) rows >>= 1;
-    const dim3 grid((unsigned)bx, (unsigned)((g.n + rows - 1) / rows));
-    if (esize == 2) {
-        if (g.kind == 1) gen_demand_kernel<int16_t, 1><<<grid, kGenThreads, 0, stream>>>(g, rows);
-        else gen_demand_kernel<int16_t, 0><<<grid, kGenThreads, 0, stream>>>(g, rows);
-    } else {
-        if (g.kind == 1) gen_demand_kernel<int32_t, 1><<<grid, kGenThreads, 0, stream>>>(g, rows);
-        else gen_demand_kernel<int32_t, 0><<<grid, kGenThreads, 0, stream>>>(g, rows);
-    }
-    return cudaGetLastError();
+    if (esize == 2) return g.kind == 1 ? launch_gen<int16_t, 1>(g, stream) : launch_gen<int16_t, 0>(g, stream);
+    return g.kind == 1 ? launch_gen<int32_t, 1>(g, stream) : launch_gen<int32_t, 0>(g, stream);
 }
 
 }  // namespace cvrpsd

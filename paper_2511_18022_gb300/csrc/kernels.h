@@ -283,6 +283,7 @@ struct GenParams {
     int32_t n;
     int64_t S, ld;
     void *out;
+    int32_t mu_min, mu_max;       // of mu
 };
 cudaError_t launch_gen_demand(const GenParams &g, int esize, cudaStream_t stream);
 
