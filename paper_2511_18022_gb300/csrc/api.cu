@@ -461,6 +461,7 @@ int split_eval_impl(cvrpsd_ctx *ctx, const int32_t *tour, int32_t n, const int32
     };
     if (!(one_launch && param_walk)) CK(upload_table(), "upload tour table");
 
+    const int table_kernels = capture == cudaStreamCaptureStatusNone ? 0 : store_table_launches(n);
     cvrpsd_stats st{};
     st.overflow = -1;
     st.kernel_ms = st.fallback_ms = -1.0f;
@@ -608,6 +609,7 @@ launched:
         fallback_launched = true;
         if (timed) CK(cudaEventRecord(ctx->ev_t[2], stream), "cudaEventRecord");
     }
+    st.launches += table_kernels;
     ctx->stats = st;
     log_msg(ctx, CVRPSD_LOG_DEBUG, "split n=%d S=%lld: kernel %d walk %d threads %d spt %d ring %d rounds %d", n,
             (long long)S, st.kernel, st.variant, st.threads, st.spt, st.ring, st.rounds);

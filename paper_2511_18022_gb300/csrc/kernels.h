@@ -102,6 +102,7 @@ cudaError_t launch_split_host_i32_nocap(const SplitParams &p, cudaStream_t st);
 // Writes a tour table of n entries to d_tab, from the launches' own parameters:
 // `tab` is free again when this returns, also under stream capture.
 cudaError_t launch_store_table(const TourStep *tab, int n, TourStep *d_tab, cudaStream_t stream);
+int store_table_launches(int n);
 
 // Dynamic shared memory of the deque kernel: its rings ([spt][ring][threads] int2).
 inline size_t split_deque_smem(const SplitParams &p, const DequeShape &shape)
@@ -203,6 +204,16 @@ inline DequeShape batch_default_shape(int max_n, long long scenarios, int sm_cou
 // reports blocks per SM in *blocks_per_sm.
 cudaError_t launch_split_batch(const BatchParams &b, int esize, bool lcap, const DequeShape &shape, int grid,
                                bool configure_only, int *blocks_per_sm, cudaStream_t stream);
+// Shapes that the second walk has for smooth tours too: the library's own where the
+// scenarios outgrow the device (n > 64), and those a tuner picks. In blocks of 64 or
+// 128 threads, for scenarios that fit at once, it does not pay: batches in strips
+// of 64 tours, n = 200, S = 3000 118 us by the other walk, 119; of 16 tours,
+// n = 500, S = 4000 327, 317; candidate tours, whose order only the device knows,
+// pay for a second launch: 64 in random order, n = 200, S = 3000 133, 141.
+inline bool batch2_smooth_compiled(const DequeShape &s)
+{
+    return s.spt == 1 && s.ring == 16 && (s.threads == 256 || s.threads == 512);
+}
 // The batch kernel on the second walk (split_batch2.cu), which
 // launch_split_batch picks where b.walk2 is set and the shape has one
 // scenario per thread.

@@ -175,7 +175,8 @@ int cvrpsd_split_eval_tours(cvrpsd_ctx *ctx, const int32_t *d_tours, int32_t T, 
     ctx->stats.spt = 1;
     ctx->stats.ring = shape.ring;
     ctx->stats.overflow = -1;
-    ctx->stats.launches = 4;
+    // tables, walk (both, where only the device knows which applies), set-aside pass, means
+    ctx->stats.launches = 4 + (bp.walk2 && batch2_smooth_compiled(shape));
     ctx->stats.kernel_ms = ctx->stats.fallback_ms = -1.0f;
     return CVRPSD_OK;
 }

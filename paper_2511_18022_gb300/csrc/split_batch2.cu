@@ -194,9 +194,7 @@ template <typename DT, bool LCAP>
 static cudaError_t dispatch2(BatchParams b, const DequeShape &s, int grid, bool configure_only,
                              int *blocks_per_sm, cudaStream_t st)
 {
-    // The walk of smooth tours is compiled for the library's own shape and the
-    // one a tuner picks.
-    if (b.smooth != 0 && s.spt == 1 && s.ring == 16 && (s.threads == 256 || s.threads == 512)) {
+    if (b.smooth != 0 && batch2_smooth_compiled(s)) {
         const cudaError_t e = s.threads == 256
             ? launch2_one<DT, 16, 256, LCAP, true>(b, s, grid, configure_only, blocks_per_sm, st)
             : launch2_one<DT, 16, 512, LCAP, true>(b, s, grid, configure_only, blocks_per_sm, st);

@@ -710,6 +710,8 @@ __global__ void store_table_kernel(const __grid_constant__ TabPart part, TourSte
     if (k < count) out[k] = part.e[k];
 }
 
+int store_table_launches(int n) { return (n + kTabPart - 1) / kTabPart; }
+
 cudaError_t launch_store_table(const TourStep *tab, int n, TourStep *d_tab, cudaStream_t stream)
 {
     static thread_local TabPart part;
