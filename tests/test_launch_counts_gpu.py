@@ -21,7 +21,7 @@ def cv():
 # capacities whose keys the second walk cannot hold
 @pytest.mark.parametrize("n,T,S,Q,threads,launches", [(60, 4, 100, 100, 64, 4), (400, 64, 3000, 100, 128, 4),
                                                      (700, 64, 9000, 100, 512, 5), (2000, 16, 20_000, 100, 256, 5),
-                                                     (65, 64, 9000, 30_000_000, 256, 4)])
+                                                     (65, 64, 9000, 1_000_000, 256, 4)])
 def test_tours_of_one_instance(cv, n, T, S, Q, threads, launches):
     rng = np.random.default_rng(n)
     inst = make_instance(n, 1, 10, seed=3, Q=Q)
