@@ -467,7 +467,7 @@ int split_eval_impl(cvrpsd_ctx *ctx, const int32_t *tour, int32_t n, const int32
     st.kernel_ms = st.fallback_ms = -1.0f;
     const bool timed = ctx->profiling && (out_sum || out_infeasible || out_mean || host_buffers) && S > 0;
     bool fallback_launched = false;
-    const int warp_grid = kAsideBlocks * (ctx->sm_count > 0 ? ctx->sm_count : 152);
+    const int warp_grid = aside_grid(n, ctx->sm_count);
     const auto aside_pass = [&](unsigned long long listed = ULLONG_MAX) {   // four to a block, at most warp_grid blocks
         const int grid = listed / 4 < (unsigned long long)warp_grid ? (int)(listed / 4) + 1 : warp_grid;
         return launch_split_warp(p, demand_dtype, p.ovf_list, p.acc + ACC_OVERFLOW, grid, ctx->max_smem, stream);

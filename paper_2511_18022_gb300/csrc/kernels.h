@@ -133,6 +133,15 @@ WalkRing walk_ring(int n, int L, long long S, int sm_count);
 // than walk_ring's go on p.ovf_list (count in ACC_OVERFLOW) for launch_split_warp.
 cudaError_t launch_split_walk(const SplitParams &p, int esize, int sm_count, cudaStream_t stream);
 inline size_t split_warp_smem_per_warp(int n) { return (size_t)2 * (n + 1) * sizeof(int); }
+// Blocks of that pass over one tour's list: no more than are resident, since the
+// list is dealt out evenly and a second wave would start when the first ends (n =
+// 1000, six fit: S = 140,000 with 37,906 listed 682 -> 621 us). A batch's pass, whose tours
+// differ, keeps all eight (8 tours, n = 1000, S = 200,000 in strips 41.7 ms, 44.1 by six).
+inline int aside_grid(int n, int sm_count)
+{
+    const int fit = (int)(233472 / (4 * split_warp_smem_per_warp(n) + 4096));
+    return (sm_count > 0 ? sm_count : 152) * (fit < 1 ? 1 : fit < kAsideBlocks ? fit : kAsideBlocks);
+}
 
 // ---- batches of tours (one persistent launch) ----
 

@@ -416,6 +416,34 @@ __device__ WarpResult warp_split_scenario(const TourStep *tab, int n, int Q, int
     return r;
 }
 
+// Whether the scenarios of a warp's lanes (s < 0: none) hold a demand above Q, one
+// lane each: the rows in tour order, so that all warps read the same few rows at
+// a time and neighbours on the list share their sectors.
+template <typename DT>
+__device__ __forceinline__ void scan_lanes(const TourStep *__restrict__ tab, int n, int Q, const DT *__restrict__ dem,
+                                           long long ld, long long s, bool &neg, bool &bad, unsigned long long *status)
+{
+    neg = bad = false;
+    if (s < 0) return;
+#pragma unroll 8
+    for (int i = 0; i < n; ++i) {
+        const int row = tab[i].row & kRowMask;
+        const int q = index_ok(row < n && s < ld, status) ? (int)__ldg(dem + (long long)row * ld + s) : 0;
+        neg |= q < 0;
+        bad |= q > Q;
+    }
+}
+
+// A warp's share of the list from which its lanes look for demands above Q, each in
+// a scenario of its own, once the first of the share has one (why a scenario is
+// listed, that or a long deque, the list doesn't say). Calls that enqueue, scenarios
+// listed for such a demand, a warp each and by lanes: n = 1000, S = 500,000, 136,017
+// listed 3404 us, 1251; S = 200,000, 54,320 1116, 597; n = 200, S = 1,000,000,
+// 126,039 563, 400. Four a warp: n = 1000, S = 500,000, 17,300 listed 1134, 1113;
+// n = 200, S = 140,000, 17,318 106, 113. Listed for their deques, n = 1000: 476,146
+// of 500,000 14.0 ms, 12.5; 133,460 of 140,000 3297 us, 3534.
+constexpr int kScanItems = 6;
+
 template <typename DT>
 __global__ void __launch_bounds__(128) split_warp_kernel(SplitParams p, const int32_t *list,
                                                          const unsigned long long *count)
@@ -431,14 +459,7 @@ __global__ void __launch_bounds__(128) split_warp_kernel(SplitParams p, const in
 
     long long sum = 0;
     unsigned inf = 0, status = 0;
-    for (long long item = (long long)blockIdx.x * wpb + w; item < total;
-         item += (long long)gridDim.x * wpb) {
-        const long long s = list ? (long long)list[item] : item;
-        if (list && s < 0) continue;                         // settled by split_list_kernel (warp-uniform)
-        if (!index_ok(s >= 0 && s < p.S, p.acc + ACC_STATUS)) continue;   // warp-uniform
-        WarpResult r{};
-        r.wide = true;
-        if (!p.pred) r = warp_aside_scenario<DT>(p.tab, n, p.Q, p.L, p.g0, dem, p.ld, s, s_walk[w], p.acc + ACC_STATUS);
+    const auto settle = [&](long long s, WarpResult r) {     // r.wide: not walked yet
         if (r.wide)
             r = warp_split_scenario<DT>(p.tab, n, p.Q, p.L, p.g0, dem, p.ld, s, P, g, p.acc + ACC_STATUS, p.pred,
                                         p.ldp);
@@ -447,7 +468,56 @@ __global__ void __launch_bounds__(128) split_warp_kernel(SplitParams p, const in
             if (r.bad) ++inf; else sum += r.cost;
             if (p.out_cost) p.out_cost[s] = r.cost;
         }
+    };
+    const long long warps = (long long)gridDim.x * wpb, first = (long long)blockIdx.x * wpb + w;
+    const long long share = (total + warps - 1) / warps;
+    if (list && !p.pred && share >= kScanItems) {
+        const long long rounds = (share + 31) / 32;
+        const int items = (int)((share + rounds - 1) / rounds);
+        // a block's warps take neighbours at the same time: they share sectors
+        for (long long base = (long long)blockIdx.x * wpb * items; base < total; base += warps * items) {
+            const long long at = base + lane * wpb + w;
+            long long mine = lane < items && at < total ? (long long)list[at] : -1;
+            if (!index_ok(mine < p.S, p.acc + ACC_STATUS)) mine = -1;
+            unsigned left = __ballot_sync(0xffffffffu, mine >= 0);
+            bool begun = false, scan = false, scanned = false;
+            while (left) {
+                if (scan && !scanned) {
+                    bool neg, bad;
+                    scan_lanes<DT>(p.tab, n, p.Q, dem, p.ld, (left >> lane) & 1u ? mine : -1, neg, bad, p.acc + ACC_STATUS);
+                    if (neg) status |= ST_NEGATIVE_DEMAND;
+                    if (bad) {
+                        ++inf;
+                        if (p.out_cost) p.out_cost[mine] = INT32_MAX;
+                    }
+                    left &= ~__ballot_sync(0xffffffffu, bad);
+                    scanned = true;
+                    continue;
+                }
+                const long long s = __shfl_sync(0xffffffffu, mine, __ffs(left) - 1);
+                left &= left - 1;
+                const WarpResult r = scanned ? warp_walk_scenario<DT, false>(p.tab, n, p.Q, p.L, p.g0, dem, p.ld, s,
+                                                   WalkStore{s_walk[w].P, s_walk[w].lo, s_walk[w].c}, p.acc + ACC_STATUS)
+                                             : warp_aside_scenario<DT>(p.tab, n, p.Q, p.L, p.g0, dem, p.ld, s, s_walk[w],
+                                                                       p.acc + ACC_STATUS);
+                if (!begun) scan = r.bad;
+                begun = true;
+                settle(s, r);
+            }
+        }
+    } else {
+        for (long long item = first; item < total; item += warps) {
+            const long long s = list ? (long long)list[item] : item;
+            if (list && s < 0) continue;                     // settled by split_list_kernel (warp-uniform)
+            if (!index_ok(s >= 0 && s < p.S, p.acc + ACC_STATUS)) continue;   // warp-uniform
+            WarpResult r{};
+            r.wide = true;
+            if (!p.pred) r = warp_aside_scenario<DT>(p.tab, n, p.Q, p.L, p.g0, dem, p.ld, s, s_walk[w], p.acc + ACC_STATUS);
+            settle(s, r);
+        }
     }
+    inf = __reduce_add_sync(0xffffffffu, inf);
+    status = __reduce_or_sync(0xffffffffu, status);
     if (lane == 0) {
         if (sum) atomicAdd(p.acc + ACC_SUM, (unsigned long long)sum);
         if (inf) atomicAdd(p.acc + ACC_INFEASIBLE, (unsigned long long)inf);
