@@ -395,8 +395,8 @@ int split_eval_impl(cvrpsd_ctx *ctx, const int32_t *tour, int32_t n, const int32
     // S = 37 91, 101; 3000, S = 1 121, 115, S = 37 123, 128; 4000, S = 37 150,
     // 140), so one warp per scenario up to 8192 scenarios, and the
     // sequence-parallel kernel for a few dozen on a very long tour. Below 64
-    // positions the deque kernel stays (15 us against 9 at n = 50: its walk
-    // is short, and callers read the kernel back). Scenarios in host memory
+    // positions the deque kernel stays, though the walk's is the shorter one
+    // (15 us against 9 at n = 50, of a call's 37). Scenarios in host memory
     // keep the kernels whose warps read whole sectors of a row.
     // The walk is taken where it holds every window that n and L allow, so its
     // time does not hang on the demands. Whole calls with L = n and a Q of 70

@@ -2,8 +2,9 @@
 // level of parallelism of Section 3: the candidate predecessors of a position). For each position i the 32 lanes take the
 // candidates p of the feasible window [mask(i), i-1] of Eq. 2/3 in a strided
 // pattern and a warp min-reduction picks the best, so the cost per position
-// is O(|window| / 32 + log 32) and no candidate bound is needed. It serves the
-// scenarios the deque kernel sets aside, and any tour when forced.
+// is O(|window| / 32 + log 32) and no candidate bound is needed. It serves
+// calls of up to 8192 scenarios, the scenarios the deque kernel sets aside, and any
+// tour when forced.
 //
 // Per warp, shared memory holds the scenario's prefix loads P[0..n] (demands
 // loaded by all lanes at once, then a warp scan) and the values
